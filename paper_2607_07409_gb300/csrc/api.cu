@@ -1161,18 +1161,9 @@ int dels_gru_build_input_table(const dels_local_head* head, int V, float* table,
   if (sms <= 0) return DELS_ERR_CUDA;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int* status = at<int>(workspace, 0);
-  const uint16_t* E = static_cast<const uint16_t*>(head->emb);
-  // G[v0 : v0 + 128] = E[v0 : v0 + 128] W_ih^T, one 128-row block of the
-  // vocabulary per launch (the rows sit on the MMA's M like a batch).
-  for (int v0 = 0; v0 < V; v0 += kMaxBatchTile) {
-    const int rows = std::min(kMaxBatchTile, V - v0);
-    Gemm g;
-    if (!plan_store(g, rows, 3 * H, E + (size_t)v0 * D, head->w[0], D, nullptr, nullptr, 0, 128, 1, 0, ACT_NONE,
-                    table + (size_t)v0 * 3 * H, nullptr, 0, status, sms))
-      return DELS_ERR_CUDA;
-    PROF(DELS_KCLASS_HEAD_GEMM);
-    DELS_CUDA(run(g, s));
-  }
+  PROF(DELS_KCLASS_HEAD_GEMM);
+  DELS_CUDA(launch_input_table(static_cast<const uint16_t*>(head->emb), static_cast<const uint16_t*>(head->w[0]), table,
+                               V, 3 * H, D, status, sms, s));
   return DELS_OK;
 }
 

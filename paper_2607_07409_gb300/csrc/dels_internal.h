@@ -384,6 +384,10 @@ int device_max_smem_optin();
 // least `bytes`, once per kernel, device and size (safe from several host
 // threads; the attribute is per device).
 cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes);
+// G = E W^T: E [V, D] and W [O, D] bf16, G [V, O] float32, all row-major and
+// 16-byte aligned, D and O multiples of 16.
+cudaError_t launch_input_table(const uint16_t* E, const uint16_t* W, float* G, int V, int O, int D, int* status,
+                               int sms, cudaStream_t s);
 bool encode_tmap_2d(CUtensorMap* m, const void* base, CUtensorMapDataType dt, int elem_bytes, uint64_t inner,
                     uint64_t outer, uint64_t row_pitch_bytes, uint32_t box_inner, uint32_t box_outer,
                     CUtensorMapSwizzle swz);

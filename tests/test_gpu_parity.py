@@ -300,6 +300,34 @@ def test_gru_input_table_is_the_input_product(V):
     assert torch.all((got - ref).abs() <= bound), float(((got - ref).abs() / bound).max())
 
 
+@pytest.mark.parametrize("V,D,H", [
+    (1, 16, 16),         # one row, one ragged K chunk, 48 columns
+    (255, 80, 16),       # a row and a K tail inside one tile
+    (257, 64, 96),       # one row into the second pair of row blocks, 288 columns
+    (600, 1040, 176),    # 528 columns: the last tile holds 16
+    (20000, 128, 256),   # more tiles than CTA pairs: both accumulator buffers reused
+])
+def test_gru_input_table_tile_edges(V, D, H):
+    g = torch.Generator(device=DEV).manual_seed(V + D + H)
+    E = torch.randn(V, D, generator=g, device=DEV).to(torch.bfloat16)
+    Wih = torch.randn(3 * H, D, generator=g, device=DEV).to(torch.bfloat16)
+    spec = synth.HeadSpec("gru", "bf16", d_model=D, d_hidden=H, d_rank=16)
+    head = dels.make_head(spec, {"emb": E, "w_ih": Wih, "w_vocab": E})
+    nbytes = dels.dels_gru_input_table_bytes(head, V)
+    assert nbytes == V * 3 * H * 4
+    buf = torch.full((V * 3 * H + 1024,), -7.0, device=DEV)
+    ws = _ws(256)
+    r = dels.dels_gru_build_input_table(head, V, buf, nbytes, ws, 256)
+    assert r == 0, dels.dels_status_string(r)
+    torch.cuda.synchronize()
+    assert _status(ws) == 0
+    got, ref = buf[:V * 3 * H].view(V, 3 * H).double(), E.double() @ Wih.double().T
+    # exact products, a float32 sum of D terms (as in the test above)
+    bound = D * 2.0 ** -23 * (E.double().abs() @ Wih.double().abs().T) + 1e-30
+    assert torch.all((got - ref).abs() <= bound), float(((got - ref).abs() / bound).max())
+    assert torch.all(buf[V * 3 * H:] == -7.0)      # nothing past the table is written
+
+
 @pytest.mark.parametrize("stress", [False, True])
 @pytest.mark.parametrize("name", ["gru", "gru_b64"])
 def test_draft_with_input_table_matches_oracle(name, stress):
