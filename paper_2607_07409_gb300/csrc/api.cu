@@ -1223,6 +1223,36 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
   mb.smp.R = head->d_rank;
   mb.smp.r_bytes = es;
 
+  // float32 heads: the vocabulary projection of position j from `feat` [B, K]
+  VocabF32Args vf{};
+  int vf_chunks = 0;
+  auto vocab_f32 = [&](const void* feat, int K, int j) {
+    if (vf_chunks == 0) {
+      vf_chunks = vocab_f32_chunks(B, K, V, L.partial_ld, sms, &vf.chunk_rows);
+      vf.feat = static_cast<const float*>(feat);
+      vf.W = static_cast<const float*>(head->w_vocab);
+      vf.K = K;
+      vf.B = B;
+      vf.V = V;
+      vf.long_f32 = logit_dtype == DELS_F32;
+      vf.ld_long = (long long)n * V;
+      vf.prior = log_prior;
+      vf.partials = partials;
+      vf.partial_ld = L.partial_ld;
+      vf.smp = sm;
+    }
+    vf.longp = static_cast<const uint8_t*>(long_logits) + (size_t)j * V * (logit_dtype == DELS_F32 ? 4 : 2);
+    vf.alpha = aw(j);
+    vf.beta = bw(j);
+    vf.j = j;
+    PROF(DELS_KCLASS_VOCAB_COMBINE);
+    return launch_vocab_combine_f32(vf, vf_chunks, s);
+  };
+  auto gemv_f32 = [&](const GemvF32Jobs& jobs, int njobs, int O, int act) {
+    PROF(DELS_KCLASS_HEAD_MISC);
+    return launch_gemv_f32(jobs, njobs, B, O, act, O, sms, s);
+  };
+
   switch (head->kind) {
     case DELS_HEAD_GRU: {
       const int D = head->d_model, H = head->d_hidden, R = head->d_rank;
@@ -1489,19 +1519,17 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         const float* Whh = static_cast<const float*>(head->w[1]);
         const float* Wr = static_cast<const float*>(head->w[2]);
         float* feat = static_cast<float*>(rr);
-        const int nch = std::max(1, std::min(L.partial_ld, (V + 255) / 256));
+        GemvF32Jobs gates{}, rank{};
+        gates.j[0] = GemvF32Job{E, Wih, gpart, D, D};
+        gates.j[1] = GemvF32Job{h, Whh, gpart + (size_t)B * 3 * H, H, H};
+        rank.j[0] = GemvF32Job{h, Wr, feat, H, H};
         for (int j = 1; j < n; ++j) {
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gemv_f32(E, D, Wih, B, 3 * H, D, ACT_NONE, gpart, 3 * H, s)); }
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gemv_f32(h, H, Whh, B, 3 * H, H, ACT_NONE, gpart + (size_t)B * 3 * H, 3 * H, s)); }
+          DELS_CUDA(gemv_f32(gates, 2, 3 * H, ACT_NONE));
           { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, 1, 1, B, H, h, hb, s)); }
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gemv_f32(h, H, Wr, B, R, H, ACT_SILU, feat, R, s)); }
-          { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(launch_vocab_combine_f32(feat, R, static_cast<const float*>(head->w_vocab),
-                                             static_cast<const uint8_t*>(long_logits) +
-                                                 (size_t)j * V * (logit_dtype == DELS_F32 ? 4 : 2),
-                                             logit_dtype == DELS_F32, (long long)n * V, log_prior, aw(j), bw(j), B, V,
-                                             partials, L.partial_ld, nch, status, s, &sm, j)); }
+          DELS_CUDA(gemv_f32(rank, 1, R, ACT_SILU));
+          DELS_CUDA(vocab_f32(feat, R, j));
           MergeArgs m = mb;
-          m.count = nch;
+          m.count = vf_chunks;
           m.j = j;
           if (j == n - 1) m.table = nullptr;
           { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
@@ -1570,21 +1598,17 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
         }
       } else {
-        const int nch = std::max(1, std::min(L.partial_ld, (V + 255) / 256));
+        GemvF32Jobs l1{}, l2{};
+        l1.j[0] = GemvF32Job{static_cast<const float*>(u), static_cast<const float*>(head->w[0]),
+                             static_cast<float*>(h1), K1, K1};
+        l2.j[0] = GemvF32Job{static_cast<const float*>(h1), static_cast<const float*>(head->w[1]),
+                             static_cast<float*>(h2), Hd, Hd};
         for (int j = 1; j < n; ++j) {
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gemv_f32(static_cast<const float*>(u), K1, static_cast<const float*>(head->w[0]), B, Hd,
-                                    K1, ACT_GELU, static_cast<float*>(h1), Hd, s)); }
-          if (head->n_layers == 2)
-            { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gemv_f32(static_cast<const float*>(h1), Hd, static_cast<const float*>(head->w[1]), B,
-                                      Hd, Hd, ACT_GELU, static_cast<float*>(h2), Hd, s)); }
-          { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(launch_vocab_combine_f32(static_cast<const float*>(feat), Hd,
-                                             static_cast<const float*>(head->w_vocab),
-                                             static_cast<const uint8_t*>(long_logits) +
-                                                 (size_t)j * V * (logit_dtype == DELS_F32 ? 4 : 2),
-                                             logit_dtype == DELS_F32, (long long)n * V, log_prior, aw(j), bw(j), B, V,
-                                             partials, L.partial_ld, nch, status, s, &sm, j)); }
+          DELS_CUDA(gemv_f32(l1, 1, Hd, ACT_GELU));
+          if (head->n_layers == 2) DELS_CUDA(gemv_f32(l2, 1, Hd, ACT_GELU));
+          DELS_CUDA(vocab_f32(feat, Hd, j));
           MergeArgs m = mb;
-          m.count = nch;
+          m.count = vf_chunks;
           m.j = j;
           if (j == n - 1) m.table = nullptr;
           { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
@@ -1682,7 +1706,6 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       if (bf && !plan_combine(gv, B, V, n, feat, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
                               partials, L.partial_ld, status, sms, true))
         return DELS_ERR_CUDA;
-      const int nch = std::max(1, std::min(L.partial_ld, (V + 255) / 256));
       for (int j = 1; j < n; ++j) {
         int count;
         if (bf) {
@@ -1695,13 +1718,8 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
           count = gv.grid;
         } else {
-          { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(launch_vocab_combine_f32(static_cast<const float*>(feat), R,
-                                             static_cast<const float*>(head->w_vocab),
-                                             static_cast<const uint8_t*>(long_logits) +
-                                                 (size_t)j * V * (logit_dtype == DELS_F32 ? 4 : 2),
-                                             logit_dtype == DELS_F32, (long long)n * V, log_prior, aw(j), bw(j), B, V,
-                                             partials, L.partial_ld, nch, status, s, &sm, j)); }
-          count = nch;
+          DELS_CUDA(vocab_f32(feat, R, j));
+          count = vf_chunks;
         }
         MergeArgs m = mb;
         m.count = count;
@@ -1897,10 +1915,10 @@ int dels_verify_block_sampled(const dels_local_head* head, const int32_t* draft_
       return DELS_ERR_CUDA;
     { PROF(DELS_KCLASS_VERIFY); DELS_CUDA(run(g, s)); }
   } else {
-    { PROF(DELS_KCLASS_VERIFY);
-      DELS_CUDA(launch_gemv_f32(static_cast<const float*>(a.rg), head->d_rank,
-                                static_cast<const float*>(head->w_vocab), B, V, head->d_rank, ACT_NONE,
-                                at<float>(workspace, L.ls), V, s)); }
+    GemvF32Jobs jobs{};
+    jobs.j[0] = GemvF32Job{static_cast<const float*>(a.rg), static_cast<const float*>(head->w_vocab),
+                           at<float>(workspace, L.ls), head->d_rank, head->d_rank};
+    { PROF(DELS_KCLASS_VERIFY); DELS_CUDA(launch_gemv_f32(jobs, 1, B, V, ACT_NONE, V, sms, s)); }
   }
   // 4. the bonus draw: the residual at the rejection, or p_n after n acceptances
   { PROF(DELS_KCLASS_VERIFY); DELS_CUDA(launch_residual_rows(a, s)); }

@@ -44,6 +44,12 @@ __device__ __forceinline__ uint16_t f32_to_bf16_rne(float f) {
   return (uint16_t)(u >> 16);
 }
 
+__device__ __forceinline__ float act_f(int act, float x) {
+  if (act == ACT_SILU) return x / (1.f + __expf(-x));
+  if (act == ACT_GELU) return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
+  return x;
+}
+
 // ----------------------------------------------------------------------------
 // RowAcc: top-1 / top-2 / online log-sum-exp of one row
 // ----------------------------------------------------------------------------

@@ -356,8 +356,6 @@ cudaError_t launch_xfmr_embed(const uint16_t* e_rows, const uint16_t* pos_table,
                               float* t_out, uint16_t* a_bf16, cudaStream_t s, int terms = 1);
 cudaError_t launch_attention(const float* q, const float* kcache, const float* vcache, int B, int D, int nh,
                              int npos, int cache_ld_pos, uint16_t* o_bf16, cudaStream_t s, int terms = 1);
-cudaError_t launch_gemv_f32(const float* X, int ldx, const float* W, int B, int O, int K, int act, float* Y,
-                            int ldy, cudaStream_t s);
 // bf16 weights and activations, bf16 output after the activation, B <= kGemvBf16MaxRows.
 constexpr int kGemvBf16MaxRows = 4;
 // the X rows are staged in (at most 48 KB of) shared memory
@@ -366,11 +364,39 @@ inline bool gemv_bf16_ok(int B, int K) {
 }
 cudaError_t launch_gemv_bf16(const uint16_t* X, int ldx, const uint16_t* W, int B, int O, int K, int act,
                              uint16_t* Y, int ldy, cudaStream_t s);
-cudaError_t launch_vocab_combine_f32(const float* feat, int K, const float* Wv, const void* longp, int long_f32,
-                                     long long ld_long, const float* prior, float alpha, float beta, int B,
-                                     int V, void* partials, int partial_ld, int nchunks, int* status,
-                                     cudaStream_t s,
-                                     const SampleArgs* smp = nullptr, int j = 0);
+// float32 products of one or two jobs with the same O, B and output pitch:
+// Y[b, o] = act(sum_k X[b, k] W[o, k]); K a multiple of 4, X 16-byte aligned.
+struct GemvF32Job {
+  const float* X;
+  const float* W;
+  float* Y;
+  int ldx, K;
+};
+struct GemvF32Jobs {
+  GemvF32Job j[2];
+};
+cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, int act, int ldy, int sms,
+                            cudaStream_t s);
+// float32 vocabulary projection fused with the combine: one record per
+// (request, vocabulary chunk of chunk_rows rows).
+struct VocabF32Args {
+  const float* feat;             // [B, K]
+  const float* W;                // [V, K]
+  int K, B, V;
+  const void* longp;             // position j's rows, pitch ld_long elements
+  int long_f32;
+  long long ld_long;
+  const float* prior;
+  float alpha, beta;
+  int chunk_rows;
+  void* partials;
+  int partial_ld;
+  int j;
+  SampleArgs smp;
+};
+// Chunks (records per request) and the rows of each.
+int vocab_f32_chunks(int B, int K, int V, int partial_ld, int sms, int* chunk_rows);
+cudaError_t launch_vocab_combine_f32(const VocabF32Args& a, int nchunks, cudaStream_t s);
 
 // ---- host utilities ---------------------------------------------------------
 // Host-side checks of dels_combine_argmax's input and output pointers (NULL,

@@ -1,7 +1,7 @@
 // Element-wise and small reduction kernels of the local heads (Appendix A
 // GRU head; the window-MLP and transformer heads of the synthetic
-// workloads), plus the float32 CUDA-core path used when the head's weights
-// are float32. The large matrix products of bf16 heads run in tc_gemm.cu.
+// workloads). The large matrix products of bf16 heads run in tc_gemm.cu, the
+// float32 heads' in heads_f32.cu.
 #include <climits>
 
 #include <algorithm>
@@ -13,12 +13,6 @@ namespace dels {
 namespace {
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + __expf(-x)); }
-
-__device__ __forceinline__ float act_f(int act, float x) {
-  if (act == ACT_SILU) return x / (1.f + __expf(-x));
-  if (act == ACT_GELU) return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
-  return x;
-}
 
 // GRU gates (PyTorch bias-free form; gate rows r, z, n):
 //   gi = sum of the S0 input-product partials, gh = sum of the S1 recurrent ones
@@ -482,85 +476,6 @@ __global__ void k_gemv_bf16(const uint16_t* __restrict__ X, int ldx, const uint1
   }
 }
 
-// float32 skinny product on CUDA cores: Y[b, o] = act(sum_k X[b, k] W[o, k]);
-// one warp per output row o, lanes stride over k, all batch rows at once.
-template <int BMAX>
-__global__ void k_gemv_f32(const float* __restrict__ X, int ldx, const float* __restrict__ W, int B, int O, int K,
-                           int act, float* __restrict__ Y, int ldy) {
-  if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
-  const int lane = threadIdx.x & 31;
-  const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (o >= O) return;
-  const float* w = W + (long long)o * K;
-  for (int b0 = 0; b0 < B; b0 += BMAX) {
-    float acc[BMAX];
-#pragma unroll
-    for (int i = 0; i < BMAX; ++i) acc[i] = 0.f;
-    for (int k = lane; k < K; k += 32) {
-      const float wk = w[k];
-#pragma unroll
-      for (int i = 0; i < BMAX; ++i)
-        if (b0 + i < B) acc[i] = fmaf(wk, X[(long long)(b0 + i) * ldx + k], acc[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < BMAX; ++i) {
-      float v = acc[i];
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, d);
-      if (lane == 0 && b0 + i < B) Y[(long long)(b0 + i) * ldy + o] = act_f(act, v);
-    }
-  }
-}
-
-// float32 vocabulary projection fused with the combine: CTA (chunk, b)
-// computes l_S[v] = W_vocab[v] . feat[b] for its vocabulary chunk (one warp
-// per row v), fuses l = l_L + alpha l_S - beta l_P and reduces to one RowAcc.
-__global__ void __launch_bounds__(256) k_vocab_combine_f32(const float* __restrict__ feat, int K,
-                                                           const float* __restrict__ Wv, const void* longp,
-                                                           int long_f32, long long ld_long,
-                                                           const float* __restrict__ prior, float alpha, float beta,
-                                                           int V, void* partials, int partial_ld, int nchunks,
-                                                           int* status, SampleArgs smp, int j) {
-  if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
-  const int chunk = blockIdx.x % nchunks, b = blockIdx.x / nchunks;
-  const int per = (V + nchunks - 1) / nchunks;
-  const int v0 = chunk * per, v1 = min(V, v0 + per);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const float* fb = feat + (long long)b * K;
-  float best = -INFINITY, second = -INFINITY, m = -INFINITY, s = 0.f;
-  int idx = INT_MAX;
-  for (int v = v0 + warp; v < v1; v += nw) {
-    const float* w = Wv + (long long)v * K;
-    float d = 0.f;
-    for (int k = lane; k < K; k += 32) d = fmaf(w[k], fb[k], d);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xFFFFFFFFu, d, o);
-    const float l = long_f32 ? static_cast<const float*>(longp)[(long long)b * ld_long + v]
-                             : bf16_to_f(static_cast<const uint16_t*>(longp)[(long long)b * ld_long + v]);
-    float f[1] = {fmaf(-beta, prior[v], fmaf(alpha, d, l))};
-    // temperature 1: the top-2 over the keys f + g (see write_decode_sampled)
-    const float key = smp.on ? f[0] + gumbel_at(smp.seed, smp.step, b, j, kStreamDraft, v) : f[0];
-    top2_push(key, v, best, second, idx);
-    lse_chunk<1>(f, best, m, s);
-  }
-  RowAcc r;
-  r.m = best; r.s = s; r.second = second; r.idx = idx;
-  // lanes of a warp hold identical states; merge across warps
-  __shared__ RowAcc red[32];
-  if (lane == 0) red[warp] = r;
-  __syncthreads();
-  if (warp == 0) {
-    RowAcc x = lane < nw ? red[lane] : rowacc_init();
-    x = rowacc_warp_reduce(x);
-    if (lane == 0)
-      reinterpret_cast<float4*>(partials)[(long long)b * partial_ld + chunk] =
-          make_float4(x.m, x.s, x.second, __int_as_float(x.idx));
-  }
-  (void)status;
-}
-
 inline int grid_for(long long total, int threads) {
   long long g = (total + threads - 1) / threads;
   return (int)std::min<long long>(std::max<long long>(g, 1), 65535LL * 16);
@@ -626,22 +541,6 @@ cudaError_t launch_gemv_bf16(const uint16_t* X, int ldx, const uint16_t* W, int 
   const int warps = 4;
   return launch_pdl(k_gemv_bf16<kGemvBf16MaxRows>, dim3((O + warps - 1) / warps), dim3(warps * 32),
                     (size_t)B * K * 2, s, X, ldx, W, B, O, K, act, Y, ldy);
-}
-
-cudaError_t launch_gemv_f32(const float* X, int ldx, const float* W, int B, int O, int K, int act, float* Y, int ldy,
-                            cudaStream_t s) {
-  const int warps = 8;
-  return launch_pdl(k_gemv_f32<8>, dim3((O + warps - 1) / warps), dim3(warps * 32), 0, s, X, ldx, W, B, O, K, act, Y,
-                    ldy);
-}
-
-cudaError_t launch_vocab_combine_f32(const float* feat, int K, const float* Wv, const void* longp, int long_f32,
-                                     long long ld_long, const float* prior, float alpha, float beta, int B, int V,
-                                     void* partials, int partial_ld, int nchunks, int* status, cudaStream_t s,
-                                     const SampleArgs* smp, int j) {
-  const SampleArgs sm = smp ? *smp : SampleArgs{};
-  return launch_pdl(k_vocab_combine_f32, dim3(B * nchunks), dim3(256), 0, s, feat, K, Wv, longp, long_f32, ld_long,
-                    prior, alpha, beta, V, partials, partial_ld, nchunks, status, sm, j);
 }
 
 }  // namespace dels

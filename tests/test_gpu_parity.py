@@ -261,6 +261,24 @@ def test_draft_small_matches_oracle(name, stress):
     print(name, stress, record(f"draft {name}, stress {stress}", info))
 
 
+@pytest.mark.parametrize("head,B,V,d,h,r", [
+    ("gru", 1, 1000, 132, 36, 20),          # one request; widths just past and below a 128-wide step
+    ("gru", 2, 72, 8, 4, 4),                # two requests, the smallest widths
+    ("gru", 9, 4104, 260, 128, 132),        # a second group of one request
+    ("mlp", 4, 2000, 64, 520, 520),         # four requests
+    ("mlp", 17, 1504, 32, 100, 100),        # three groups
+    ("markov", 3, 136, 0, 0, 12000),        # two requests' rows fit the staging limit
+    ("markov", 6, 64, 0, 0, 24580),         # not one row does: the rows are read through L2
+])
+def test_draft_f32_head_tile_edges(head, B, V, d, h, r):
+    spec = synth.HeadSpec(head, "f32", d, h, r, window=3, n_layers=2)
+    w = synth.stress(synth.Workload("f32_edges", B=B, n=4, V=V, logit_dtype="bf16" if B == 9 else "f32", head=spec,
+                                    weight=0.5, seed=B))
+    dd = synth.make_inputs(w, device=DEV, target=False)
+    tok, lp, gap, W, prior = _draft(w, dd)
+    check_draft(tok, lp, gap, _oracle_head(w, W), dd["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_F32)
+
+
 @pytest.mark.parametrize("stress", [False, True])
 @pytest.mark.parametrize("name", ["gru", "gru_b64"])
 def test_draft_persistent_kernel_matches_oracle(name, stress, monkeypatch):
