@@ -12,13 +12,17 @@
 // tiles fastest, so that the pairs running at one time share a few row blocks
 // of E and all of W_ih (25 MB) in L2: E is read from memory once.
 //
-// Measured at V = 151936, D = 4096, H = 1024: 2.64 ms, 1.45 PFLOP/s; 32.2 ms
+// Measured at V = 151936, D = 4096, H = 1024: 2.78 ms, 1.38 PFLOP/s; 32.2 ms
 // with one launch of 24 CTAs per 128 rows of E, as it was before.
 //
-// Roles: warp 0 loads (TMA, a ring of 6 K chunks), warp 1 issues the MMAs (the pair's
-// even CTA), warps 2..5 store: accumulators are double-buffered in TMEM (2 x
-// 256 columns), so a tile's stores (TMA, through two 4 KB staging buffers per
-// warp) run under the next tile's products.
+// Roles: warp 0 loads (TMA, a ring of 6 K chunks), warp 1 issues the MMAs (the
+// pair's even CTA), warps 4..11 keep the sums and store. The tensor cores
+// accumulate a segment of 512 along K at a time in one of two TMEM buffers;
+// the sum warps add the segments in registers (128 columns per thread) under
+// the next segment's products, rounding to nearest, where one accumulator over
+// all of K truncates at every step (error against float64 at D = 4096 4.4e-6
+// with one accumulator, 4.8e-7 with segments, for 5 % more time). A tile's stores
+// (TMA, through a 4 KB staging buffer per warp) run under the next tile.
 #include <algorithm>
 
 #include "dels_device.cuh"
@@ -31,10 +35,15 @@ constexpr int kTM = 256, kTN = 256;          // a pair's tile
 constexpr int kTK = 64;                      // K chunk (one 128-byte swizzled row)
 constexpr int kChunkBytes = 128 * 128;       // 128 rows of one K chunk
 constexpr int kRing = 6;                     // K chunks of E and of W_ih that the stages hold
-constexpr int kStoreWarps = 4;
+constexpr int kSegChunks = 8;                // K chunks accumulated in TMEM before they are added up
+constexpr int kStoreWarps = 8;               // two per TMEM lane quadrant, 128 columns each
 constexpr int kStoreBytes = 32 * 128;        // one staging buffer: 32 rows x 32 floats
-constexpr int kThreads = (2 + kStoreWarps) * 32;
-constexpr int kTableSmem = 2 * kRing * kChunkBytes + kStoreWarps * 2 * kStoreBytes + 256 + 1024;
+constexpr int kSumWarp0 = 4;                 // after the loading, issuing and two idle warps of the first warpgroup
+constexpr int kThreads = (kSumWarp0 + kStoreWarps) * 32;
+// Registers: 168 per thread at launch (12 warps); the first warpgroup keeps
+// 56 and the two that hold the sums take 224 (128 x 56 + 256 x 224 = 384 x 168).
+constexpr int kRegsFew = 56, kRegsMany = 224;
+constexpr int kTableSmem = 2 * kRing * kChunkBytes + kStoreWarps * kStoreBytes + 256 + 1024;
 
 __device__ __forceinline__ void tmem_alloc2(uint32_t* smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)),
@@ -102,7 +111,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
   uint8_t* staging = smem + kStages * kStageBytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kStoreWarps * 2 * kStoreBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kStoreWarps * kStoreBytes);
   uint64_t* full = bars;                 // [kStages], the even CTA's: both CTAs' bytes
   uint64_t* empty = bars + kStages;      // [kStages], in each CTA
   uint64_t* accf = empty + kStages;      // [2], in each CTA
@@ -143,107 +152,134 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   const int chunks = (D + kTK - 1) / kTK;
   const int fills = (chunks + C - 1) / C;                // stages per tile; the last may hold fewer chunks
+  constexpr int kSegFills = kSegChunks / C;
+  const int segs = (fills + kSegFills - 1) / kSegFills;  // accumulations per tile
 
-  if (warp == 0) {
-    if (lane == 0) {
-      const uint64_t pol_e = l2_policy_evict_normal();
-      const uint64_t pol_w = l2_policy_evict_last();   // read by every pair for every row block
-      int f = 0;
-      bool ok = true;
-      for (int t = pair; t < tiles && ok; t += pairs) {
-        const uint64_t deadline = globaltimer_ns() + budget_ns;   // of each tile: a table may take longer
-        const int m0 = (t / nt) * kTM + (int)rank * 128, n0 = (t % nt) * kTN + (int)rank * 128;
-        for (int k = 0; k < fills; ++k, ++f) {
-          const int s = f % kStages;
-          ok = mbar_wait(&empty[s], ((f / kStages) & 1) ^ 1, deadline, abort_flag);
-          if (!ok) break;
-          const uint32_t bar = cluster_map(smem_u32(&full[s]), 0);
-          if (rank == 0)
-            mbar_arrive_expect_tx(&full[s], 2u * kStageBytes);   // both CTAs' loads
-          else
-            mbar_arrive_remote(bar);
-          uint8_t* dst = smem + s * kStageBytes;
-          if constexpr (C == 1) {
-            tma_load_2d_pair(dst, &mE, bar, k * kTK, m0, pol_e);
-            tma_load_2d_pair(dst + kStageBytes / 2, &mW, bar, k * kTK, n0, pol_w);
-          } else {
-            tma_load_3d_pair(dst, &mE, bar, 0, m0, k * C, pol_e);
-            tma_load_3d_pair(dst + kStageBytes / 2, &mW, bar, 0, n0, k * C, pol_w);
+  if (warp < kSumWarp0) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
+    if (warp == 0) {
+      if (lane == 0) {
+        const uint64_t pol_e = l2_policy_evict_normal();
+        const uint64_t pol_w = l2_policy_evict_last();   // read by every pair for every row block
+        int f = 0;
+        bool ok = true;
+        for (int t = pair; t < tiles && ok; t += pairs) {
+          const uint64_t deadline = globaltimer_ns() + budget_ns;   // of each tile: a table may take longer
+          const int m0 = (t / nt) * kTM + (int)rank * 128, n0 = (t % nt) * kTN + (int)rank * 128;
+          for (int k = 0; k < fills; ++k, ++f) {
+            const int s = f % kStages;
+            ok = mbar_wait(&empty[s], ((f / kStages) & 1) ^ 1, deadline, abort_flag);
+            if (!ok) break;
+            const uint32_t bar = cluster_map(smem_u32(&full[s]), 0);
+            if (rank == 0)
+              mbar_arrive_expect_tx(&full[s], 2u * kStageBytes);   // both CTAs' loads
+            else
+              mbar_arrive_remote(bar);
+            uint8_t* dst = smem + s * kStageBytes;
+            if constexpr (C == 1) {
+              tma_load_2d_pair(dst, &mE, bar, k * kTK, m0, pol_e);
+              tma_load_2d_pair(dst + kStageBytes / 2, &mW, bar, k * kTK, n0, pol_w);
+            } else {
+              tma_load_3d_pair(dst, &mE, bar, 0, m0, k * C, pol_e);
+              tma_load_3d_pair(dst + kStageBytes / 2, &mW, bar, 0, n0, k * C, pol_w);
+            }
           }
         }
+        // after an abort, wait (bounded) for the loads issued to land
+        if (!ok && rank == 0) {
+          const uint64_t dd = globaltimer_ns() + 100000000ull;
+          volatile int dummy = 0;
+          for (int k = max(0, f - kStages); k < f; ++k) mbar_wait(&full[k % kStages], (k / kStages) & 1, dd, &dummy);
+        }
       }
-      // after an abort, wait (bounded) for the loads issued to land
-      if (!ok && rank == 0) {
-        const uint64_t dd = globaltimer_ns() + 100000000ull;
-        volatile int dummy = 0;
-        for (int k = max(0, f - kStages); k < f; ++k) mbar_wait(&full[k % kStages], (k / kStages) & 1, dd, &dummy);
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc = idesc_bf16_f32(kTM, kTN);
-      int f = 0, i = 0;
-      bool ok = true;
-      for (int t = pair; t < tiles && ok; t += pairs, ++i) {
-        const int buf = i & 1;
-        const uint64_t deadline = globaltimer_ns() + budget_ns;
-        ok = mbar_wait_cluster(&acce[buf], ((i >> 1) & 1) ^ 1, deadline, abort_flag);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(buf * kTN);
-        for (int k = 0; k < fills; ++k, ++f) {
-          const int s = f % kStages;
-          ok = mbar_wait_cluster(&full[s], (f / kStages) & 1, deadline, abort_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t ea = smem_u32(smem + s * kStageBytes), wa = ea + kStageBytes / 2;
+    } else if (warp == 1) {
+      if (lane == 0 && rank == 0) {
+        const uint32_t idesc = idesc_bf16_f32(kTM, kTN);
+        int f = 0, i = 0;
+        bool ok = true;
+        for (int t = pair; t < tiles && ok; t += pairs) {
+          const uint64_t deadline = globaltimer_ns() + budget_ns;
+          for (int k = 0; k < fills && ok; ++i) {
+            const int buf = i & 1;
+            ok = mbar_wait_cluster(&acce[buf], ((i >> 1) & 1) ^ 1, deadline, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t d = tmem + (uint32_t)(buf * kTN);
+            const int k0 = k, k1 = min(fills, k + kSegFills);
+            for (; k < k1; ++k, ++f) {
+              const int s = f % kStages;
+              ok = mbar_wait_cluster(&full[s], (f / kStages) & 1, deadline, abort_flag);
+              if (!ok) break;
+              tc_fence_after();
+              const uint32_t ea = smem_u32(smem + s * kStageBytes), wa = ea + kStageBytes / 2;
 #pragma unroll
-          for (int kk = 0; kk < C * kTK / 16; ++kk) {
-            const uint32_t off = (kk / 4) * kChunkBytes + (kk % 4) * 32;
-            if (C == 1 || k * C + kk / 4 < chunks)
-              tc_mma2_f16(d, smem_desc_sw128(ea + off), smem_desc_sw128(wa + off), idesc, (k > 0 || kk > 0) ? 1u : 0u);
+              for (int kk = 0; kk < C * kTK / 16; ++kk) {
+                const uint32_t off = (kk / 4) * kChunkBytes + (kk % 4) * 32;
+                if (C == 1 || k * C + kk / 4 < chunks)
+                  tc_mma2_f16(d, smem_desc_sw128(ea + off), smem_desc_sw128(wa + off), idesc,
+                              (k > k0 || kk > 0) ? 1u : 0u);
+              }
+              tc_commit2(&empty[s]);
+            }
+            if (ok) tc_commit2(&accf[buf]);
           }
-          tc_commit2(&empty[s]);
         }
-        if (ok) tc_commit2(&accf[buf]);
-      }
-      if (!ok) {
-        tc_commit2(mmadone);   // the MMAs issued have completed before TMEM is freed
-        volatile int dummy = 0;
-        mbar_wait(mmadone, 0, globaltimer_ns() + 100000000ull, &dummy);
+        if (!ok) {
+          tc_commit2(mmadone);   // the MMAs issued have completed before TMEM is freed
+          volatile int dummy = 0;
+          mbar_wait(mmadone, 0, globaltimer_ns() + 100000000ull, &dummy);
+        }
       }
     }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsMany));
     const int q = warp & 3;                                    // TMEM lane quadrant
-    uint8_t* stage = staging + (warp - 2) * 2 * kStoreBytes;
+    const int half = (warp - kSumWarp0) >> 2;                  // columns [128 half, 128 half + 128)
+    uint8_t* stage = staging + (warp - kSumWarp0) * kStoreBytes;
     const uint64_t pol = l2_policy_evict_first();
-    int i = 0, sb = 0;
-    for (int t = pair; t < tiles; t += pairs, ++i) {
-      const int buf = i & 1;
-      if (!mbar_wait(&accf[buf], (i >> 1) & 1, globaltimer_ns() + budget_ns, abort_flag)) break;
-      tc_fence_after();
-      const int m0 = (t / nt) * kTM + (int)rank * 128 + q * 32, n0 = (t % nt) * kTN;
-      const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kTN);
-      for (int c = 0; c < kTN / 32; ++c) {
-        if (n0 + c * 32 >= O) break;                           // whole chunks past the table's width
-        float acc[32];
-        tmem_ld_32x32b_x32(base + (uint32_t)(c * 32), acc);
-        tmem_ld_wait();
-        // the buffer's previous store has been read out (one store may stay in flight)
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-        __syncwarp();
-        float4* dst = reinterpret_cast<float4*>(stage + sb * kStoreBytes + lane * 128);
+    int i = 0;
+    bool ok = true;
+    for (int t = pair; t < tiles && ok; t += pairs) {
+      const uint64_t deadline = globaltimer_ns() + budget_ns;
+      float sum[kTN / 2];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          dst[k ^ (lane & 7)] = make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      for (int x = 0; x < kTN / 2; ++x) sum[x] = 0.f;
+      for (int sg = 0; sg < segs; ++sg, ++i) {
+        const int buf = i & 1;
+        ok = mbar_wait(&accf[buf], (i >> 1) & 1, deadline, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kTN + half * (kTN / 2));
+#pragma unroll
+        for (int c = 0; c < kTN / 64; ++c) {
+          float acc[32];
+          tmem_ld_32x32b_x32(base + (uint32_t)(c * 32), acc);
+          tmem_ld_wait();
+#pragma unroll
+          for (int x = 0; x < 32; ++x) sum[c * 32 + x] += acc[x];
+        }
+        tc_fence_before();
         __syncwarp();
-        if (lane == 0 && m0 < V) tma_store_2d(&mG, stage + sb * kStoreBytes, n0 + c * 32, m0, pol);
-        sb ^= 1;
+        if (lane == 0) mbar_arrive_remote(cluster_map(smem_u32(&acce[buf]), 0));
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_remote(cluster_map(smem_u32(&acce[buf]), 0));
+      if (!ok) break;
+      const int m0 = (t / nt) * kTM + (int)rank * 128 + q * 32, n0 = (t % nt) * kTN + half * (kTN / 2);
+#pragma unroll
+      for (int c = 0; c < kTN / 64; ++c) {
+        if (n0 + c * 32 < O) {                                 // not whole chunks past the table's width
+          // the staging buffer's previous store has been read out
+          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          __syncwarp();
+          float4* dst = reinterpret_cast<float4*>(stage + lane * 128);
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            dst[k ^ (lane & 7)] =
+                make_float4(sum[c * 32 + 4 * k], sum[c * 32 + 4 * k + 1], sum[c * 32 + 4 * k + 2], sum[c * 32 + 4 * k + 3]);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0 && m0 < V) tma_store_2d(&mG, stage, n0 + c * 32, m0, pol);
+        }
+      }
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
@@ -265,8 +301,9 @@ cudaError_t launch_input_table(const uint16_t* E, const uint16_t* W, float* G, i
   CUtensorMap mE, mW, mG;
   // Two K chunks per stage, each operand's as one 3-D box whose rows are
   // 256-byte spans, where the width is whole chunks (the 3-D view has no
-  // ragged tail): 2.64 ms for the table above, against 4.55 ms with one chunk
-  // (128-byte spans) per box, which the loads bind (30 GB at 6.6 TB/s).
+  // ragged tail): 2.64 ms for the table above before its segments, against
+  // 4.55 ms with one chunk (128-byte spans) per box, which the loads bind (30
+  // GB at 6.6 TB/s).
   const bool pair = D % kTK == 0;
   auto load_map = [&](CUtensorMap* m, const uint16_t* x, int rows) {
     return pair ? encode_tmap_3d(m, x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kTK, (uint64_t)rows, (uint64_t)(D / kTK),
