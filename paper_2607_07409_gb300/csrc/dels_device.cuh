@@ -96,7 +96,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// Hardware base-2 logarithm (PTX lg2.approx, flush-to-zero: one instruction,
+// where __log2f scales denormal arguments first; the same value for normal
+// ones).
+__device__ __forceinline__ float lg2_approx(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kLn2 = 0.693147180559945309f;
 
 // lse_chunk with the exponent pre-scaled to base 2: one FFMA + one ex2 per
 // element (exp(x - best) = 2^(x*log2e - best*log2e)). The running sum is
@@ -276,14 +286,16 @@ __device__ __forceinline__ float neg_log_uniform(float u) {
   p = fmaf(d, p, 0.5f);
   p = fmaf(d, p, 1.0f);
   const float near_one = d * p;
-  const float elsewhere = -0.693147180559945309f * __log2f(u);
+  const float elsewhere = -kLn2 * lg2_approx(u);   // u >= 2^-24: never denormal
   return d <= 0.125f ? near_one : elsewhere;
 }
 
 // Standard Gumbel variate g = -ln E = -ln(-ln u): E as above (its relative
-// error is what g's absolute error inherits), the outer logarithm through
-// the fast log. |g - g_exact| stays within a few 1e-6.
-__device__ __forceinline__ float gumbel_from_bits(uint32_t h) { return -__logf(neg_log_uniform(uniform_from_bits(h))); }
+// error is what g's absolute error inherits; E >= 5.9e-8), the outer logarithm
+// through the base-2 one. |g - g_exact| stays within a few 1e-6.
+__device__ __forceinline__ float gumbel_from_bits(uint32_t h) {
+  return -kLn2 * lg2_approx(neg_log_uniform(uniform_from_bits(h)));
+}
 
 // Key (seed mod 2^32, seed div 2^32), counter (c, step, b + 2^16 j + 2^24
 // stream, 0): the 4 uniforms of vocabulary indices 4c .. 4c + 3, one per
