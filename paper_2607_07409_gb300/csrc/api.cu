@@ -1792,8 +1792,9 @@ VerifySampledLayout verify_sampled_layout(const dels_local_head* head, int B, in
   const int es_t = tdt == DELS_F32 ? 4 : 2;
   const bool vec = (V % 8) == 0;
   const int rows = B * (n + 1);
-  L.t = plan_rows(std::max(rows, 1), V, es_t, sms, vec, 1 << 20);
-  L.r_nchunks = std::max(1, std::min((V + 2047) / 2048, (4 * sms + std::max(B, 1) - 1) / std::max(B, 1)));
+  L.t = plan_rows(std::max(rows, 1), V, es_t, sms, vec, 1 << 20, false, lse_slots_per_sm(tdt == DELS_F32));
+  // one wave of the residual kernel's four CTAs per SM, at least 2048 columns each
+  L.r_nchunks = std::max(1, std::min((V + 2047) / 2048, 4 * sms / std::max(B, 1)));
   L.r_chunk_cols = (int)round_up((size_t)((V + L.r_nchunks - 1) / L.r_nchunks), 8);
   L.r_nchunks = (V + L.r_chunk_cols - 1) / L.r_chunk_cols;
   const size_t es_w = head->wdtype == DELS_BF16 ? 2 : 4;
@@ -1856,20 +1857,18 @@ int dels_verify_block_sampled(const dels_local_head* head, const int32_t* draft_
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int* status = at<int>(workspace, 0);
   // 1. records of the target rows (their LSEs)
-  RowsArgs t{};
-  t.longp = target_logits;
+  const bool vec = (V % 8) == 0;
+  SampleRowsArgs t{};
+  t.src = target_logits;
+  t.ld = V;
   t.rows = B * (n + 1);
   t.V = V;
-  t.ld_long = V;
   t.chunk_cols = L.t.chunk_cols;
   t.nchunks = L.t.nchunks;
-  t.rows_per_cta = 1;
+  t.vec = vec;
   t.partials = at<void>(workspace, L.t_rec);
   t.partial_ld = L.t.nchunks;
-  t.status = status;
-  const int es_t = target_dtype == DELS_F32 ? 4 : 2;
-  const bool vec = (V % 8) == 0;
-  { PROF(DELS_KCLASS_VERIFY); DELS_CUDA(launch_combine_rows(t, target_dtype, vec, false, s)); }
+  { PROF(DELS_KCLASS_VERIFY); DELS_CUDA(launch_lse_rows(t, target_dtype == DELS_F32, s)); }
   // 2. the acceptance tests and the rejected position's input
   VerifySampledArgs a{};
   a.B = B;
@@ -1902,6 +1901,7 @@ int dels_verify_block_sampled(const dels_local_head* head, const int32_t* draft_
   a.r_records = at<void>(workspace, L.r_rec);
   a.r_nchunks = L.r_nchunks;
   a.r_chunk_cols = L.r_chunk_cols;
+  a.vec = vec && (!log_prior || aligned16(log_prior));
   a.out_accept = out_accept_len;
   a.out_bonus = out_bonus;
   a.out_bonus_gap = out_bonus_gap;

@@ -131,6 +131,10 @@ struct SampleRowsArgs {
   int partial_ld;
 };
 cudaError_t launch_sample_rows(const SampleRowsArgs& a, bool f32, cudaStream_t s);
+// Records of the rows' largest values and sums of exponentials (the seed,
+// step, stream and position fields are not used).
+cudaError_t launch_lse_rows(const SampleRowsArgs& a, bool f32, cudaStream_t s);
+int lse_slots_per_sm(bool f32);   // resident CTAs per SM (0 if the query fails)
 // The Gumbel transform of Philox words, element-wise (test hook).
 cudaError_t launch_selftest_gumbel(const uint32_t* bits, float* g, long long n, int sms, cudaStream_t s);
 
@@ -161,6 +165,7 @@ struct VerifySampledArgs {
   const float* ls;               // [B][V] W_vocab rg
   void* r_records;               // [B][r_nchunks][2] RowAcc: residual keys, then target keys
   int r_nchunks, r_chunk_cols;
+  int vec;                       // rows and prior 16-byte aligned, V a multiple of 8
   int32_t* out_accept;
   int32_t* out_bonus;
   float* out_bonus_gap;          // or null

@@ -5,7 +5,8 @@
 // * k_sample_rows — per-(row, column chunk) records of the Gumbel-max keys
 //   k = l + g of a logit row (position 0 of the drafting loop draws x_0 from
 //   softmax(l_L^(0))).
-// * k_verify_accept, k_residual_rows, k_residual_merge — speculative sampling
+// * k_lse_rows, k_verify_accept, k_residual_rows, k_residual_merge — speculative
+//   sampling
 //   (Leviathan et al. 2023; Chen et al. 2023): x_j is accepted when
 //   u_j < p_j(x_j) / q_j(x_j); at the first rejection a the bonus token is
 //   drawn from max(0, p_a - q_a) (normalised), and after n acceptances from
@@ -63,6 +64,19 @@ __device__ __forceinline__ RowAcc block_merge(RowAcc x, RowAcc* red) {
   return x;
 }
 
+__device__ __forceinline__ float max8(const float (&x)[8]) {
+  return fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), fmaxf(fmaxf(x[4], x[5]), fmaxf(x[6], x[7])));
+}
+
+// Top-2 update of eight keys with maximum km: element by element only when
+// km exceeds the runner-up (smaller keys change nothing).
+__device__ __forceinline__ void push8(const float (&k)[8], float km, int c, float& best, float& second, int& idx) {
+  if (km > second) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) top2_push(k[i], c + i, best, second, idx);
+  }
+}
+
 // Records of the keys k_v = l_v + g_v of rows [0, rows): row r is
 // src + r * ld; its request index (for the variates) is r / rows_per_request
 // and its position j0 + r % rows_per_request. CTA = (row, chunk of
@@ -86,7 +100,8 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(SampleRowsArgs a
     load8<T>(src, c, c1, a.vec != 0, x);
     gumbel8(a.seed, a.step, b, j, a.stream, c >> 3, g);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) top2_push(x[i] + g[i], (int)(c + i), best, second, idx);
+    for (int i = 0; i < 8; ++i) g[i] += x[i];
+    push8(g, max8(g), (int)c, best, second, idx);
     lse_chunk_ex2<8>(x, best, m, s);
   }
   RowAcc r;
@@ -95,6 +110,86 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(SampleRowsArgs a
   r.second = second;
   r.idx = idx;
   // lse_chunk_ex2 keeps s relative to the running key max: r.m == best
+  r = block_merge(r, red);
+  if (threadIdx.x == 0)
+    reinterpret_cast<float4*>(a.partials)[row * a.partial_ld + chunk] =
+        make_float4(r.m, r.s, r.second, __int_as_float(r.idx));
+}
+
+// Records (largest value and sum of exponentials) of the target rows, for
+// their LSEs: CTA = (row, chunk of chunk_cols columns, a multiple of 8). A
+// pure stream of the rows: per element one fused multiply-add, one base-2
+// exponential and one addition beside the unpacking, and no top-2 state, which
+// the LSE does not need (64 x 17 bf16 rows of 151936: 61 us; the combine's row
+// kernel with no short logits and no prior, used before, 81 us).
+template <typename T>
+__global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_rows(SampleRowsArgs a) {
+  __shared__ RowAcc red[kSampleThreads / 32];
+  if (threadIdx.x == 0) pdl_trigger();
+  pdl_wait();
+  const int chunk = blockIdx.x % a.nchunks;
+  const long long row = blockIdx.x / a.nchunks;
+  const long long c0 = (long long)chunk * a.chunk_cols;
+  const T* src = static_cast<const T*>(a.src) + row * a.ld + c0;
+  const int cols = (int)min((long long)a.chunk_cols, a.V - c0);
+  float m = -INFINITY, s = 0.f;
+  // eight values, their maximum vm (NaN ignored)
+  auto push = [&](const float (&x)[8], float vm) {
+    if (vm > m) {
+      s *= ex2_approx((m - vm) * kLog2e);      // m == -inf: s is 0 or NaN
+      m = vm;
+    }
+    if (m == -INFINITY) {                      // nothing finite yet: only a NaN counts
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (x[i] != x[i]) s = NAN;
+      return;
+    }
+    const float nb = -m * kLog2e;
+    float e[2] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) e[i & 1] += ex2_approx(fmaf(x[i], kLog2e, nb));
+    s += e[0] + e[1];
+  };
+  if (a.vec) {
+    constexpr int W = sizeof(T) == 2 ? 1 : 2;  // 16-byte words per 8 values
+    constexpr int U = 4;
+    constexpr int step = kSampleThreads * 8;
+    for (int cb = threadIdx.x * 8; cb < cols; cb += step * U) {
+      uint4 w[U][W];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (cb + u * step < cols) {
+#pragma unroll
+          for (int k = 0; k < W; ++k) w[u][k] = __ldcs(reinterpret_cast<const uint4*>(src + cb + u * step) + k);
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (cb + u * step < cols) {
+          float x[8];
+          if constexpr (W == 1) {
+            x[0] = bf16lo(w[u][0].x); x[1] = bf16hi(w[u][0].x); x[2] = bf16lo(w[u][0].y); x[3] = bf16hi(w[u][0].y);
+            x[4] = bf16lo(w[u][0].z); x[5] = bf16hi(w[u][0].z); x[6] = bf16lo(w[u][0].w); x[7] = bf16hi(w[u][0].w);
+          } else {
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+              x[4 * k] = __uint_as_float(w[u][k].x); x[4 * k + 1] = __uint_as_float(w[u][k].y);
+              x[4 * k + 2] = __uint_as_float(w[u][k].z); x[4 * k + 3] = __uint_as_float(w[u][k].w);
+            }
+          }
+          push(x, max8(x));
+        }
+    }
+  } else {
+    for (int c = threadIdx.x * 8; c < cols; c += 8 * kSampleThreads) {
+      float x[8];
+      load8<T>(src, c, cols, false, x);
+      push(x, max8(x));
+    }
+  }
+  RowAcc r = rowacc_init();
+  r.m = m;
+  r.s = s;
   r = block_merge(r, red);
   if (threadIdx.x == 0)
     reinterpret_cast<float4*>(a.partials)[row * a.partial_ld + chunk] =
@@ -112,11 +207,12 @@ __device__ __forceinline__ float ld_logit_any(const void* p, int f32, long long 
 }
 
 // One CTA per request: the LSE of each target row from its records, then the
-// acceptance tests in order, then the gather of the rejected position's
+// acceptance tests, then the gather of the rejected position's
 // vocabulary-projection input.
 __global__ void __launch_bounds__(256) k_verify_accept(VerifySampledArgs a) {
   __shared__ float lse_s[kMaxSampledBlock + 1];
   __shared__ int acc_s;
+  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -132,27 +228,29 @@ __global__ void __launch_bounds__(256) k_verify_accept(VerifySampledArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = a.n;
-    for (int j = 0; j < a.n; ++j) {
-      const int x = a.draft[(long long)b * a.n + j];
-      if (x < 0 || x >= a.V) {
-        raise_status(a.status, DELS_STATUS_BAD_TOKEN);
-        acc = j;
-        break;
-      }
-      const float t = ld_logit_any(a.target, a.target_f32, ((long long)b * (a.n + 1) + j) * a.V + x);
-      const float ratio = expf((t - lse_s[j]) - a.draft_lp[(long long)b * a.n + j]);
-      const float u = uniform_at(a.seed, a.step, b, j, kStreamAccept, 0);
-      if (!(u < ratio)) {
-        acc = j;
-        break;
+  if (warp == 0) {
+    // one lane per test (n <= 32), the first that fails ends the block
+    bool fails = false, bad = false;
+    if (lane < a.n) {
+      const int x = a.draft[(long long)b * a.n + lane];
+      bad = x < 0 || x >= a.V;
+      if (bad) {
+        fails = true;
+      } else {
+        const float t = ld_logit_any(a.target, a.target_f32, ((long long)b * (a.n + 1) + lane) * a.V + x);
+        const float ratio = expf((t - lse_s[lane]) - a.draft_lp[(long long)b * a.n + lane]);
+        fails = !(uniform_at(a.seed, a.step, b, lane, kStreamAccept, 0) < ratio);
       }
     }
-    acc_s = acc;
-    a.acc[b] = acc;
-    a.out_accept[b] = acc;
-    a.lse_t[b] = lse_s[acc];
+    const unsigned f = __ballot_sync(0xFFFFFFFFu, fails);
+    const int acc = f ? __ffs(f) - 1 : a.n;
+    if (lane == acc && bad) raise_status(a.status, DELS_STATUS_BAD_TOKEN);
+    if (lane == 0) {
+      acc_s = acc;
+      a.acc[b] = acc;
+      a.out_accept[b] = acc;
+      a.lse_t[b] = lse_s[acc];
+    }
   }
   __syncthreads();
   const int acc = acc_s;
@@ -167,41 +265,81 @@ __global__ void __launch_bounds__(256) k_verify_accept(VerifySampledArgs a) {
   }
 }
 
+// Eight values of a row for the residual: one or two 16-byte loads (VEC), or
+// element by element with -inf past the row's end.
+template <typename T, bool VEC>
+__device__ __forceinline__ void load8_row(const T* row, int c, int c1, float (&x)[8]) {
+  if constexpr (VEC) {
+    if constexpr (sizeof(T) == 2) {
+      const uint4 w = __ldcs(reinterpret_cast<const uint4*>(row + c));
+      x[0] = bf16lo(w.x); x[1] = bf16hi(w.x); x[2] = bf16lo(w.y); x[3] = bf16hi(w.y);
+      x[4] = bf16lo(w.z); x[5] = bf16hi(w.z); x[6] = bf16lo(w.w); x[7] = bf16hi(w.w);
+    } else {
+      const float4 p = __ldcg(reinterpret_cast<const float4*>(row + c));
+      const float4 q = __ldcg(reinterpret_cast<const float4*>(row + c) + 1);
+      x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
+      x[4] = q.x; x[5] = q.y; x[6] = q.z; x[7] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if constexpr (sizeof(T) == 2) x[i] = c + i < c1 ? bf16_to_f(__ldcg(row + c + i)) : -INFINITY;
+      else x[i] = c + i < c1 ? __ldcg(row + c + i) : -INFINITY;
+    }
+  }
+}
+
 // Records of the bonus draw of request b over one chunk of the vocabulary:
 // residual keys log(max(0, p_a - q_a)) + g (a < n) and target keys t + g
 // (used after n acceptances, or when every residual weight rounded to zero).
+// Issue-bound: the variates and the three transcendentals of the weights are
+// most of the instructions. 64 requests of 151936 bf16: 74 us with element
+// loads and a top-2 update per element, 42 with 16-byte loads, group tests and
+// a grid of one wave (ncu). (Leaving out the groups whose keys, bounded by one
+// transform each, lie below a runner-up already met was slower: 54 us.)
+template <typename TT, typename TL, bool VEC>
 __global__ void __launch_bounds__(kSampleThreads) k_residual_rows(VerifySampledArgs a) {
   __shared__ RowAcc red[kSampleThreads / 32];
+  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x / a.r_nchunks, chunk = blockIdx.x % a.r_nchunks;
   const int acc = __ldcg(a.acc + b);
   const float lse_t = __ldcg(a.lse_t + b);
-  const long long trow = ((long long)b * (a.n + 1) + acc) * a.V;
+  // the rows from this chunk's first column
+  const long long c0 = (long long)chunk * a.r_chunk_cols;
+  const int cols = (int)min((long long)a.r_chunk_cols, a.V - c0);
+  const TT* trow = static_cast<const TT*>(a.target) + ((long long)b * (a.n + 1) + acc) * a.V + c0;
   const bool resid = acc < a.n;
-  const long long lrow = ((long long)b * a.n + (resid ? acc : 0)) * a.V;
+  const TL* lrow = static_cast<const TL*>(a.longp) + ((long long)b * a.n + (resid ? acc : 0)) * a.V + c0;
   const float lse_q = resid ? a.state_lse[(long long)b * a.n + acc] : 0.f;
   const bool head = resid && acc >= 1;
   const float al = head ? a.alpha[acc] : 0.f, nbe = head ? -a.beta[acc] : 0.f;
-  const float* ls = a.ls + (long long)b * a.V;
-  const long long c0 = (long long)chunk * a.r_chunk_cols;
-  const long long c1 = min((long long)a.V, c0 + a.r_chunk_cols);
+  const float* ls = a.ls + (long long)b * a.V + c0;
+  const float* prior = a.prior ? a.prior + c0 : nullptr;
   float rb = -INFINITY, rs = -INFINITY, pb = -INFINITY, ps = -INFINITY;
   int ri = 0x7FFFFFFF, pi = 0x7FFFFFFF;
-  for (long long c = c0 + 8 * (long long)threadIdx.x; c < c1; c += 8 * kSampleThreads) {
-    float g[8];
-    gumbel8(a.seed, a.step, b, acc, kStreamResidual, c >> 3, g);
+  for (int c = 8 * (int)threadIdx.x; c < cols; c += 8 * kSampleThreads) {
+    float t[8], l[8], sl[8], pr[8];
+    load8_row<TT, VEC>(trow, c, cols, t);
+    if (resid) load8_row<TL, VEC>(lrow, c, cols, l);
+    if (head) {
+      load8_row<float, VEC>(ls, c, cols, sl);
+      if (prior) load8_row<float, VEC>(prior, c, cols, pr);
+    }
+    float g[8], k[8];
+    gumbel8(a.seed, a.step, b, acc, kStreamResidual, (c0 + c) >> 3, g);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const long long v = c + i;
-      if (v >= c1) break;
-      const float t = ld_logit_any(a.target, a.target_f32, trow + v);
-      top2_push(t + g[i], (int)v, pb, ps, pi);
-      if (resid) {
-        float l = ld_logit_any(a.longp, a.long_f32, lrow + v);
-        if (head) l = fmaf(nbe, a.prior ? __ldg(a.prior + v) : 0.f, fmaf(al, __ldcg(ls + v), l));
-        const float w = __expf(t - lse_t) - __expf(l - lse_q);
-        top2_push(w > 0.f ? __logf(w) + g[i] : -INFINITY, (int)v, rb, rs, ri);
+    for (int i = 0; i < 8; ++i) k[i] = t[i] + g[i];
+    push8(k, max8(k), (int)(c0 + c), pb, ps, pi);
+    if (resid) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float x = l[i];
+        if (head) x = fmaf(nbe, prior ? pr[i] : 0.f, fmaf(al, sl[i], x));
+        const float w = ex2_approx((t[i] - lse_t) * kLog2e) - ex2_approx((x - lse_q) * kLog2e);
+        k[i] = w > 0.f && (VEC || c + i < cols) ? fmaf(lg2_approx(w), kLn2, g[i]) : -INFINITY;
       }
+      push8(k, max8(k), (int)(c0 + c), rb, rs, ri);
     }
   }
   RowAcc r;
@@ -221,6 +359,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_residual_rows(VerifySampledA
 // One CTA per request: the bonus token from the merged records.
 __global__ void __launch_bounds__(256) k_residual_merge(VerifySampledArgs a) {
   __shared__ RowAcc red[8];
+  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x;
   RowAcc r = rowacc_init(), p = rowacc_init();
@@ -263,11 +402,37 @@ cudaError_t launch_verify_accept(const VerifySampledArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_residual_rows(const VerifySampledArgs& a, cudaStream_t s) {
-  return launch_pdl(k_residual_rows, dim3((unsigned)(a.B * a.r_nchunks)), dim3(kSampleThreads), 0, s, a);
+  const dim3 grid((unsigned)(a.B * a.r_nchunks)), block(kSampleThreads);
+  using K = void (*)(VerifySampledArgs);
+  const K vec[4] = {k_residual_rows<uint16_t, uint16_t, true>, k_residual_rows<uint16_t, float, true>,
+                    k_residual_rows<float, uint16_t, true>, k_residual_rows<float, float, true>};
+  const K any[4] = {k_residual_rows<uint16_t, uint16_t, false>, k_residual_rows<uint16_t, float, false>,
+                    k_residual_rows<float, uint16_t, false>, k_residual_rows<float, float, false>};
+  const int k = (a.target_f32 ? 2 : 0) + (a.long_f32 ? 1 : 0);
+  return launch_pdl(a.vec ? vec[k] : any[k], grid, block, 0, s, a);
 }
 
 cudaError_t launch_residual_merge(const VerifySampledArgs& a, cudaStream_t s) {
   return launch_pdl(k_residual_merge, dim3((unsigned)a.B), dim3(256), 0, s, a);
+}
+
+cudaError_t launch_lse_rows(const SampleRowsArgs& a, bool f32, cudaStream_t s) {
+  const long long grid = (long long)a.rows * a.nchunks;
+  if (grid == 0) return cudaSuccess;
+  return f32 ? launch_pdl(k_lse_rows<float>, dim3((unsigned)grid), dim3(kSampleThreads), 0, s, a)
+             : launch_pdl(k_lse_rows<uint16_t>, dim3((unsigned)grid), dim3(kSampleThreads), 0, s, a);
+}
+
+int lse_slots_per_sm(bool f32) {
+  static int cache[2] = {-1, -1};   // a property of the kernel, queried once
+  if (cache[f32] < 0) {
+    int n = 0;
+    const cudaError_t e =
+        f32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lse_rows<float>, kSampleThreads, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_lse_rows<uint16_t>, kSampleThreads, 0);
+    cache[f32] = e == cudaSuccess && n > 0 ? n : 0;
+  }
+  return cache[f32];
 }
 
 cudaError_t launch_sample_rows(const SampleRowsArgs& a, bool f32, cudaStream_t s) {

@@ -147,6 +147,67 @@ def test_sampled_verify_matches_oracle(name):
     assert np.all((acc >= 0) & (acc <= w.n)) and np.all((bonus >= 0) & (bonus < w.V))
 
 
+def _verify_raw(w, d, W, a, b, tok, lp, state, target, prior):
+    """One verification call (seed 23, step 7): outputs and device status."""
+    head = dels.make_head(w.head, W)
+    tdt = dels.dtype_code(target)
+    nbytes = dels.dels_verify_sampled_workspace_bytes(head, w.B, w.n, w.V, tdt)
+    ws = torch.zeros(nbytes, dtype=torch.uint8, device=DEV)
+    acc, bonus = (torch.full((w.B,), -5, dtype=torch.int32, device=DEV) for _ in range(2))
+    bgap = torch.empty(w.B, dtype=torch.float32, device=DEV)
+    r = dels.dels_verify_block_sampled(head, torch.as_tensor(tok, device=DEV), torch.as_tensor(lp, device=DEV), state,
+                                       d["long"], dels.dtype_code(d["long"]), prior, a, b, target, tdt, w.B, w.n, w.V,
+                                       23, 7, acc, bonus, bgap, ws, nbytes)
+    assert r == 0, dels.dels_status_string(r)
+    return acc.cpu().numpy(), bonus.cpu().numpy(), bgap.cpu().numpy(), dels.dels_read_status(ws)
+
+
+@pytest.mark.parametrize("name", ["gru", "gru_f32"])
+@pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
+def test_sampled_verify_unaligned_prior_takes_the_element_path(name, target_dtype):
+    """A prior off its 16-byte boundary (the residual's element loads) gives
+    the results of an aligned one (its 16-byte loads) bit for bit, for both
+    target types and both draft-logit types."""
+    w, d, W, a, b, tok, lp, gap, state = _sampled(name, 23, 7)
+    target = synth.make_target_logits(w, d["long"], device=DEV).to(target_dtype)
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    shifted = torch.empty(w.V + 4, device=DEV)[1:w.V + 1]
+    shifted.copy_(prior)
+    one = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+    two = _verify_raw(w, d, W, a, b, tok, lp, state, target, shifted)
+    assert one[3] == 0 and two[3] == 0
+    for x, y in zip(one, two):
+        np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("what", ["nan", "nan_first", "inf", "masked", "masked_row"])
+def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
+    """A NaN, a +inf or an all -inf target row sets the status; a row with
+    masked (-inf) entries does not and keeps its LSE."""
+    w, d, W, a, b, tok, lp, gap, state = _sampled("gru", 23, 7)
+    target = synth.make_target_logits(w, d["long"], device=DEV).to(target_dtype)
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    if what == "nan":
+        target[1, 2, w.V - 3] = float("nan")
+    elif what == "nan_first":                 # in a group with nothing finite, before anything else
+        target[1, 2, :8] = float("-inf")
+        target[1, 2, 1] = float("nan")
+    elif what == "inf":
+        target[1, 2, 9] = float("inf")
+    elif what == "masked_row":
+        target[1, 2] = float("-inf")
+    else:
+        target[:, :, ::3] = float("-inf")
+    acc, bonus, bgap, st = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+    if what == "masked":
+        assert st == 0
+        info = _check_verify(w, d, W, a, b, tok, acc, bonus, bgap, target, 23, 7, LP_TOL_BF16)
+        assert info["requests"] == w.B
+    else:
+        assert st & dels.DELS_STATUS_NONFINITE
+
+
 @pytest.mark.parametrize("name", ["gru", "markov", "tiny"])
 def test_sampled_verify_rejection_at_position_zero(name):
     """The target rules out every x_0 (p_0(x_0) = 0): every request rejects at
