@@ -430,7 +430,7 @@ struct DraftLayout {
   // GRU
   size_t eg = 0, h = 0, hb = 0, gpart = 0, r = 0;
   int gru_s0 = 0, gru_s1 = 0;
-  int rank_grid = 0, hh_splits = 0;          // input-table path: grouped rank + recurrent product
+  int rank_grid = 0, hh_splits = 0, ih_splits = 0;   // grouped rank + recurrent product; input product alone
   // MLP
   size_t u = 0, mpart = 0, h1 = 0, h2 = 0;
   int mlp_s1 = 0, mlp_s2 = 0;
@@ -466,12 +466,12 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
         L.gru_s1 = 1;
         L.rank_grid = (R + kRankTile - 1) / kRankTile * kRankSplits;
         L.hh_splits = splits_for(3 * H, kHhTile, H, std::max(1, sms - L.rank_grid));
+        L.ih_splits = splits_for(3 * H, 128, D, sms);
       } else {
         L.gru_s0 = 1;
         L.gru_s1 = 1;
       }
-      L.gpart = c.take((size_t)std::max(L.gru_s0 + L.gru_s1, L.hh_splits) * B * 3 * H * 4);
-
+      L.gpart = c.take((size_t)std::max(L.gru_s0 + L.gru_s1, L.ih_splits + L.hh_splits) * B * 3 * H * 4);
       L.r = c.take((size_t)B * R * es);
       break;
     }
@@ -524,6 +524,40 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
   L.total = c.off;
   L.ok = true;
   return L;
+}
+
+// The GRU's two products of the new state h_j (bf16 rows hb), one grouped
+// launch: r_j = SiLU(W_rank h_j), its K splits reduced inside a cluster (one
+// cluster per output tile, no partials in memory; its SiLU needs the whole
+// sum), and beside it the split partials of W_hh h_j (hh_part) for the next
+// position's gates.
+bool plan_rank_hh(Gemm& gr, Gemm& gh, const dels_local_head* hd, const DraftLayout& L, int B, const uint16_t* hb,
+                  uint16_t* r, float* hh_part, int* status) {
+  const int H = hd->d_hidden, R = hd->d_rank, sms = L.sms;
+  if (!plan_store(gr, B, R, hb, hd->w[2], H, nullptr, nullptr, 0, kRankTile, kRankSplits, 0, ACT_SILU, nullptr, r, R,
+                  status, sms) ||
+      !plan_store(gh, B, 3 * H, hb, hd->w[1], H, nullptr, nullptr, 0, kHhTile, L.hh_splits, 0, ACT_NONE, hh_part,
+                  nullptr, 0, status, sms))
+    return false;
+  const int ck = gr.a.total_splits;
+  if (ck > 1) {
+    gr.a.cluster_k = ck;
+    gr.grid = gr.a.num_o_tiles * ck;
+    const int per = (gr.a.seg_chunks[0] + ck - 1) / ck;
+    gr.a.stages = std::max(2, std::min(gr.a.stages, per));
+    gr.smem = tc_gemm_smem_bytes(gr.a);
+  }
+  // both products fit one wave next to each other; whole clusters only
+  gh.grid = std::min(gh.grid, std::max(ck, sms - gr.grid));
+  gh.grid = std::max(ck, gh.grid / ck * ck);
+  return true;
+}
+
+// gh: null when no position follows.
+cudaError_t run_rank_hh(const Gemm& gr, const Gemm* gh, cudaStream_t s) {
+  TcGemmGroup hh{};
+  if (gh) hh = TcGemmGroup{&gh->a, &gh->mA0, &gh->mB0, gh->grid};
+  return launch_tc_gemm(gr.a, &gr.mA0, &gr.mB0, &gr.mA1, &gr.mB1, &gr.mL, gr.grid, gr.smem, s, gh ? &hh : nullptr);
 }
 
 int validate_head(const dels_local_head* h, int n) {
@@ -1417,27 +1451,10 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
                            &mb.smp);
         if (r != DELS_OK) return r;
         Gemm gr, gh, gv;
-        if (!plan_store(gr, B, R, hb, head->w[2], H, nullptr, nullptr, 0, kRankTile, kRankSplits, 0, ACT_SILU,
-                        nullptr, static_cast<uint16_t*>(rr), R, status, sms) ||
-            !plan_store(gh, B, 3 * H, hb, head->w[1], H, nullptr, nullptr, 0, kHhTile, L.hh_splits, 0, ACT_NONE,
-                        gpart, nullptr, 0, status, sms) ||
+        if (!plan_rank_hh(gr, gh, head, L, B, hb, static_cast<uint16_t*>(rr), gpart, status) ||
             !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
                           partials, L.partial_ld, status, sms, true))
           return DELS_ERR_CUDA;
-        // The rank product's K splits reduce inside a cluster (one cluster per
-        // output tile, no partials in HBM); its SiLU needs the whole sum.
-        const int ck = gr.a.total_splits;
-        if (ck > 1) {
-          gr.a.cluster_k = ck;
-          gr.grid = gr.a.num_o_tiles * ck;
-          const int per = (gr.a.seg_chunks[0] + ck - 1) / ck;
-          gr.a.stages = std::max(2, std::min(gr.a.stages, per));
-          gr.smem = tc_gemm_smem_bytes(gr.a);
-        }
-        // both products fit one wave next to each other; whole clusters only
-        gh.grid = std::min(gh.grid, std::max(ck, sms - gr.grid));
-        gh.grid = std::max(ck, gh.grid / ck * ck);
-        const TcGemmGroup hh{&gh.a, &gh.mA0, &gh.mB0, gh.grid};
         GatesTableArgs ga{};
         ga.partials = partials;
         ga.partial_ld = L.partial_ld;
@@ -1459,9 +1476,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           ga.jprev = j - 1;
           ga.S = j == 1 ? 0 : gh.a.total_splits;
           { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates_table(ga, s)); }
-          { PROF(DELS_KCLASS_HEAD_GEMM);
-            DELS_CUDA(launch_tc_gemm(gr.a, &gr.mA0, &gr.mB0, &gr.mA1, &gr.mB1, &gr.mL, gr.grid, gr.smem, s,
-                                     j + 1 < n ? &hh : nullptr)); }
+          { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rank_hh(gr, j + 1 < n ? &gh : nullptr, s)); }
           gv.a.j = j;
           gv.a.sample = sm.on;
           gv.a.seed = sm.seed;
@@ -1486,20 +1501,25 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       mb.zero_len = 0;
       if (r != DELS_OK || n == 1) return r;
       if (bf) {
-        Gemm gg, gr, gv;
-        if (!plan_store(gg, B, 3 * H, eg, head->w[0], D, hb, head->w[1], H, 128, L.gru_s0, L.gru_s1, ACT_NONE,
-                        gpart, nullptr, 0, status, sms))
-          return DELS_ERR_CUDA;
-        if (!plan_store(gr, B, R, hb, head->w[2], H, nullptr, nullptr, 0, 32, 1, 0, ACT_SILU, nullptr,
-                        static_cast<uint16_t*>(rr), R, status, sms))
-          return DELS_ERR_CUDA;
-        if (!plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
+        // Per position: the merge gathers e = E[x_{j-1}]; the input product
+        // W_ih e alone waits for it (all SMs); gates; then r_j beside the
+        // recurrent product of the next position, as on the table path;
+        // vocabulary. (The recurrent product used to sit beside the input
+        // product and the rank product ran on 8 CTAs: 27 requests, V 50008,
+        // 43 -> 38 us per position.)
+        Gemm gi, gr, gh, gv;
+        float* hh_part = gpart + (size_t)L.ih_splits * B * 3 * H;
+        if (!plan_store(gi, B, 3 * H, eg, head->w[0], D, nullptr, nullptr, 0, 128, L.ih_splits, 0, ACT_NONE, gpart,
+                        nullptr, 0, status, sms) ||
+            !plan_rank_hh(gr, gh, head, L, B, hb, static_cast<uint16_t*>(rr), hh_part, status) ||
+            !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
                           partials, L.partial_ld, status, sms, true))
           return DELS_ERR_CUDA;
         for (int j = 1; j < n; ++j) {
-          { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run(gg, s)); }
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, gg.a.seg_splits[0], gg.a.seg_splits[1], B, H, h, hb, s)); }
-          { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run(gr, s)); }
+          { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run(gi, s)); }
+          { PROF(DELS_KCLASS_HEAD_MISC);
+            DELS_CUDA(launch_gru_gates(gpart, gi.a.total_splits, hh_part, j == 1 ? 0 : gh.a.total_splits, B, H, h, hb, s)); }
+          { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rank_hh(gr, j + 1 < n ? &gh : nullptr, s)); }
           gv.a.j = j;
           gv.a.sample = sm.on;
           gv.a.seed = sm.seed;
@@ -1525,7 +1545,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         rank.j[0] = GemvF32Job{h, Wr, feat, H, H};
         for (int j = 1; j < n; ++j) {
           DELS_CUDA(gemv_f32(gates, 2, 3 * H, ACT_NONE));
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, 1, 1, B, H, h, hb, s)); }
+          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, 1, gpart + (size_t)B * 3 * H, 1, B, H, h, hb, s)); }
           DELS_CUDA(gemv_f32(rank, 1, R, ACT_SILU));
           DELS_CUDA(vocab_f32(feat, R, j));
           MergeArgs m = mb;

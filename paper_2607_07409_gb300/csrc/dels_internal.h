@@ -305,8 +305,8 @@ cudaError_t launch_prod_vocab(const ProdVocabArgs& P, const CUtensorMap* maps, i
                               cudaStream_t s);
 
 // ---- small head kernels -------------------------------------------------------
-cudaError_t launch_gru_gates(const float* part, int S0, int S1, int B, int H, float* h, uint16_t* h_bf16,
-                             cudaStream_t s);
+cudaError_t launch_gru_gates(const float* gi, int Si, const float* gh, int Sh, int B, int H, float* h,
+                             uint16_t* h_bf16, cudaStream_t s);
 // GRU step with a precomputed input table G = E W_ih^T [V, 3H] (f32), fused
 // with the merge of the previous position: x = the merged argmax of request
 // b's `count` records [B][partial_ld] (written to tokens/lp/gap at column

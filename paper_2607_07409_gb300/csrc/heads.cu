@@ -15,11 +15,31 @@ namespace {
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + __expf(-x)); }
 
 // GRU gates (PyTorch bias-free form; gate rows r, z, n):
-//   gi = sum of the S0 input-product partials, gh = sum of the S1 recurrent ones
+//   gi = sum of the Si input-product partials, gh = sum of the Sh recurrent
+//   ones ([S][B][3H] each; Sh = 0 at the step from h = 0)
 //   r = sigmoid(gi_r + gh_r), z = sigmoid(gi_z + gh_z)
 //   c = tanh(gi_n + r * gh_n), h' = (1 - z) * c + z * h
-__global__ void k_gru_gates(const float* __restrict__ part, int S0, int S1, int B, int H, float* __restrict__ h,
-                            uint16_t* __restrict__ h_bf16) {
+// A thread keeps the loads of four splits in flight, added in split order.
+__device__ __forceinline__ void sum_gates(const float* p, int S, long long stride, int H, float& r, float& z,
+                                          float& n) {
+  r = z = n = 0.f;
+  for (int s0 = 0; s0 < S; s0 += 4) {
+    float v[4][3];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int g = 0; g < 3; ++g) v[k][g] = s0 + k < S ? __ldcg(p + (s0 + k) * stride + g * H) : 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      r += v[k][0];
+      z += v[k][1];
+      n += v[k][2];
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) k_gru_gates(const float* gi, int Si, const float* gh, int Sh, int B, int H,
+                                                   float* __restrict__ h, uint16_t* __restrict__ h_bf16) {
   if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const long long total = (long long)B * H;
@@ -28,15 +48,9 @@ __global__ void k_gru_gates(const float* __restrict__ part, int S0, int S1, int 
        e += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(e / H), i = (int)(e % H);
     const long long base = (long long)b * 3 * H + i;
-    float gir = 0.f, giz = 0.f, gin = 0.f, ghr = 0.f, ghz = 0.f, ghn = 0.f;
-    for (int s = 0; s < S0; ++s) {
-      const float* p = part + s * split_stride + base;
-      gir += p[0]; giz += p[H]; gin += p[2 * H];
-    }
-    for (int s = S0; s < S0 + S1; ++s) {
-      const float* p = part + s * split_stride + base;
-      ghr += p[0]; ghz += p[H]; ghn += p[2 * H];
-    }
+    float gir, giz, gin, ghr, ghz, ghn;
+    sum_gates(gh + base, Sh, split_stride, H, ghr, ghz, ghn);
+    sum_gates(gi + base, Si, split_stride, H, gir, giz, gin);
     const float r = sigmoidf_(gir + ghr);
     const float z = sigmoidf_(giz + ghz);
     const float c = tanhf(gin + r * ghn);
@@ -483,9 +497,10 @@ inline int grid_for(long long total, int threads) {
 
 }  // namespace
 
-cudaError_t launch_gru_gates(const float* part, int S0, int S1, int B, int H, float* h, uint16_t* h_bf16,
-                             cudaStream_t s) {
-  return launch_pdl(k_gru_gates, dim3(grid_for((long long)B * H, 256)), dim3(256), 0, s, part, S0, S1, B, H, h, h_bf16);
+cudaError_t launch_gru_gates(const float* gi, int Si, const float* gh, int Sh, int B, int H, float* h,
+                             uint16_t* h_bf16, cudaStream_t s) {
+  return launch_pdl(k_gru_gates, dim3(grid_for((long long)B * H, 256)), dim3(256), 0, s, gi, Si, gh, Sh, B, H, h,
+                    h_bf16);
 }
 
 cudaError_t launch_gru_gates_table(const GatesTableArgs& a, cudaStream_t s) {
