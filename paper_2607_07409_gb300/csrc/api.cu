@@ -767,6 +767,7 @@ struct PriorWs {
   unsigned long long* partials; // [kPriorMaxPartials] (sum of the counts)
   unsigned* ticket;
   unsigned long long* total;
+  unsigned* halves;             // [slices][members][slice / 2] (half-word slices)
   // hot ids on chip (when the plan uses them)
   unsigned* hist;               // [kPriorHistBuckets]
   unsigned* cta_total;          // [select CTAs]
@@ -790,6 +791,10 @@ PriorWs prior_ws_layout(void* ws, int V, const PriorPlan& p) {
   w.ticket = at<unsigned>(ws, off);
   w.total = at<unsigned long long>(ws, off + 8);
   off = round_up(off + 16, 256);
+  if (p.halves > 0) {
+    w.halves = at<unsigned>(ws, off);
+    off = round_up(off + (size_t)p.halves * p.members * (p.slice / 2) * 4, 256);
+  }
   if (p.use_hot) {
     w.hist = at<unsigned>(ws, off);
     off = round_up(off + (size_t)kPriorHistBuckets * 4, 256);
@@ -834,6 +839,22 @@ int prior_count_impl(const int32_t* tokens, const uint8_t* loss_mask, long long 
                      unsigned long long* tally, int* status, const PriorPlan& p, const PriorWs& w, int sms,
                      cudaStream_t s) {
   if (N == 0) return DELS_OK;
+  if (p.halves > 0) {
+    PriorHalvesArgs h{};
+    h.V = V;
+    h.slices = p.halves;
+    h.slice = p.slice;
+    h.members = p.members;
+    h.partials = w.halves;
+    h.counts = counts;
+    h.tally = tally;
+    h.status = status;
+    for (long long b = 0; b < N; b += kPriorChunk) {
+      h.range = prior_range(tokens, loss_mask, b, std::min(kPriorChunk, N - b));
+      if (launch_prior_halves(h, p.slice_smem, s) != cudaSuccess) return DELS_ERR_CUDA;
+    }
+    return DELS_OK;
+  }
   PriorSliceArgs sa{};
   sa.V = V;
   sa.slices = p.slices;

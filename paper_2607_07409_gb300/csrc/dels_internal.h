@@ -429,6 +429,7 @@ bool encode_tmap_3d(CUtensorMap* m, const void* base, CUtensorMapDataType dt, in
 // ---- unigram prior estimation (Appendix A) -----------------------------------
 constexpr int kPriorMaxPartials = 1024;            // CTAs of the two-level count sum
 constexpr int kPriorHistBuckets = 3776;            // count buckets of the hot-set choice
+constexpr long long kPriorHalvesMinN = 1ll << 23;  // shorter ranges: 32-bit slice histograms
 constexpr long long kPriorHotMinN = 1ll << 24;     // shorter ranges: slice histograms only
 constexpr long long kPriorChunk = 1ll << 36;       // positions per launch (per-thread tallies stay < 2^32)
 
@@ -441,6 +442,17 @@ struct PriorRange {
   long long n;
   long long head;
   long long nvec;
+};
+
+struct PriorHalvesArgs {
+  PriorRange range;
+  int V;
+  int slices, slice;                // P slices of `slice` ids (a multiple of 8)
+  int members;                      // CTAs per slice
+  unsigned* partials;               // [slices][members][slice / 2] words of two bins
+  unsigned long long* counts;       // [V], accumulated
+  unsigned long long* tally;        // [2] or null
+  int* status;
 };
 
 struct PriorSliceArgs {
@@ -497,6 +509,8 @@ struct PriorLogArgs {
 // How a count call runs for (V, N) on this device.
 struct PriorPlan {
   bool ok;
+  int halves;                 // half-word slices (0: the schemes below), of `slice` ids
+  int members;                // CTAs per half-word slice
   int slices, slice;          // slice histograms: P slices of `slice` ids
   size_t slice_smem;
   bool use_hot;               // hot ids on chip
@@ -508,6 +522,7 @@ struct PriorPlan {
 };
 
 PriorPlan plan_prior(int V, long long N, int sms);
+cudaError_t launch_prior_halves(const PriorHalvesArgs& a, size_t smem, cudaStream_t s);
 cudaError_t launch_prior_slices(const PriorSliceArgs& a, size_t smem, int max_members, int sms, cudaStream_t s);
 cudaError_t launch_prior_select(const PriorSelectArgs& a, int ctas, cudaStream_t s);
 cudaError_t launch_prior_hot(const PriorHotArgs& a, size_t smem, cudaStream_t s);

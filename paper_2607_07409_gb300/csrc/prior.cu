@@ -10,11 +10,17 @@
 // kept per CTA in shared memory, which holds 227 KB: about 57K 32-bit bins,
 // a third of a 152K vocabulary. Two pieces:
 //
-// * Slice histograms (k_prior_slices): the vocabulary is cut into P slices
-//   that each fit; P groups of CTAs read the same positions, each group
-//   counting one slice. Used alone when P = 1 (small vocabularies) or when
-//   the range is short.
-// * Hot ids on chip (large vocabularies, long corpora): a short prefix is
+// * Half-word slices (k_prior_halves): the vocabulary is cut into P slices of
+//   16-bit bins, two to a word, that each fit (115K ids a slice); P groups of
+//   CTAs read the same positions (the second reading hits L2), each counting
+//   one slice, and the bins of a group's CTAs are summed at the end
+//   (k_prior_halves_reduce). A bin that reaches 2^15 hands 2^15 to the global
+//   count, so it never carries into its neighbour. Used over long ranges for
+//   vocabularies that two slices cover.
+// * Slice histograms (k_prior_slices): the same with 32-bit bins, added to
+//   the counts by atomics: short ranges, small vocabularies, and the prefix
+//   of the hot scheme.
+// * Hot ids on chip (more than two slices, long corpora): a short prefix is
 //   counted exactly by the slices; the ids with the largest counts so far
 //   become the hot set, at most K of them (k_prior_hist, k_prior_mark,
 //   k_prior_place: a count histogram, presence bits, slot numbers). A remap
@@ -28,6 +34,7 @@
 //
 // The log step is a map over V after a two-level sum of the counts.
 #include <algorithm>
+#include <type_traits>
 
 #include "dels_device.cuh"
 
@@ -42,7 +49,6 @@ constexpr int kWarpSpan = 512;               // positions a warp takes per vecto
 constexpr int kSelectBuckets = kPriorHistBuckets;   // count buckets of the hot-set choice (32 x 118)
 constexpr int kIdsPerWord = 15;              // remap word: 15 presence bits + a 17-bit slot number
 constexpr unsigned kFlush = 0x8000u;         // a 16-bit hot bin hands this to the global count
-constexpr int kLogTable = 256;               // log(c + lambda) tabulated for counts below this
 
 struct Tally {   // per thread; a thread sees far fewer than 2^32 positions per launch
   unsigned in = 0, out = 0;
@@ -119,6 +125,182 @@ __device__ __forceinline__ void visit(const PriorRange& r, long long worker, lon
   }
 }
 
+// One position of a half-word slice: adds `one` (1 or 2^16, by the bin's half)
+// to the word of id's bin if its mask byte is set and id lies in [lo, lo + nb);
+// returns the word before the add, or 0 if there was none. Written as
+// predicated instructions: as C++ conditionals the compiler branched around
+// each add (20.7 instructions per position instead of 19.8).
+template <int Q>
+__device__ __forceinline__ unsigned count_half(unsigned id, uint32_t mk, unsigned lo, unsigned nb, unsigned base2,
+                                               unsigned& one) {
+  unsigned old;
+  asm volatile(
+      "{\n\t.reg .pred p, h;\n\t.reg .u32 t, v;\n\t"
+      "and.b32 t, %3, %4;\n\t"
+      "setp.ne.u32 p, t, 0;\n\t"
+      "sub.u32 t, %2, %5;\n\t"
+      "setp.lt.and.u32 p, t, %6, p;\n\t"
+      "mad.lo.u32 v, %2, 2, %7;\n\t"
+      "and.b32 t, v, 2;\n\t"
+      "setp.ne.u32 h, t, 0;\n\t"
+      "selp.u32 %1, 65536, 1, h;\n\t"
+      "and.b32 v, v, -4;\n\t"
+      "mov.u32 %0, 0;\n\t"
+      "@p atom.shared.add.u32 %0, [v], %1;\n\t}"
+      : "=&r"(old), "=&r"(one)
+      : "r"(id), "r"(mk), "n"(0xFFu << (8 * Q)), "r"(lo), "r"(nb), "r"(base2)
+      : "memory");
+  return old;
+}
+
+// Half-word slices. CTA b counts slice b % P over the positions its group
+// member index b / P takes. Issue-bound, about 20 instructions per position and
+// group: the bin's word and half follow from the id directly, where the hot
+// scheme looks its slot up (about 43 per position). Out-of-range ids are
+// tallied by one group for each vector step, so that the groups do equal work;
+// the positions counted are the sum of the bins, which go to the partials.
+__global__ void __launch_bounds__(kThreads, 1) k_prior_halves(PriorHalvesArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned* words = reinterpret_cast<unsigned*>(smem_raw);
+  __shared__ unsigned long long red[2 * kWarps];
+  if (threadIdx.x == 0) pdl_trigger();
+  const int P = a.slices;   // 1 or 2
+  const int g = blockIdx.x % P;
+  const int member = blockIdx.x / P, members = gridDim.x / P;
+  const unsigned lo = (unsigned)(g * a.slice);
+  const unsigned nb = (unsigned)max(0, min(a.slice, a.V - (int)lo));
+  const int kw = a.slice / 2;
+  for (int w = threadIdx.x; w < kw / 4; w += kThreads) reinterpret_cast<uint4*>(words)[w] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  pdl_wait();
+  const int lane = threadIdx.x & 31;
+  Tally t;
+  // bin u has reached 2^15: its word goes back by that much
+  auto hand_off = [&](unsigned u) {
+    atomicSub(words + (u >> 1), (u & 1u) ? 0x80000000u : 0x8000u);
+    atomicAdd(a.counts + lo + u, 1ull << 15);
+    t.in += 1u << 15;
+  };
+  const PriorRange& r = a.range;
+  const long long nworkers = (long long)members * kWarps;
+  const long long steps = r.nvec / kWarpSpan;
+  const int4* tv = reinterpret_cast<const int4*>(r.tokens + r.head);
+  const uint32_t* mv = reinterpret_cast<const uint32_t*>(r.mask + r.head);
+  // Four positions at a time: the adds go out together, then one test for
+  // their hand-offs. (A bin has room for 2^15 more adds between reaching 2^15
+  // and the subtraction, eight from every quad of the CTA's threads.)
+  const unsigned base2 = smem_u32(words) - 2u * lo;   // byte address of bin u's half word: 2 id + base2
+  auto quad = [&](const int4& tk, uint32_t mk, auto tally) {
+    unsigned old[4];
+    unsigned flips = 0;   // bit 15 of a bin changes only when it reaches 2^15
+    unsigned one[4];
+    old[0] = count_half<0>((unsigned)tk.x, mk, lo, nb, base2, one[0]);
+    old[1] = count_half<1>((unsigned)tk.y, mk, lo, nb, base2, one[1]);
+    old[2] = count_half<2>((unsigned)tk.z, mk, lo, nb, base2, one[2]);
+    old[3] = count_half<3>((unsigned)tk.w, mk, lo, nb, base2, one[3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      flips |= old[q] ^ (old[q] + one[q]);
+      if constexpr (decltype(tally)::value)
+        t.out += (mk & (0xFFu << (8 * q))) != 0u && (unsigned)int4_at(tk, q) >= (unsigned)a.V ? 1u : 0u;
+    }
+    if (flips & 0x80008000u) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if ((old[q] ^ (old[q] + one[q])) & 0x80008000u) hand_off((unsigned)int4_at(tk, q) - lo);
+      }
+    }
+  };
+  for (long long st = (long long)member * kWarps + (threadIdx.x >> 5); st < steps; st += nworkers) {
+    const long long w0 = st * (kWarpSpan / 4) + lane;   // units of 4 positions
+    int4 tk[4];
+    uint32_t mk[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tk[k] = __ldcg(tv + w0 + 32 * k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mk[k] = __ldcg(mv + w0 + 32 * k);
+    if (((int)st & (P - 1)) == g) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) quad(tk[k], mk[k], std::true_type{});
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) quad(tk[k], mk[k], std::false_type{});
+    }
+  }
+  const long long rest = r.n - r.nvec;
+  for (long long j = ((long long)member * kWarps + (threadIdx.x >> 5)) * 32 + lane; j < rest; j += nworkers * 32) {
+    const long long i = j < r.head ? j : j + r.nvec;
+    const int id = r.tokens[i];
+    if (!r.mask[i]) continue;
+    if (g == 0 && (unsigned)id >= (unsigned)a.V) ++t.out;
+    const unsigned u = (unsigned)id - lo;
+    if (u < nb) {
+      const unsigned one = (u & 1u) ? 0x10000u : 1u;
+      const unsigned old = atomicAdd(words + (u >> 1), one);
+      if ((old ^ (old + one)) & 0x80008000u) hand_off(u);
+    }
+  }
+  __syncthreads();
+  uint4* out = reinterpret_cast<uint4*>(a.partials + ((long long)g * members + member) * kw);
+  for (int w = threadIdx.x; w < kw / 4; w += kThreads) out[w] = reinterpret_cast<const uint4*>(words)[w];
+  flush_tally(t, a.tally, a.status, red);
+}
+
+// counts[v] += the sum over a group's members of bin v: a thread takes four
+// words (eight ids) of every eighth member, the eight sums meet in shared
+// memory, and each thread adds one id's total.
+__global__ void __launch_bounds__(256) k_prior_halves_reduce(PriorHalvesArgs a) {
+  __shared__ __align__(8) unsigned sums[8][32][9];
+  if (threadIdx.x == 0) pdl_trigger();
+  pdl_wait();
+  const int kw4 = a.slice / 8;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int w4 = blockIdx.x * 32 + x;
+  const uint4* src = reinterpret_cast<const uint4*>(a.partials) + (long long)blockIdx.y * a.members * kw4;
+  unsigned s[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) s[i] = 0u;
+  if (w4 < kw4) {
+    constexpr int U = 5;
+    for (int m0 = y; m0 < a.members; m0 += 8 * U) {
+      uint4 v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        v[k] = m0 + 8 * k < a.members ? __ldcg(src + (long long)(m0 + 8 * k) * kw4 + w4) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        s[0] += v[k].x & 0xFFFFu; s[1] += v[k].x >> 16;
+        s[2] += v[k].y & 0xFFFFu; s[3] += v[k].y >> 16;
+        s[4] += v[k].z & 0xFFFFu; s[5] += v[k].z >> 16;
+        s[6] += v[k].w & 0xFFFFu; s[7] += v[k].w >> 16;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sums[y][x][i] = s[i];
+  __syncthreads();
+  // thread: id (threadIdx.x) of the block's 256
+  const int xi = threadIdx.x >> 3, i = threadIdx.x & 7;
+  unsigned total = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) total += sums[k][xi][i];
+  const int u = blockIdx.x * 256 + threadIdx.x;
+  const long long v = (long long)blockIdx.y * a.slice + u;
+  if (u < a.slice && v < a.V && total) a.counts[v] += total;
+  if (a.tally) {
+    const unsigned long long in = warp_sum_u64(total);
+    __syncthreads();
+    unsigned long long* part = reinterpret_cast<unsigned long long*>(sums);
+    if (x == 0) part[y] = in;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned long long all = 0;
+      for (int k = 0; k < 8; ++k) all += part[k];
+      if (all) atomicAdd(a.tally, all);
+    }
+  }
+}
+
 // Slice histograms. CTA b counts slice b % P of the vocabulary over the
 // positions its group member index b / P takes; the bins are added to the
 // 64-bit counts at the end (coalesced atomics). Group 0 keeps the tallies.
@@ -131,6 +313,7 @@ __global__ void __launch_bounds__(kThreads) k_prior_slices(PriorSliceArgs a) {
   const long long member = blockIdx.x / P, members = gridDim.x / P;
   const int lo = g * a.slice;
   const int nb = max(0, min(a.slice, a.V - lo));
+  if (threadIdx.x == 0) pdl_trigger();
   for (int b = threadIdx.x; b < nb; b += kThreads) bins[b] = 0u;
   __syncthreads();
   pdl_wait();
@@ -491,23 +674,47 @@ __global__ void __launch_bounds__(kMapThreads) k_prior_total(PriorLogArgs a) {
   *a.ticket = 0u;
 }
 
+// ln x of a positive, normal double by table lookup and a short series (Tang,
+// "Table-driven implementation of the logarithm function in IEEE
+// floating-point arithmetic", 1990): x = 2^e m, c the middle of the 1/128-wide
+// interval that holds m, r = m / c - 1 (|r| <= 2^-8), ln x = e ln 2 + ln c +
+// ln(1 + r); the series stops at r^4, an error below |r|^5 / 5 = 2e-13.
+// Float64 units are few here (two operations per cycle and SM): this is about
+// a quarter of log()'s operations.
+__device__ __forceinline__ double log_table(double x, const double2* tab) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) - 1023;
+  const double m = __hiloint2double((hi & 0x000FFFFF) | 0x3FF00000, __double2loint(x));
+  const double2 t = tab[(hi >> 13) & 127];     // (1 / c, ln c)
+  const double r = fma(m, t.x, -1.0);
+  double p = fma(r, -0.25, 1.0 / 3.0);
+  p = fma(r, p, -0.5);
+  p = fma(r * r, p, r);
+  return fma((double)e, 0.693147180559945309417, t.y) + p;
+}
+
 // l_P(v) = log(c(v) + lambda) - log(sum_u c(u) + V lambda), in float64,
-// stored as float32; log(c + lambda) of the small counts (most ids) comes
-// from a per-CTA table. Optionally copies the counts and the tally out (the
+// stored as float32. Optionally copies the counts and the tally out (the
 // one-call estimate keeps both in its workspace).
-__global__ void __launch_bounds__(kMapThreads) k_prior_log(PriorLogArgs a) {
-  __shared__ double tab[kLogTable];
+__global__ void __launch_bounds__(kThreads) k_prior_log(PriorLogArgs a) {
+  __shared__ double2 tab[128];
   __shared__ double log_s_sh;
   const double lam = a.lambda;
-  for (int i = threadIdx.x; i < kLogTable; i += kMapThreads) tab[i] = log((double)i + lam);
+  if (threadIdx.x == 0) pdl_trigger();
+  if (threadIdx.x < 128) {
+    const double c = 1.0 + ((double)threadIdx.x + 0.5) / 128.0;
+    tab[threadIdx.x] = make_double2(1.0 / c, log(c));
+  }
   pdl_wait();
   if (threadIdx.x == 0) log_s_sh = log((double)__ldcg(a.total) + (double)a.V * lam);
   __syncthreads();
   const double log_s = log_s_sh;
-  const long long stride = (long long)gridDim.x * kMapThreads;
-  for (long long v = (long long)blockIdx.x * kMapThreads + threadIdx.x; v < a.V; v += stride) {
+  const long long stride = (long long)gridDim.x * kThreads;
+  for (long long v = (long long)blockIdx.x * kThreads + threadIdx.x; v < a.V; v += stride) {
     const unsigned long long c = __ldcg(a.counts + v);
-    const double lc = c < (unsigned long long)kLogTable ? tab[c] : log((double)c + lam);
+    const double x = (double)c + lam;
+    // lambda may be any positive float64, denormal or large
+    const double lc = x >= 1e-300 && x <= 1e300 ? log_table(x, tab) : log(x);
     a.out[v] = (float)(lc - log_s);
     if (a.counts_out) a.counts_out[v] = c;
   }
@@ -533,6 +740,21 @@ PriorPlan plan_prior(int V, long long N, int sms) {
   p.slices = (V + bins_max - 1) / bins_max;
   p.slice = (V + p.slices - 1) / p.slices;
   p.slice_smem = (size_t)p.slice * 4;
+  // Half-word slices (a multiple of 8 ids) where two of them at most take the
+  // place of two or three 32-bit ones, from 2^23 positions on (151936 ids, both
+  // with the same logarithm kernel's older form: 2^22 positions 29 us as 32-bit
+  // slices, 33 as halves; 2^24 - 1 positions 58 and 52; against the hot scheme
+  // 2^24 positions 100 and 52, 2^28 466 and 376).
+  const long long half_max = (smem - 2048) / 2 / 8 * 8;
+  const long long halves = ((long long)V + half_max - 1) / half_max;
+  if (p.slices > 1 && halves <= 2 && N >= kPriorHalvesMinN) {
+    p.halves = (int)halves;
+    p.slice = (int)(((V + halves - 1) / halves + 7) / 8 * 8);
+    p.slice_smem = (size_t)p.slice * 2;
+    p.members = std::max(1, sms / p.halves);
+    p.ok = true;
+    return p;
+  }
   // hot ids: the remap and as many 16-bit bins as fit beside it (slot
   // numbers have 17 bits in a remap word)
   p.nent = (V + kIdsPerWord - 1) / kIdsPerWord;
@@ -547,6 +769,14 @@ PriorPlan plan_prior(int V, long long N, int sms) {
   if (p.use_hot) p.prefix = std::min<long long>(N, std::max<long long>(kPriorHotMinN / 4, N / 64));
   p.ok = true;
   return p;
+}
+
+cudaError_t launch_prior_halves(const PriorHalvesArgs& a, size_t smem, cudaStream_t s) {
+  cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_prior_halves), smem);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_prior_halves, dim3((unsigned)(a.members * a.slices)), dim3(kThreads), smem, s, a);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_prior_halves_reduce, dim3((unsigned)((a.slice + 255) / 256), (unsigned)a.slices), dim3(256), 0, s, a);
 }
 
 cudaError_t launch_prior_slices(const PriorSliceArgs& a, size_t smem, int max_members, int sms, cudaStream_t s) {
@@ -581,9 +811,8 @@ cudaError_t launch_prior_total(const PriorLogArgs& a, int sms, cudaStream_t s) {
 }
 
 cudaError_t launch_prior_log(const PriorLogArgs& a, int sms, cudaStream_t s) {
-  long long blocks = ((long long)a.V + 4 * kMapThreads - 1) / (4 * kMapThreads);
-  blocks = std::max<long long>(1, std::min<long long>(blocks, (long long)sms));
-  return launch_pdl(k_prior_log, dim3((unsigned)blocks), dim3(kMapThreads), 0, s, a);
+  const long long blocks = std::max<long long>(1, std::min<long long>(((long long)a.V + kThreads - 1) / kThreads, sms));
+  return launch_pdl(k_prior_log, dim3((unsigned)blocks), dim3(kThreads), 0, s, a);
 }
 
 }  // namespace dels

@@ -231,3 +231,45 @@ def test_hot_path_vocabulary_a_multiple_of_15_with_bad_ids():
     out, c, tally = _estimate(tok.to(DEV), mask.to(DEV), V)
     np.testing.assert_array_equal(c, c_ref)
     assert tally.tolist() == [n_in, n_out] and n_out == 57
+
+
+# ----------------------------------------------------------- half-word slices
+
+
+@pytest.mark.parametrize("V,N", [
+    (57601, 1 << 23),              # past one slice of 32-bit bins: one slice of halves
+    (115200, (1 << 23) + 77),      # the largest vocabulary of one slice
+    (115201, (1 << 23) + 5),       # two slices, an odd vocabulary
+    (115208, (1 << 23) - 1),       # one position short of the rule: 32-bit slices
+    (230400, (1 << 24) + 3),       # the largest vocabulary of two slices, a range the hot scheme would take
+    (230401, (1 << 24) + 3),       # one id more: a prefix of 32-bit slices, then the hot scheme
+    (230401, 100003),              # ... and a short range
+])
+def test_half_word_slices_match_oracle(V, N):
+    """Uniform ids (every bin used), a share of bad ids and of one hot id, at the edges of the plan."""
+    g = torch.Generator().manual_seed(V + N)
+    tok = torch.randint(-2, V + 2, (N,), generator=g, dtype=torch.int32)
+    tok[torch.rand(N, generator=g) < 0.2] = V - 1
+    tok[::4999] = -(2 ** 31)
+    mask = (torch.rand(N, generator=g) < 0.75).to(torch.uint8) * 2
+    c_ref, n_in, n_out = oracle.count_masked_tokens(tok.numpy(), mask.numpy(), V)
+    out, c, tally = _estimate(tok.to(DEV), mask.to(DEV), V)
+    np.testing.assert_array_equal(c, c_ref)
+    assert tally.tolist() == [n_in, n_out] and n_out > 0
+    _check_log_prior(out, c_ref, 1.0)
+
+
+@pytest.mark.parametrize("lam", [5e-324, 1e-310, 1e-5, 0.3, 3e7, 1e301])
+def test_log_prior_over_smoothing_weights(lam):
+    """The table-driven logarithm and, outside [1e-300, 1e300], the general one."""
+    V = 3000
+    c_ref = np.concatenate([np.arange(2000), 2 ** np.linspace(0, 50, 1000)]).astype(np.int64)
+    counts = torch.from_numpy(c_ref).to(DEV)
+    ws, nbytes = _ws(V, 0)
+    out = torch.empty(V, dtype=torch.float32, device=DEV)
+    assert dels.dels_prior_log(counts, V, lam, out, ws, nbytes) == 0
+    c = c_ref.astype(np.float64)
+    ref = np.log(c + lam) - np.log(c.sum() + V * lam)
+    got = out.cpu().numpy().astype(np.float64)
+    # one float32 rounding of the result, and the float64 error of the two logarithms
+    assert np.all(np.abs(got - ref) <= np.abs(ref) * 2.0 ** -24 + 1e-12), np.abs(got - ref).max()
