@@ -1303,9 +1303,17 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
     PROF(DELS_KCLASS_VOCAB_COMBINE);
     return launch_vocab_combine_f32(vf, vf_chunks, s);
   };
-  auto gemv_f32 = [&](const GemvF32Jobs& jobs, int njobs, int O, int act) {
+  // The first product of a float32 head decodes position j - 1 and gathers its
+  // input itself when each request has few records (every CTA merges them: one
+  // request, V 1024, 16 records, 73 -> 62 us per block of 8; 8 requests with
+  // 250 records each 203 -> 219 us).
+  auto merges_f32 = [&](int K, int feat_width) {
+    int rows = 0;
+    return !bf && gemv_f32_merges(B, K) && vocab_f32_chunks(B, feat_width, V, L.partial_ld, sms, &rows) <= 32;
+  };
+  auto gemv_f32 = [&](const GemvF32Jobs& jobs, int njobs, int O, int act, const MergeArgs* merge) {
     PROF(DELS_KCLASS_HEAD_MISC);
-    return launch_gemv_f32(jobs, njobs, B, O, act, O, sms, s);
+    return launch_gemv_f32(jobs, njobs, B, O, act, O, sms, s, merge);
   };
 
   switch (head->kind) {
@@ -1512,14 +1520,12 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
         return DELS_OK;
       }
-      // h_0 = 0: the position-0 merge clears the recurrent state
-      mb.zero_f32 = h;
-      mb.zero_bf16 = hb;
-      mb.zero_len = H;
-      r = draft_position0(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, mb, sms, s);
-      mb.zero_f32 = nullptr;
-      mb.zero_bf16 = nullptr;
-      mb.zero_len = 0;
+      // (h_0 = 0: the gates of position 1 take no recurrent partials and no state)
+      const bool fused = merges_f32(std::max(D, H), R);
+      int count = 0;
+      r = fused && n > 1 ? position0_rows(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, sms, s,
+                                          &count, &mb.smp)
+                         : draft_position0(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, mb, sms, s);
       if (r != DELS_OK || n == 1) return r;
       if (bf) {
         // Per position: the merge gathers e = E[x_{j-1}]; the input product
@@ -1564,16 +1570,20 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         gates.j[0] = GemvF32Job{E, Wih, gpart, D, D};
         gates.j[1] = GemvF32Job{h, Whh, gpart + (size_t)B * 3 * H, H, H};
         rank.j[0] = GemvF32Job{h, Wr, feat, H, H};
+        // fused: the products' launch decodes position j - 1 and gathers its
+        // input itself; the recurrent product needs h_{j-1} (none at j = 1)
         for (int j = 1; j < n; ++j) {
-          DELS_CUDA(gemv_f32(gates, 2, 3 * H, ACT_NONE));
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, 1, gpart + (size_t)B * 3 * H, 1, B, H, h, hb, s)); }
-          DELS_CUDA(gemv_f32(rank, 1, R, ACT_SILU));
-          DELS_CUDA(vocab_f32(feat, R, j));
           MergeArgs m = mb;
+          m.j = j - 1;
+          m.count = j == 1 ? count : vf_chunks;
+          DELS_CUDA(gemv_f32(gates, j == 1 ? 1 : 2, 3 * H, ACT_NONE, fused ? &m : nullptr));
+          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates(gpart, 1, gpart + (size_t)B * 3 * H, j == 1 ? 0 : 1, B, H, h, hb, s)); }
+          DELS_CUDA(gemv_f32(rank, 1, R, ACT_SILU, nullptr));
+          DELS_CUDA(vocab_f32(feat, R, j));
           m.count = vf_chunks;
           m.j = j;
           if (j == n - 1) m.table = nullptr;
-          { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
+          if (!fused || j == n - 1) { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
         }
       }
       return DELS_OK;
@@ -1589,7 +1599,16 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       mb.window = W;
       mb.dest = u;
       mb.smp.src_r = feat;
-      r = draft_position0(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, mb, sms, s);
+      // a few requests: each layer is one CUDA-core launch (product, GELU and
+      // bf16 rounding together) instead of a split-K product plus its reduction
+      const bool gemv = bf && gemv_bf16_ok(B, K1) && gemv_bf16_ok(B, Hd);
+      // Not at temperature 1 with one layer: the position's kept feature would
+      // be overwritten by the launch that copies it.
+      const bool fused = merges_f32(K1, Hd) && !(sm.on && head->n_layers == 1);
+      int count = 0;
+      r = fused && n > 1 ? position0_rows(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, sms, s,
+                                          &count, &mb.smp)
+                         : draft_position0(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, mb, sms, s);
       if (r != DELS_OK || n == 1) return r;
       if (bf) {
         Gemm g1, g2, gv;
@@ -1603,9 +1622,6 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         if (!plan_combine(gv, B, V, n, feat, Hd, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
                           partials, L.partial_ld, status, sms, true))
           return DELS_ERR_CUDA;
-        // a few requests: each layer is one CUDA-core launch (product, GELU and
-        // bf16 rounding together) instead of a split-K product plus its reduction
-        const bool gemv = gemv_bf16_ok(B, K1) && gemv_bf16_ok(B, Hd);
         for (int j = 1; j < n; ++j) {
           if (gemv) {
             { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(launch_gemv_bf16(static_cast<const uint16_t*>(u), K1,
@@ -1645,14 +1661,16 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         l2.j[0] = GemvF32Job{static_cast<const float*>(h1), static_cast<const float*>(head->w[1]),
                              static_cast<float*>(h2), Hd, Hd};
         for (int j = 1; j < n; ++j) {
-          DELS_CUDA(gemv_f32(l1, 1, Hd, ACT_GELU));
-          if (head->n_layers == 2) DELS_CUDA(gemv_f32(l2, 1, Hd, ACT_GELU));
-          DELS_CUDA(vocab_f32(feat, Hd, j));
           MergeArgs m = mb;
+          m.j = j - 1;
+          m.count = j == 1 ? count : vf_chunks;
+          DELS_CUDA(gemv_f32(l1, 1, Hd, ACT_GELU, fused ? &m : nullptr));
+          if (head->n_layers == 2) DELS_CUDA(gemv_f32(l2, 1, Hd, ACT_GELU, nullptr));
+          DELS_CUDA(vocab_f32(feat, Hd, j));
           m.count = vf_chunks;
           m.j = j;
           if (j == n - 1) m.table = nullptr;
-          { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
+          if (!fused || j == n - 1) { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
         }
       }
       return DELS_OK;

@@ -188,10 +188,6 @@ struct MergeArgs {
   int table_f32;
   int D, window;
   void* dest;                    // [B, window*D] same dtype as table
-  // optional per-row zeroing (recurrent state at the start of a block)
-  float* zero_f32;               // [B, zero_len]
-  uint16_t* zero_bf16;           // [B, zero_len]
-  int zero_len;
   SampleArgs smp;
 };
 cudaError_t launch_draft_merge(const MergeArgs& a, cudaStream_t s);
@@ -380,8 +376,11 @@ struct GemvF32Job {
 struct GemvF32Jobs {
   GemvF32Job j[2];
 };
+// merge: decode position merge->j and take job 0's input from the gathered
+// head input (job 0's X is not read); allowed when gemv_f32_merges.
+bool gemv_f32_merges(int B, int K);
 cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, int act, int ldy, int sms,
-                            cudaStream_t s);
+                            cudaStream_t s, const MergeArgs* merge = nullptr);
 // float32 vocabulary projection fused with the combine: one record per
 // (request, vocabulary chunk of chunk_rows rows).
 struct VocabF32Args {

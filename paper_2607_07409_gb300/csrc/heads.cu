@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) k_gru_gates(const float* gi, int Si, cons
     const float r = sigmoidf_(gir + ghr);
     const float z = sigmoidf_(giz + ghz);
     const float c = tanhf(gin + r * ghn);
-    const float hp = h[e];
+    const float hp = Sh > 0 ? h[e] : 0.f;   // h_0 = 0
     const float hn = (1.f - z) * c + z * hp;
     h[e] = hn;
     h_bf16[e] = f32_to_bf16_rne(hn);

@@ -13,11 +13,14 @@
 // vocabulary of 32000 x 256 57 -> 14 us (33 MB of weights: 5 us) and the two
 // GRU products of 1536 x 1024 and 1536 x 512 25 + 17 -> 7.3 us in one launch;
 // for one request, the vocabulary of 1024 x 128 33 us on 4 CTAs -> 5.3 us on
-// 16, where a launch with nothing to do takes about 4.
+// 16, where a launch with nothing to do takes about 4. First weights loaded
+// before the wait for the predecessor: block of 8 for that request 62 -> 59 us,
+// the 8-request block 203 -> 193 us (215 where the vocabulary's chunks are
+// several tiles per warp, so those do without).
 #include <algorithm>
 #include <climits>
 
-#include "dels_device.cuh"
+#include "merge_rows.cuh"
 
 namespace dels {
 
@@ -33,34 +36,51 @@ __device__ __forceinline__ float4 load4w(const float* p) {
   return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
 }
 
-// acc[r * BG + b] += sum over this lane's k (k0, k0 + kstep, ..., 4 at a time)
-// of W[o0 + r, k] x[b, k]; rows past o_last repeat it (their sums are unused).
+// The R weight rows from o0 at this lane's k; rows past o_last repeat it (their
+// sums are unused).
+template <int R, bool VEC>
+__device__ __forceinline__ void load_rows(const float* __restrict__ W, int o0, int o_last, int K, int k,
+                                          float4 (&w)[R]) {
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    w[r] = k < K ? load4w<VEC>(W + (long long)min(o0 + r, o_last) * K + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+// acc[r * BG + b] += w[r] . x[b, k .. k + 3]
+template <int R, int BG, bool STAGED>
+__device__ __forceinline__ void fma_rows(const float4 (&w)[R], const float* x, long long ldx, int nb, int K, int k,
+                                         float (&acc)[R * BG]) {
+#pragma unroll
+  for (int b = 0; b < BG; ++b) {
+    float4 v;
+    if constexpr (STAGED) v = *reinterpret_cast<const float4*>(x + b * K + k);
+    else v = b < nb ? __ldcg(reinterpret_cast<const float4*>(x + b * ldx + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      float& s = acc[r * BG + b];
+      s = fmaf(w[r].x, v.x, s);
+      s = fmaf(w[r].y, v.y, s);
+      s = fmaf(w[r].z, v.z, s);
+      s = fmaf(w[r].w, v.w, s);
+    }
+  }
+}
+
+// acc[r * BG + b] = sum over this lane's k (k0, k0 + kstep, ..., 4 at a time)
+// of W[o0 + r, k] x[b, k]; `w` holds the rows at k0 (load_rows).
 // x: [BG][K] in shared memory, or (STAGED false) request rows in global memory.
 template <int R, int BG, bool STAGED, bool VEC>
 __device__ __forceinline__ void dot_rows(const float* __restrict__ W, int o0, int o_last, int K, const float* x,
-                                         long long ldx, int nb, int k0, int kstep, float (&acc)[R * BG]) {
-  const float* wr[R];
+                                         long long ldx, int nb, int k0, int kstep, const float4 (&w)[R],
+                                         float (&acc)[R * BG]) {
 #pragma unroll
-  for (int r = 0; r < R; ++r) wr[r] = W + (long long)min(o0 + r, o_last) * K;
+  for (int i = 0; i < R * BG; ++i) acc[i] = 0.f;
+  if (k0 < K) fma_rows<R, BG, STAGED>(w, x, ldx, nb, K, k0, acc);
 #pragma unroll 2
-  for (int k = k0; k < K; k += kstep) {
-    float4 w[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = load4w<VEC>(wr[r] + k);
-#pragma unroll
-    for (int b = 0; b < BG; ++b) {
-      float4 v;
-      if constexpr (STAGED) v = *reinterpret_cast<const float4*>(x + b * K + k);
-      else v = b < nb ? __ldcg(reinterpret_cast<const float4*>(x + b * ldx + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        float& s = acc[r * BG + b];
-        s = fmaf(w[r].x, v.x, s);
-        s = fmaf(w[r].y, v.y, s);
-        s = fmaf(w[r].z, v.z, s);
-        s = fmaf(w[r].w, v.w, s);
-      }
-    }
+  for (int k = k0 + kstep; k < K; k += kstep) {
+    float4 v[R];
+    load_rows<R, VEC>(W, o0, o_last, K, k, v);
+    fma_rows<R, BG, STAGED>(v, x, ldx, nb, K, k, acc);
   }
 }
 
@@ -101,33 +121,51 @@ __device__ __forceinline__ void stage_rows(float* sx, const float* X, long long 
 }
 
 // Y[b, o] = act(sum_k X[b, k] W[o, k]) for up to two independent products
-// with the same O (blockIdx.z). KS warps split each row group's K (their sums
+// with the same O (blockIdx.z). MERGE: the first product's input is the head
+// input of the position that m decodes (merge_requests), not X. KS warps split each row group's K (their sums
 // are added in order), so that small matrices still fill the chip.
-template <int R, int BG, bool STAGED, bool VEC>
+template <int R, int BG, bool STAGED, bool VEC, bool MERGE>
 __global__ void __launch_bounds__(kThreadsF32, 2)
-    k_gemv_f32(const __grid_constant__ GemvF32Jobs jobs, int B, int O, int act, int ldy, int KS) {
+    k_gemv_f32(const __grid_constant__ GemvF32Jobs jobs, int B, int O, int act, int ldy, int KS,
+               const __grid_constant__ MergeArgs m) {
   extern __shared__ __align__(16) float sx[];
   __shared__ float red[kWarpsF32][32];
+  __shared__ int s_tok[MERGE ? BG : 1];
   constexpr int NV = R * BG;
   if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
   const GemvF32Job& jb = jobs.j[blockIdx.z];
   const int b0 = blockIdx.y * BG, nb = min(BG, B - b0);
   const int K = jb.K;
   const float* X = jb.X + (long long)b0 * jb.ldx;
-  if constexpr (STAGED) stage_rows<BG>(sx, X, jb.ldx, nb, K);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int rg = warp / KS, kw = warp % KS;
   const int per = kWarpsF32 / KS * R;
+  const int k0 = (kw * 32 + lane) * 4;
+  // the first weights go out before the wait: they are not the predecessor's
+  float4 w[R];
+  load_rows<R, VEC>(jb.W, blockIdx.x * per + rg * R, O - 1, K, k0, w);
+  pdl_wait();
+  if (MERGE && blockIdx.z == 0) {
+    const bool writer = blockIdx.x == 0;
+    merge_requests(m, b0, nb, writer, s_tok);
+    if (writer)
+      for (int q = 0; q < nb; ++q) keep_draft_input(m.smp, b0 + q, m.n, m.j);
+    const int vecs = m.D / 4;
+    for (int i = threadIdx.x; i < BG * (K / 4); i += kThreadsF32) {
+      const int q = i / (K / 4), v = i - q * (K / 4);
+      reinterpret_cast<uint4*>(sx)[i] = q < nb ? gather_vec(m, b0, q, v, vecs, s_tok) : make_uint4(0, 0, 0, 0);
+    }
+    __syncthreads();
+  } else if constexpr (STAGED) {
+    stage_rows<BG>(sx, X, jb.ldx, nb, K);
+  }
   const int idx = lane / (32 / NV), r = idx / BG, b = idx % BG;
   const bool leader = lane % (32 / NV) == 0;
   for (int base = blockIdx.x * per; base < O; base += gridDim.x * per) {
     const int o0 = base + rg * R;
     float acc[NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] = 0.f;
-    if (o0 < O)
-      dot_rows<R, BG, STAGED, VEC>(jb.W, o0, O - 1, K, STAGED ? sx : X, jb.ldx, nb, (kw * 32 + lane) * 4, KS * 128, acc);
+    if (base > (int)(blockIdx.x * per)) load_rows<R, VEC>(jb.W, o0, O - 1, K, k0, w);
+    dot_rows<R, BG, STAGED, VEC>(jb.W, o0, O - 1, K, STAGED ? sx : X, jb.ldx, nb, k0, KS * 128, w, acc);
     float s = transpose_reduce<NV>(acc);
     if (KS > 1) {
       red[warp][lane] = s;
@@ -143,22 +181,25 @@ __global__ void __launch_bounds__(kThreadsF32, 2)
 // Vocabulary projection fused with the combine: CTA (chunk, request group)
 // computes l_S[v] = W_vocab[v] . feat[b] over its vocabulary chunk, fuses
 // l = l_L + alpha l_S - beta l_P (at temperature 1 the top-2 runs over l + g)
-// and writes one record per request.
-template <int R, int BG, bool STAGED>
+// and writes one record per request. ONE: the chunk is one tile per warp, whose
+// first weights are loaded before the wait for the predecessor.
+template <int R, int BG, bool STAGED, bool ONE>
 __global__ void __launch_bounds__(kThreadsF32, 2)
     k_vocab_combine_f32(const __grid_constant__ VocabF32Args a) {
   extern __shared__ __align__(16) float sx[];
   __shared__ RowAcc red[kWarpsF32][32];
   constexpr int NV = R * BG;
   if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
   const int groups = (a.B + BG - 1) / BG;
   const int chunk = blockIdx.x / groups, b0 = (int)(blockIdx.x % groups) * BG;
   const int nb = min(BG, a.B - b0);
   const int v0 = chunk * a.chunk_rows, v1 = min(a.V, v0 + a.chunk_rows);
   const float* X = a.feat + (long long)b0 * a.K;
-  if constexpr (STAGED) stage_rows<BG>(sx, X, a.K, nb, a.K);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4 w[R];
+  if constexpr (ONE) load_rows<R, true>(a.W, v0 + warp * R, a.V - 1, a.K, lane * 4, w);
+  pdl_wait();
+  if constexpr (STAGED) stage_rows<BG>(sx, X, a.K, nb, a.K);
   const int idx = lane / (32 / NV), r = idx / BG, b = idx % BG;
   const bool mine = lane % (32 / NV) == 0 && b < nb;
   const long long lrow = (long long)(b0 + b) * a.ld_long;
@@ -174,9 +215,8 @@ __global__ void __launch_bounds__(kThreadsF32, 2)
       p = __ldg(a.prior + v);
     }
     float acc[NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) acc[i] = 0.f;
-    dot_rows<R, BG, STAGED, true>(a.W, o0, a.V - 1, a.K, STAGED ? sx : X, a.K, nb, lane * 4, 128, acc);
+    if constexpr (!ONE) load_rows<R, true>(a.W, o0, a.V - 1, a.K, lane * 4, w);
+    dot_rows<R, BG, STAGED, true>(a.W, o0, a.V - 1, a.K, STAGED ? sx : X, a.K, nb, lane * 4, 128, w, acc);
     const float d = transpose_reduce<NV>(acc);
     if (live) {
       const float f[1] = {fmaf(-a.beta, p, fmaf(a.alpha, d, l))};
@@ -213,18 +253,21 @@ int rows_per_warp(int bg) { return bg == 8 ? 4 : 8; }
 bool staged(int bg, int K) { return (size_t)bg * K * 4 <= kStageLimit; }
 
 template <int R, int BG>
-cudaError_t launch_gemv_bg(const GemvF32Jobs& jobs, int njobs, int B, int O, int act, int ldy, bool stage, bool vec,
-                           int KS, dim3 grid, size_t smem, cudaStream_t s) {
-  auto kern = stage ? (vec ? k_gemv_f32<R, BG, true, true> : k_gemv_f32<R, BG, true, false>)
-                    : (vec ? k_gemv_f32<R, BG, false, true> : k_gemv_f32<R, BG, false, false>);
+cudaError_t launch_gemv_bg(const GemvF32Jobs& jobs, int B, int O, int act, int ldy, bool stage, bool vec, int KS,
+                           dim3 grid, size_t smem, const MergeArgs* merge, cudaStream_t s) {
+  auto kern = merge   ? k_gemv_f32<R, BG, true, true, true>
+              : stage ? (vec ? k_gemv_f32<R, BG, true, true, false> : k_gemv_f32<R, BG, true, false, false>)
+                      : (vec ? k_gemv_f32<R, BG, false, true, false> : k_gemv_f32<R, BG, false, false, false>);
   const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, grid, dim3(kThreadsF32), smem, s, jobs, B, O, act, ldy, KS);
+  return launch_pdl(kern, grid, dim3(kThreadsF32), smem, s, jobs, B, O, act, ldy, KS, merge ? *merge : MergeArgs{});
 }
 
 template <int R, int BG>
 cudaError_t launch_vocab_bg(const VocabF32Args& a, bool stage, dim3 grid, size_t smem, cudaStream_t s) {
-  auto kern = stage ? k_vocab_combine_f32<R, BG, true> : k_vocab_combine_f32<R, BG, false>;
+  const bool one = a.chunk_rows <= kWarpsF32 * R;
+  auto kern = stage ? (one ? k_vocab_combine_f32<R, BG, true, true> : k_vocab_combine_f32<R, BG, true, false>)
+                    : k_vocab_combine_f32<R, BG, false, false>;
   const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(kern, grid, dim3(kThreadsF32), smem, s, a);
@@ -232,8 +275,10 @@ cudaError_t launch_vocab_bg(const VocabF32Args& a, bool stage, dim3 grid, size_t
 
 }  // namespace
 
+bool gemv_f32_merges(int B, int K) { return staged(group_size(B, K), K); }
+
 cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, int act, int ldy, int sms,
-                            cudaStream_t s) {
+                            cudaStream_t s, const MergeArgs* merge) {
   if (njobs < 1 || njobs > 2 || B < 1 || O < 1) return cudaErrorInvalidValue;
   int K = jobs.j[0].K;
   bool vec = true;
@@ -244,6 +289,7 @@ cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, in
   }
   const int bg = group_size(B, K), R = rows_per_warp(bg);
   const bool stage = staged(bg, K);
+  if (merge && (!stage || !vec)) return cudaErrorInvalidValue;
   const int groups = (B + bg - 1) / bg;
   if (groups > 65535) return cudaErrorInvalidValue;
   // K split over the warps of a CTA until about eight warps per SM have work
@@ -256,10 +302,10 @@ cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, in
   const dim3 grid((unsigned)ctas, (unsigned)groups, (unsigned)njobs);
   const size_t smem = stage ? (size_t)bg * K * 4 : 0;
   switch (bg) {
-    case 1: return launch_gemv_bg<8, 1>(jobs, njobs, B, O, act, ldy, stage, vec, KS, grid, smem, s);
-    case 2: return launch_gemv_bg<8, 2>(jobs, njobs, B, O, act, ldy, stage, vec, KS, grid, smem, s);
-    case 4: return launch_gemv_bg<8, 4>(jobs, njobs, B, O, act, ldy, stage, vec, KS, grid, smem, s);
-    default: return launch_gemv_bg<4, 8>(jobs, njobs, B, O, act, ldy, stage, vec, KS, grid, smem, s);
+    case 1: return launch_gemv_bg<8, 1>(jobs, B, O, act, ldy, stage, vec, KS, grid, smem, merge, s);
+    case 2: return launch_gemv_bg<8, 2>(jobs, B, O, act, ldy, stage, vec, KS, grid, smem, merge, s);
+    case 4: return launch_gemv_bg<8, 4>(jobs, B, O, act, ldy, stage, vec, KS, grid, smem, merge, s);
+    default: return launch_gemv_bg<4, 8>(jobs, B, O, act, ldy, stage, vec, KS, grid, smem, merge, s);
   }
 }
 

@@ -1,0 +1,50 @@
+// The per-position merge inside a consumer's launch: every CTA that needs the
+// next head input merges its requests' records itself (one warp per request)
+// and gathers the embedding rows into shared memory, so that the merge costs
+// no launch of its own. One CTA per request group writes the decoded outputs.
+#pragma once
+
+#include "dels_device.cuh"
+
+namespace dels {
+
+// Tokens of requests b0 .. b0 + nb - 1 at position m.j into s_tok (valid after
+// the __syncthreads that ends the call).
+__device__ __forceinline__ void merge_requests(const MergeArgs& m, int b0, int nb, bool writer, int* s_tok) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int q = warp; q < nb; q += nw) {
+    const int b = b0 + q;
+    const float4* rec = reinterpret_cast<const float4*>(m.partials) + (long long)b * m.partial_ld;
+    RowAcc x = rowacc_init();
+    for (int k0 = lane; k0 < m.count; k0 += 4 * 32) {   // four records in flight
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * 32 < m.count) v[u] = __ldcg(rec + k0 + u * 32);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * 32 < m.count) {
+          RowAcc y;
+          y.m = v[u].x; y.s = v[u].y; y.second = v[u].z; y.idx = __float_as_int(v[u].w);
+          x = rowacc_merge(x, y);
+        }
+    }
+    x = rowacc_warp_reduce(x);
+    if (lane == 0) {
+      s_tok[q] = (m.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
+      if (writer) decode_record(x, m.smp, b, m.n, m.j, m.tokens, m.out_lp, m.out_gap, m.status);
+    }
+  }
+  __syncthreads();
+}
+
+// 16-byte vector v of request b0 + q's head input (the embedding rows of its
+// last m.window tokens, zeros before the block): vecs of them per token row.
+__device__ __forceinline__ uint4 gather_vec(const MergeArgs& m, int b0, int q, int v, int vecs, const int* s_tok) {
+  const int w = v / vecs, k = v - w * vecs;
+  const int j = m.j - w;
+  const int tok = w == 0 ? s_tok[q] : j >= 0 ? __ldcg(m.tokens + (long long)(b0 + q) * m.n + j) : -1;
+  return tok >= 0 ? __ldg(reinterpret_cast<const uint4*>(m.table) + (long long)tok * vecs + k) : make_uint4(0, 0, 0, 0);
+}
+
+}  // namespace dels

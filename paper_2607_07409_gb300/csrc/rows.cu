@@ -432,12 +432,6 @@ __global__ void __launch_bounds__(256) k_draft_merge(MergeArgs a) {
   if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x;
-  if (a.zero_len > 0) {
-    for (int i = threadIdx.x; i < a.zero_len; i += blockDim.x) {
-      if (a.zero_f32) a.zero_f32[(long long)b * a.zero_len + i] = 0.f;
-      if (a.zero_bf16) a.zero_bf16[(long long)b * a.zero_len + i] = 0;
-    }
-  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ RowAcc red[8];
   __shared__ int s_tok;

@@ -266,7 +266,9 @@ def test_draft_small_matches_oracle(name, stress):
     ("gru", 2, 72, 8, 4, 4),                # two requests, the smallest widths
     ("gru", 9, 4104, 260, 128, 132),        # a second group of one request
     ("mlp", 4, 2000, 64, 520, 520),         # four requests
-    ("mlp", 17, 1504, 32, 100, 100),        # three groups
+    ("mlp", 17, 1504, 32, 100, 100),        # three groups, 47 records per request: merge launches
+    ("mlp", 17, 1024, 32, 100, 100),        # 32 records: the first product's launch merges and gathers
+    ("mlp", 1, 8, 16, 4, 4),                # the smallest vocabulary
     ("markov", 3, 136, 0, 0, 12000),        # two requests' rows fit the staging limit
     ("markov", 6, 64, 0, 0, 24580),         # not one row does: the rows are read through L2
 ])
