@@ -261,6 +261,17 @@ def test_draft_small_matches_oracle(name, stress):
     print(name, stress, record(f"draft {name}, stress {stress}", info))
 
 
+@pytest.mark.parametrize("head,r", [("markov", 112), ("markov", 208), ("gru", 240), ("gru", 368), ("gru", 160)])
+def test_draft_ragged_feature_width(head, r):
+    """Feature widths whose last 64-wide K chunk is ragged, in an even and an
+    odd number of chunks: every column of W_vocab counts."""
+    spec = synth.HeadSpec(head, "bf16", 256 if head == "gru" else 0, 128 if head == "gru" else 0, r)
+    w = synth.stress(synth.Workload("ragged", B=6, n=4, V=3000, logit_dtype="bf16", head=spec, weight=1.0, seed=r))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    tok, lp, gap, W, prior = _draft(w, d)
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 @pytest.mark.parametrize("head,B,V,d,h,r", [
     ("gru", 1, 1000, 132, 36, 20),          # one request; widths just past and below a 128-wide step
     ("gru", 2, 72, 8, 4, 4),                # two requests, the smallest widths
