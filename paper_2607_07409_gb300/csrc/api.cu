@@ -180,17 +180,28 @@ bool map_w(CUtensorMap* m, const void* W, int O, int K, int n_tile) {
                         (uint32_t)n_tile, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// W as [K / 64][O][64], boxes of two K chunks (K a multiple of 64).
+bool map_w_pairs(CUtensorMap* m, const void* W, int O, int K, int n_tile) {
+  return encode_tmap_3d(m, W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, (uint64_t)O, (uint64_t)(K / 64),
+                        (uint64_t)K * 2, 128, 64, (uint32_t)n_tile, 2, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
 int pick_stages(const TcGemmArgs& a, int per_stage, int fixed) {
   const int budget = device_max_smem_optin() - kSmemReserve - fixed;
   int st = budget / per_stage;
   return std::max(2, std::min(st, 12));
 }
 
+// pair_stages: two K chunks per pipeline stage where K is whole pairs. Taken
+// for the GRU's rank and recurrent products (64 requests, block of 16: 518 ->
+// 501 us with both, 521 and 509 with one); the input product and the
+// transformer head's products were no faster with it (374 -> 381 us for the
+// ragged block of 11, 3108 -> 3118 us).
 // Y = act(X0 W0^T) over K split into `splits` pieces (segment 1 optional:
 // + X1 W1^T with its own splits, written as separate partials).
 bool plan_store(Gemm& g, int B, int O, const void* X0, const void* W0, int K0, const void* X1, const void* W1,
                 int K1, int n_tile, int splits0, int splits1, int act, float* out_f32, uint16_t* out_bf16,
-                int ldo_bf16, int* status, int sms) {
+                int ldo_bf16, int* status, int sms, bool pair_stages = false) {
   TcGemmArgs& a = g.a;
   a.B = B;
   a.O = O;
@@ -198,15 +209,16 @@ bool plan_store(Gemm& g, int B, int O, const void* X0, const void* W0, int K0, c
   a.num_o_tiles = (O + n_tile - 1) / n_tile;
   a.seg_chunks[0] = (K0 + 63) / 64;
   a.seg_chunks[1] = K1 > 0 ? (K1 + 63) / 64 : 0;
-  // make every split non-empty
-  auto fix = [](int nch, int s) {
-    if (nch == 0) return 0;
-    s = std::max(1, std::min(s, nch));
-    const int per = (nch + s - 1) / s;
-    return (nch + per - 1) / per;
-  };
-  a.seg_splits[0] = fix(a.seg_chunks[0], splits0);
-  a.seg_splits[1] = fix(a.seg_chunks[1], splits1);
+  // two K chunks per stage, the weights' as one 3-D box (K in whole pairs)
+  a.b_chunks = pair_stages && K0 % 128 == 0 && K1 % 128 == 0 ? 2 : 1;
+  // make every split non-empty (and whole pairs of chunks)
+  for (int g = 0; g < 2; ++g) {
+    const int nch = a.seg_chunks[g];
+    if (nch == 0) continue;
+    const int s = std::max(1, std::min(g ? splits1 : splits0, nch));
+    a.seg_per[g] = ((nch + s - 1) / s + a.b_chunks - 1) / a.b_chunks * a.b_chunks;
+    a.seg_splits[g] = (nch + a.seg_per[g] - 1) / a.seg_per[g];
+  }
   a.total_splits = a.seg_splits[0] + a.seg_splits[1];
   a.epi = EPI_STORE;
   a.a_resident = 0;
@@ -220,10 +232,13 @@ bool plan_store(Gemm& g, int B, int O, const void* X0, const void* W0, int K0, c
   // only the B real rows are loaded; the tile's other rows feed unused outputs
   a.a_box_rows = std::min(128, (B + 7) / 8 * 8);
   a.a_copies = 1;
-  a.stages = pick_stages(a, 128 * 128 + n_tile * 128, (out_f32 && !out_bf16) ? kStoreTransposeBytes : 0);
-  if (!map_x(&g.mA0, X0, B, K0, a.a_box_rows) || !map_w(&g.mB0, W0, O, K0, n_tile)) return false;
+  a.stages = pick_stages(a, a.b_chunks * (128 * 128 + n_tile * 128), (out_f32 && !out_bf16) ? kStoreTransposeBytes : 0);
+  auto weights = [&](CUtensorMap* m, const void* W, int K) {
+    return a.b_chunks == 2 ? map_w_pairs(m, W, O, K, n_tile) : map_w(m, W, O, K, n_tile);
+  };
+  if (!map_x(&g.mA0, X0, B, K0, a.a_box_rows) || !weights(&g.mB0, W0, K0)) return false;
   if (K1 > 0) {
-    if (!map_x(&g.mA1, X1, B, K1, a.a_box_rows) || !map_w(&g.mB1, W1, O, K1, n_tile)) return false;
+    if (!map_x(&g.mA1, X1, B, K1, a.a_box_rows) || !weights(&g.mB1, W1, K1)) return false;
   } else {
     g.mA1 = g.mA0;
     g.mB1 = g.mB0;
@@ -280,6 +295,7 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
   a.seg_chunks[1] = 0;
   a.seg_splits[0] = 1;
   a.seg_splits[1] = 0;
+  a.seg_per[0] = a.seg_chunks[0];
   a.total_splits = 1;
   a.epi = EPI_COMBINE;
   a.prior = prior;
@@ -327,9 +343,7 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
   }
   if (!map_x(&g.mA0, X, B, K, a.a_box_rows)) return false;
   if (a.b_chunks == 2) {
-    if (!encode_tmap_3d(&g.mB0, Wv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, (uint64_t)V, (uint64_t)(K / 64),
-                        (uint64_t)K * 2, 128, 64, (uint32_t)n_tile, 2, CU_TENSOR_MAP_SWIZZLE_128B))
-      return false;
+    if (!map_w_pairs(&g.mB0, Wv, V, K, n_tile)) return false;
   } else if (!map_w(&g.mB0, Wv, V, K, n_tile)) {
     return false;
   }
@@ -536,16 +550,15 @@ bool plan_rank_hh(Gemm& gr, Gemm& gh, const dels_local_head* hd, const DraftLayo
                   uint16_t* r, float* hh_part, int* status) {
   const int H = hd->d_hidden, R = hd->d_rank, sms = L.sms;
   if (!plan_store(gr, B, R, hb, hd->w[2], H, nullptr, nullptr, 0, kRankTile, kRankSplits, 0, ACT_SILU, nullptr, r, R,
-                  status, sms) ||
+                  status, sms, true) ||
       !plan_store(gh, B, 3 * H, hb, hd->w[1], H, nullptr, nullptr, 0, kHhTile, L.hh_splits, 0, ACT_NONE, hh_part,
-                  nullptr, 0, status, sms))
+                  nullptr, 0, status, sms, true))
     return false;
   const int ck = gr.a.total_splits;
   if (ck > 1) {
     gr.a.cluster_k = ck;
     gr.grid = gr.a.num_o_tiles * ck;
-    const int per = (gr.a.seg_chunks[0] + ck - 1) / ck;
-    gr.a.stages = std::max(2, std::min(gr.a.stages, per));
+    gr.a.stages = std::max(2, std::min(gr.a.stages, gr.a.seg_per[0] / gr.a.b_chunks));
     gr.smem = tc_gemm_smem_bytes(gr.a);
   }
   // both products fit one wave next to each other; whole clusters only

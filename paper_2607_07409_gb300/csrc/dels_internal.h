@@ -203,6 +203,7 @@ struct TcGemmArgs {
   int num_o_tiles;
   int seg_chunks[2];             // K chunks of 64 per segment
   int seg_splits[2];             // K splits per segment (0 splits: unused segment)
+  int seg_per[2];                // K chunks per split (the last may have fewer)
   int total_splits;
   int epi;
   int a_resident;                // A (activations) loaded once per CTA

@@ -100,11 +100,8 @@ __device__ __forceinline__ Item get_item(const TcGemmArgs& a, int i) {
   it.o0 = ot * a.n_tile;
   it.seg = (it.split < a.seg_splits[0]) ? 0 : 1;
   const int ls = it.seg ? it.split - a.seg_splits[0] : it.split;
-  const int nch = a.seg_chunks[it.seg];
-  const int ns = a.seg_splits[it.seg];
-  const int per = (nch + ns - 1) / ns;
-  it.kb = ls * per;
-  it.ke = min(nch, it.kb + per);
+  it.kb = ls * a.seg_per[it.seg];
+  it.ke = min(a.seg_chunks[it.seg], it.kb + a.seg_per[it.seg]);
   const int len = it.ke - it.kb;
   // two chunks per stage: the rotation keeps pairs of consecutive chunks
   if (a.b_chunks == 2)

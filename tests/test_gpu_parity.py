@@ -261,11 +261,13 @@ def test_draft_small_matches_oracle(name, stress):
     print(name, stress, record(f"draft {name}, stress {stress}", info))
 
 
-@pytest.mark.parametrize("head,r", [("markov", 112), ("markov", 208), ("gru", 240), ("gru", 368), ("gru", 160)])
-def test_draft_ragged_feature_width(head, r):
-    """Feature widths whose last 64-wide K chunk is ragged, in an even and an
-    odd number of chunks: every column of W_vocab counts."""
-    spec = synth.HeadSpec(head, "bf16", 256 if head == "gru" else 0, 128 if head == "gru" else 0, r)
+@pytest.mark.parametrize("head,r,h", [("markov", 112, 0), ("markov", 208, 0), ("gru", 240, 128), ("gru", 368, 128),
+                                      ("gru", 160, 240), ("gru", 64, 320), ("gru", 64, 640)])
+def test_draft_ragged_feature_width(head, r, h):
+    """Feature and state widths whose last 64-wide K chunk is ragged, in an even
+    and an odd number of chunks, and whole pairs of chunks that do not split
+    evenly: every column of W_vocab, W_rank and W_hh counts."""
+    spec = synth.HeadSpec(head, "bf16", 256 if head == "gru" else 0, h, r)
     w = synth.stress(synth.Workload("ragged", B=6, n=4, V=3000, logit_dtype="bf16", head=spec, weight=1.0, seed=r))
     d = synth.make_inputs(w, device=DEV, target=False)
     tok, lp, gap, W, prior = _draft(w, d)
