@@ -162,6 +162,84 @@ __device__ __forceinline__ RowAcc rowacc_warp_reduce(RowAcc a) {
   return a;
 }
 
+// Floats as integers of the same order (no NaN), for integer maxima.
+__device__ __forceinline__ int ordered_bits(float x) {
+  const int i = __float_as_int(x);
+  return i < 0 ? i ^ 0x7FFFFFFF : i;
+}
+__device__ __forceinline__ float from_ordered_bits(int i) { return __int_as_float(i < 0 ? i ^ 0x7FFFFFFF : i); }
+// Largest x of a whole warp (no NaN).
+__device__ __forceinline__ float warp_max(float x) {
+  return from_ordered_bits(__reduce_max_sync(0xFFFFFFFFu, ordered_bits(x)));
+}
+
+// One row scanned by a whole warp, all lanes together: each lane keeps the
+// top-2 of its own elements and its share of the sum of exponentials, and the
+// warp shares the reference of the sums (the largest element met, nb =
+// -ref log2(e)) and its runner-up T. An element below T changes neither the
+// row's top-1 nor its top-2 whichever lane holds it, so the top-2 update runs
+// only where a lane meets an element at or above T: of a warp's n-th group of
+// 256 elements about 2/n do, where a lane's own runner-up would let 64/n
+// through and some lane of the warp nearly always.
+struct WarpRow {
+  float best, second, s;   // per lane; s relative to the warp's reference
+  int idx;
+  float ref, T, nb;        // the same in every lane
+  __device__ __forceinline__ void init() {
+    best = second = ref = T = -INFINITY;
+    s = nb = 0.f;
+    idx = 0x7FFFFFFF;
+  }
+  // G groups of 8 values at columns c[g] (increasing), all lanes converged.
+  // While nothing finite has been met the values are -inf (0) or NaN (NaN).
+  template <int G>
+  __device__ __forceinline__ void push(const float (&f)[G][8], const int (&c)[G]) {
+    float vm[G], top = -INFINITY;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      vm[g] = fmaxf(fmaxf(fmaxf(f[g][0], f[g][1]), fmaxf(f[g][2], f[g][3])),
+                    fmaxf(fmaxf(f[g][4], f[g][5]), fmaxf(f[g][6], f[g][7])));
+      top = fmaxf(top, vm[g]);
+    }
+    if (__any_sync(0xFFFFFFFFu, top >= T && top > second)) {
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+        if (vm[g] > second) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) top2_push(f[g][i], c[g] + i, best, second, idx);
+        }
+      __syncwarp();
+      const float old = ref;
+      ref = warp_max(best);
+      T = warp_max(best == ref ? second : best);
+      if (ref != old) {
+        nb = -ref * kLog2e;
+        if (old != -INFINITY) s *= ex2_approx(fmaf(old, kLog2e, nb));
+      }
+    }
+    float acc[2] = {0.f, 0.f};
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i & 1] += ex2_approx(fmaf(f[g][i], kLog2e, nb));
+    s += acc[0] + acc[1];
+  }
+  // The warp's record, in every lane.
+  __device__ __forceinline__ RowAcc record() const {
+    RowAcc r;
+    r.m = ref;
+    r.second = T;
+    r.idx = __reduce_min_sync(0xFFFFFFFFu, best == ref ? idx : 0x7FFFFFFF);
+    // a tie for the top in two lanes: the runner-up equals the top
+    if (__popc(__ballot_sync(0xFFFFFFFFu, best == ref)) > 1) r.second = ref;
+    float x = s;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, d);
+    r.s = x;
+    return r;
+  }
+};
+
 // A finished row is valid when it had at least one finite entry and no
 // NaN / +inf (either of which turns s into NaN).
 __device__ __forceinline__ bool rowacc_valid(const RowAcc& a) {

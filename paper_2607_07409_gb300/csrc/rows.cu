@@ -9,6 +9,7 @@
 // ticket, reset by that CTA), so no [rows, V] intermediate is ever written.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 
@@ -72,26 +73,18 @@ __device__ __forceinline__ void st_rowacc(void* base, long long i, const RowAcc&
 }
 
 
-// Per-thread running state of one row.
+// Per-thread running state of one row, element by element (rows that cannot
+// take the vector path).
 struct RowState {
   float best, second, m, s;
   int idx;
   __device__ __forceinline__ void init() {
     best = -INFINITY; second = -INFINITY; m = -INFINITY; s = 0.f; idx = INT_MAX;
   }
-  // An element at or below the runner-up changes neither the top-1 nor the
-  // top-2, so the element-wise top-2 update runs only for groups whose
-  // maximum exceeds the runner-up (rare once the row's head is seen).
-  template <int K>
-  __device__ __forceinline__ void push(const float (&f)[K], int c) {
-    float vm = f[0];
-#pragma unroll
-    for (int i = 1; i < K; ++i) vm = fmaxf(vm, f[i]);
-    if (vm > second) {
-#pragma unroll
-      for (int i = 0; i < K; ++i) top2_push(f[i], c + i, best, second, idx);
-    }
-    lse_chunk_ex2<K>(f, best, m, s);
+  __device__ __forceinline__ void push(float x, int c) {
+    if (x > second) top2_push(x, c, best, second, idx);
+    const float f[1] = {x};
+    lse_chunk_ex2<1>(f, best, m, s);
   }
   __device__ __forceinline__ RowAcc acc() const {
     RowAcc r;
@@ -100,16 +93,15 @@ struct RowState {
   }
 };
 
-// Merge each row's RowAcc across the CTA; the results are valid in warp 0.
+// Merge each row's warp records (valid in lane 0) across the CTA; the results
+// are valid in warp 0.
 template <int R>
 __device__ __forceinline__ void block_reduce_rows(const RowAcc (&acc)[R], RowAcc (&out)[R]) {
   __shared__ RowAcc red[kRowsThreads / 32][R];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    RowAcc x = rowacc_warp_reduce(acc[r]);
-    if (lane == 0) red[warp][r] = x;
-  }
+  for (int r = 0; r < R; ++r)
+    if (lane == 0) red[warp][r] = acc[r];
   __syncthreads();
   if (warp == 0) {
 #pragma unroll
@@ -121,7 +113,12 @@ __device__ __forceinline__ void block_reduce_rows(const RowAcc (&acc)[R], RowAcc
 }
 
 // ----------------------------------------------------------------------------
-// fused combine: l = l_L + alpha l_S - beta l_P, then top-1/top-2/LSE per row
+// fused combine: l = l_L + alpha l_S - beta l_P, then top-1/top-2/LSE per row.
+// bf16 rows are close to issue-bound: 1024 rows of 151936 with both terms took
+// 126 us and 87 M warp instructions (17.9 per element) with a top-2 per thread,
+// whose update some lane of the warp needed for nearly every group, and tests
+// on every load; 106 us and 55 M (11.3) with the top-2 pruned by the warp's
+// runner-up (WarpRow) and a loop of whole blocks (115 us with the loop alone).
 // ----------------------------------------------------------------------------
 template <typename T, int R, bool VEC, bool SH, bool PR, bool FINAL>
 __global__ void __launch_bounds__(kRowsThreads, sizeof(T) == 2 ? 4 : 2) k_combine_rows(RowsArgs a) {
@@ -137,9 +134,15 @@ __global__ void __launch_bounds__(kRowsThreads, sizeof(T) == 2 ? 4 : 2) k_combin
   const T* S = SH ? static_cast<const T*>(a.shortp) + (long long)r0 * a.ld_short : nullptr;
   const float alpha = a.alpha, nbeta = -a.beta;
 
-  RowState st[R];
+  RowAcc acc[R], res[R];
+  // a last group's missing rows repeat its first (their results are not used)
+  const T* Lr[R];
+  const T* Sr[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) st[r].init();
+  for (int r = 0; r < R; ++r) {
+    Lr[r] = L + (long long)(r < nr ? r : 0) * a.ld_long;
+    Sr[r] = SH ? S + (long long)(r < nr ? r : 0) * a.ld_short : nullptr;
+  }
 
   if constexpr (VEC) {
     // Raw 16-byte words stay in registers until used: U groups of 8 values
@@ -150,89 +153,100 @@ __global__ void __launch_bounds__(kRowsThreads, sizeof(T) == 2 ? 4 : 2) k_combin
     constexpr int WPV = sizeof(T) == 2 ? 1 : 2;            // 16-byte words per 8 values
     constexpr int U = (R == 1) ? 4 : (R == 2 ? 2 : 1);
     const int step = kRowsThreads * 8;
-    for (int cb = c0 + threadIdx.x * 8; cb < c1; cb += step * U) {
+    // f32: the prior goes out with the logits; bf16: it is read where it
+    // is used (fewer registers: four CTAs per SM)
+    constexpr bool kPriorEarly = sizeof(T) == 4;
+    WarpRow st[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) st[r].init();
+    // columns cb + u * step, u < U, of every lane; CHECK: lanes past the
+    // chunk's end take -inf (its last, partial block; the others carry no tests)
+    auto block = [&](int cb, auto check) {
+      constexpr bool CHECK = decltype(check)::value;
+      constexpr uint32_t kNegInf = sizeof(T) == 2 ? 0xFF80FF80u : 0xFF800000u;
       uint4 lw[U][R][WPV];
       uint4 sw[U][R][WPV];
-      // f32: the prior goes out with the logits; bf16: it is read where it
-      // is used (fewer registers: four CTAs per SM)
-      constexpr bool kPriorEarly = sizeof(T) == 4;
       float4 pw[kPriorEarly ? U : 1][2];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int c = cb + u * step;
-        if (c < c1) {
-          if constexpr (PR && kPriorEarly) {
-            pw[u][0] = __ldg(reinterpret_cast<const float4*>(a.prior + c));
-            pw[u][1] = __ldg(reinterpret_cast<const float4*>(a.prior + c) + 1);
-          }
+        const bool in = !CHECK || c < c1;
+        if constexpr (PR && kPriorEarly) {
+          pw[u][0] = in ? __ldg(reinterpret_cast<const float4*>(a.prior + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          pw[u][1] = in ? __ldg(reinterpret_cast<const float4*>(a.prior + c) + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            if (r < nr) {
+        for (int r = 0; r < R; ++r) {
 #pragma unroll
-              for (int k = 0; k < WPV; ++k) {
-                lw[u][r][k] = __ldcs(reinterpret_cast<const uint4*>(L + (long long)r * a.ld_long + c) + k);
-                if constexpr (SH) sw[u][r][k] = __ldcs(reinterpret_cast<const uint4*>(S + (long long)r * a.ld_short + c) + k);
-              }
-            }
+          for (int k = 0; k < WPV; ++k) {
+            lw[u][r][k] = in ? __ldcs(reinterpret_cast<const uint4*>(Lr[r] + c) + k)
+                             : make_uint4(kNegInf, kNegInf, kNegInf, kNegInf);
+            if constexpr (SH)
+              sw[u][r][k] = in ? __ldcs(reinterpret_cast<const uint4*>(Sr[r] + c) + k) : make_uint4(0, 0, 0, 0);
           }
         }
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int c = cb + u * step;
-        if (c < c1) {
-          float pv[8];
-          if constexpr (PR) {
-            float4 p0, p1;
-            if constexpr (kPriorEarly) {
-              p0 = pw[u][0];
-              p1 = pw[u][1];
-            } else {
-              p0 = __ldg(reinterpret_cast<const float4*>(a.prior + c));
-              p1 = __ldg(reinterpret_cast<const float4*>(a.prior + c) + 1);
-            }
-            pv[0] = p0.x; pv[1] = p0.y; pv[2] = p0.z; pv[3] = p0.w;
-            pv[4] = p1.x; pv[5] = p1.y; pv[6] = p1.z; pv[7] = p1.w;
+        float pv[8];
+        if constexpr (PR) {
+          float4 p0, p1;
+          if constexpr (kPriorEarly) {
+            p0 = pw[u][0];
+            p1 = pw[u][1];
+          } else {
+            const int cp = !CHECK || c < c1 ? c : c0;   // a lane past the end reads any prior
+            p0 = __ldg(reinterpret_cast<const float4*>(a.prior + cp));
+            p1 = __ldg(reinterpret_cast<const float4*>(a.prior + cp) + 1);
           }
+          pv[0] = p0.x; pv[1] = p0.y; pv[2] = p0.z; pv[3] = p0.w;
+          pv[4] = p1.x; pv[5] = p1.y; pv[6] = p1.z; pv[7] = p1.w;
+        }
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            if (r < nr) {
-              float lv[8], sv[8];
-              unpack8<T, WPV>(lw[u][r], lv);
-              if constexpr (SH) unpack8<T, WPV>(sw[u][r], sv);
-              float f[8];
+        for (int r = 0; r < R; ++r) {
+          float lv[8], sv[8];
+          unpack8<T, WPV>(lw[u][r], lv);
+          if constexpr (SH) unpack8<T, WPV>(sw[u][r], sv);
+          float f[1][8];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                float x = lv[i];
-                if constexpr (SH) x = fmaf(alpha, sv[i], x);
-                if constexpr (PR) x = fmaf(nbeta, pv[i], x);
-                f[i] = x;
-              }
-              st[r].template push<8>(f, c);
-            }
+          for (int i = 0; i < 8; ++i) {
+            float x = lv[i];
+            if constexpr (SH) x = fmaf(alpha, sv[i], x);
+            if constexpr (PR) x = fmaf(nbeta, pv[i], x);
+            f[0][i] = x;
           }
+          const int at[1] = {c};
+          st[r].template push<1>(f, at);
         }
       }
-    }
+    };
+    // a warp's lanes leave together: the trip count follows its first column
+    const int lane8 = (threadIdx.x & 31) * 8;
+    int cw = c0 + (threadIdx.x >> 5) * 256;
+    const int full = c0 + (c1 - c0) / (step * U) * (step * U);
+    for (; cw < full; cw += step * U) block(cw + lane8, std::false_type{});
+    if (cw < c1) block(cw + lane8, std::true_type{});
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = st[r].record();
   } else {
+    RowState st[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) st[r].init();
     for (int c = c0 + threadIdx.x; c < c1; c += kRowsThreads) {
       const float p = PR ? __ldg(a.prior + c) : 0.f;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        if (r < nr) {
-          float x = load1(L + (long long)r * a.ld_long + c);
-          if constexpr (SH) x = fmaf(alpha, load1(S + (long long)r * a.ld_short + c), x);
-          if constexpr (PR) x = fmaf(nbeta, p, x);
-          float f[1] = {x};
-          st[r].template push<1>(f, c);
-        }
+        float x = load1(Lr[r] + c);
+        if constexpr (SH) x = fmaf(alpha, load1(Sr[r] + c), x);
+        if constexpr (PR) x = fmaf(nbeta, p, x);
+        st[r].push(x, c);
       }
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = rowacc_warp_reduce(st[r].acc());
   }
 
-  RowAcc acc[R], res[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = st[r].acc();
   block_reduce_rows<R>(acc, res);
 
   __shared__ int s_last;
