@@ -13,6 +13,7 @@
 //   p_n. q_a is rebuilt from the drafting's kept state: the fused row
 //   l_L + alpha_a W_vocab r_a - beta_a l_P and its LSE.
 #include <algorithm>
+#include <type_traits>
 
 #include "dels_device.cuh"
 
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(SampleRowsArgs a
 // their LSEs: CTA = (row, chunk of chunk_cols columns, a multiple of 8). A
 // pure stream of the rows: per element one fused multiply-add, one base-2
 // exponential and one addition beside the unpacking, and no top-2 state, which
-// the LSE does not need (64 x 17 bf16 rows of 151936: 61 us; the combine's row
+// the LSE does not need (64 x 17 bf16 rows of 151936: 58 us; the combine's row
 // kernel with no short logits and no prior, used before, 81 us).
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_rows(SampleRowsArgs a) {
@@ -132,20 +133,15 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
   const long long c0 = (long long)chunk * a.chunk_cols;
   const T* src = static_cast<const T*>(a.src) + row * a.ld + c0;
   const int cols = (int)min((long long)a.chunk_cols, a.V - c0);
-  float m = -INFINITY, s = 0.f;
-  // eight values, their maximum vm (NaN ignored)
+  float m = -INFINITY, s = 0.f, nb = 0.f;      // nb = -m log2(e), 0 while m is -inf
+  // Eight values with maximum vm (NaN ignored). While m is -inf they are -inf
+  // (0) or NaN (NaN).
   auto push = [&](const float (&x)[8], float vm) {
     if (vm > m) {
-      s *= ex2_approx((m - vm) * kLog2e);      // m == -inf: s is 0 or NaN
+      nb = -vm * kLog2e;
+      if (m != -INFINITY) s *= ex2_approx(fmaf(m, kLog2e, nb));
       m = vm;
     }
-    if (m == -INFINITY) {                      // nothing finite yet: only a NaN counts
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (x[i] != x[i]) s = NAN;
-      return;
-    }
-    const float nb = -m * kLog2e;
     float e[2] = {0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < 8; ++i) e[i & 1] += ex2_approx(fmaf(x[i], kLog2e, nb));
@@ -155,17 +151,19 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
     constexpr int W = sizeof(T) == 2 ? 1 : 2;  // 16-byte words per 8 values
     constexpr int U = 4;
     constexpr int step = kSampleThreads * 8;
-    for (int cb = threadIdx.x * 8; cb < cols; cb += step * U) {
+    // CHECK: the chunk's last, partial block (the others carry no tests)
+    auto block = [&](int cb, auto check) {
+      constexpr bool CHECK = decltype(check)::value;
       uint4 w[U][W];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (cb + u * step < cols) {
+        if (!CHECK || cb + u * step < cols) {
 #pragma unroll
           for (int k = 0; k < W; ++k) w[u][k] = __ldcs(reinterpret_cast<const uint4*>(src + cb + u * step) + k);
         }
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (cb + u * step < cols) {
+        if (!CHECK || cb + u * step < cols) {
           float x[8];
           if constexpr (W == 1) {
             x[0] = bf16lo(w[u][0].x); x[1] = bf16hi(w[u][0].x); x[2] = bf16lo(w[u][0].y); x[3] = bf16hi(w[u][0].y);
@@ -179,7 +177,11 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
           }
           push(x, max8(x));
         }
-    }
+    };
+    int cb = threadIdx.x * 8;
+    const int full = cols / (step * U) * (step * U);
+    for (; cb < full; cb += step * U) block(cb, std::false_type{});
+    if (cb < cols) block(cb, std::true_type{});
   } else {
     for (int c = threadIdx.x * 8; c < cols; c += 8 * kSampleThreads) {
       float x[8];
