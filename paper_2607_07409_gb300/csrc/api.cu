@@ -380,18 +380,22 @@ bool persistent_enabled() {
   return e && e[0] == '1';
 }
 
-// A store product over `rows` activation rows that may exceed one 128-row
-// tile (the transformer head's three-term rows, 3B): ceil(rows / 128)
-// launches over consecutive row blocks, all writing one partial buffer
-// [S][rows][O].
+// A store product over the `rows` = terms x B activation rows of three-term
+// expansions, which may exceed one 128-row tile: ceil(rows / 128) launches over
+// consecutive row blocks, all writing one partial buffer [S][rows][O]. Where
+// the rows fit one TMEM quadrant (B <= 10) the epilogue adds the terms up and
+// the buffer is [S][B][O]: a third of the partials to write and read back.
 struct RowBlocks {
   Gemm g[3];
   int count = 0;
+  int terms = 1;   // terms left in the partials
 };
 
-bool plan_store_rows(RowBlocks& rb, int rows, int O, const uint16_t* X, const void* W, int K, int splits,
+bool plan_store_rows(RowBlocks& rb, int B, int terms, int O, const uint16_t* X, const void* W, int K, int splits,
                      float* part, int* status, int sms) {
+  const int rows = terms * B;
   rb.count = 0;
+  rb.terms = rows <= 32 ? 1 : terms;
   for (int r0 = 0; r0 < rows; r0 += kMaxBatchTile) {
     if (rb.count >= 3) return false;
     const int m = std::min(kMaxBatchTile, rows - r0);
@@ -399,7 +403,8 @@ bool plan_store_rows(RowBlocks& rb, int rows, int O, const uint16_t* X, const vo
     if (!plan_store(g, m, O, X + (size_t)r0 * K, W, K, nullptr, nullptr, 0, 128, splits, 0, ACT_NONE,
                     part + (size_t)r0 * O, nullptr, 0, status, sms))
       return false;
-    g.a.out_split_stride = (long long)rows * O;
+    g.a.sum_terms = rb.terms == 1 ? terms : 1;
+    g.a.out_split_stride = (long long)rb.terms * B * O;
   }
   return rb.count > 0;
 }
@@ -450,7 +455,7 @@ struct DraftLayout {
   size_t u = 0, mpart = 0, h1 = 0, h2 = 0;
   int mlp_s1 = 0, mlp_s2 = 0;
   // XFMR
-  size_t ex = 0, t = 0, ab = 0, q = 0, kc = 0, vc = 0, xpart = 0, wqkv = 0, xpqkv = 0, ob = 0, uu = 0, anb = 0, fb = 0,
+  size_t ex = 0, t = 0, ab = 0, kc = 0, vc = 0, xpart = 0, wqkv = 0, xpqkv = 0, ob = 0, uu = 0, anb = 0, fb = 0,
          y = 0, feat = 0;
   int xs_qkv = 0, xs_o = 0, xs_1 = 0, xs_2 = 0;
   // MARKOV
@@ -507,7 +512,6 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
       L.ex = c.take((size_t)B * D * 2);
       L.t = c.take((size_t)B * D * 4);
       L.ab = c.take((size_t)T * B * D * 2);
-      L.q = c.take((size_t)B * D * 4);
       L.kc = c.take((size_t)B * P * D * 4);
       L.vc = c.take((size_t)B * P * D * 4);
       L.xs_qkv = splits_balanced(3 * D, 128, D, sms);
@@ -601,7 +605,7 @@ int validate_head(const dels_local_head* h, int n) {
         if (!h->w[i]) return DELS_ERR_NULL_POINTER;
       if (!dim_ok(h->d_model) || !dim_ok(h->d_hidden) || h->d_rank != h->d_model) return DELS_ERR_BAD_SHAPE;
       if (h->n_heads < 1 || h->d_model % h->n_heads != 0 || h->max_pos < n) return DELS_ERR_BAD_SHAPE;
-      if (h->d_model / h->n_heads > 8192) return DELS_ERR_UNSUPPORTED;   // q of one head in shared memory
+      if (h->d_model / h->n_heads > 8192) return DELS_ERR_UNSUPPORTED;   // q, k, v of one head in shared memory
       if (h->d_model > 32768) return DELS_ERR_UNSUPPORTED;               // RMSNorm rows: 8 CTAs x 4096 values
       return DELS_OK;
     case DELS_HEAD_MARKOV:
@@ -1694,7 +1698,6 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       uint16_t* ex = at<uint16_t>(workspace, L.ex);
       float* t = at<float>(workspace, L.t);
       uint16_t* ab = at<uint16_t>(workspace, L.ab);
-      float* q = at<float>(workspace, L.q);
       float* kc = at<float>(workspace, L.kc);
       float* vc = at<float>(workspace, L.vc);
       float* xpart = at<float>(workspace, L.xpart);
@@ -1722,10 +1725,10 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       constexpr int T = kXfmrTerms;
       RowBlocks gqkv, go, g1, g2;
       Gemm gv;
-      bool ok = plan_store_rows(gqkv, T * B, 3 * D, ab, wqkv, D, L.xs_qkv, xpqkv, status, sms) &&
-                plan_store_rows(go, T * B, D, ob, head->w[4], D, L.xs_o, xpart, status, sms) &&
-                plan_store_rows(g1, T * B, F, anb, head->w[5], D, L.xs_1, xpart, status, sms) &&
-                plan_store_rows(g2, T * B, D, fb, head->w[6], F, L.xs_2, xpart, status, sms) &&
+      bool ok = plan_store_rows(gqkv, B, T, 3 * D, ab, wqkv, D, L.xs_qkv, xpqkv, status, sms) &&
+                plan_store_rows(go, B, T, D, ob, head->w[4], D, L.xs_o, xpart, status, sms) &&
+                plan_store_rows(g1, B, T, F, anb, head->w[5], D, L.xs_1, xpart, status, sms) &&
+                plan_store_rows(g2, B, T, D, fb, head->w[6], F, L.xs_2, xpart, status, sms) &&
                 plan_combine(gv, B, V, n, feat, D, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
                              partials, L.partial_ld, status, sms, true);
       if (!ok) return DELS_ERR_CUDA;
@@ -1736,22 +1739,13 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         const int p = j - 1;   // position of the newest drafted token x_{j-1}
         { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_xfmr_embed(ex, pos, p, B, D, t, ab, s, T)); }
         { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rows(gqkv, s)); }
-        {
-          // q, and the k / v cache rows of position p, from the stacked partials
-          SplitkJobs3 jq{};
-          jq.j[0] = SplitkJob{xpqkv, Sqkv, 0, q, (long long)D};
-          jq.j[1] = SplitkJob{xpqkv, Sqkv, D, kc + (size_t)p * D, (long long)P * D};
-          jq.j[2] = SplitkJob{xpqkv, Sqkv, 2 * D, vc + (size_t)p * D, (long long)P * D};
-          PROF(DELS_KCLASS_HEAD_MISC);
-          DELS_CUDA(launch_splitk_finish3(jq, 3, B, D, 3 * D, T, s));
-        }
-        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_attention(q, kc, vc, B, D, NH, p + 1, P, ob, s, T)); }
+        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_attention(xpqkv, Sqkv, gqkv.terms, kc, vc, B, D, NH, p + 1, P, ob, s, T)); }
         { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rows(go, s)); }
-        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_finish_rmsnorm(xpart, So, T, B, D, t, uu, anb, T, s)); }
+        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_finish_rmsnorm(xpart, So, go.terms, B, D, t, uu, anb, T, s)); }
         { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rows(g1, s)); }
-        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_splitk_finish(xpart, S1, B, F, nullptr, ACT_GELU, nullptr, 0, fb, F, s, T, T)); }
+        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_splitk_finish(xpart, S1, B, F, nullptr, ACT_GELU, nullptr, 0, fb, F, s, g1.terms, T)); }
         { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rows(g2, s)); }
-        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_finish_rmsnorm(xpart, S2, T, B, D, uu, y, feat, 1, s)); }
+        { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_finish_rmsnorm(xpart, S2, g2.terms, B, D, uu, y, feat, 1, s)); }
         gv.a.j = j;
           gv.a.sample = sm.on;
           gv.a.seed = sm.seed;

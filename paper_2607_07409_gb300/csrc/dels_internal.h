@@ -204,6 +204,8 @@ struct TcGemmArgs {
   int seg_chunks[2];             // K chunks of 64 per segment
   int seg_splits[2];             // K splits per segment (0 splits: unused segment)
   int seg_per[2];                // K chunks per split (the last may have fewer)
+  int sum_terms;                 // EPI_STORE f32 rows: 3: the B rows are three groups of B / 3, stored as the sum of
+                                 // the groups (all in one TMEM quadrant: B <= 32); otherwise stored as they are
   int total_splits;
   int epi;
   int a_resident;                // A (activations) loaded once per CTA
@@ -334,21 +336,6 @@ cudaError_t launch_splitk_finish(const float* part, int S, int B, int O, const f
                                  float* out_f32, int ld_f32, uint16_t* out_bf16, int ld_bf16, cudaStream_t s,
                                  int in_terms = 1, int out_terms = 1);
 cudaError_t launch_rmsnorm_bf16(const float* x, int B, int D, int ld, uint16_t* out, cudaStream_t s, int terms = 1);
-// Up to three split-K reductions (float32 outputs, own row pitches) in one
-// launch: job k sums columns col0 .. col0 + O - 1 of partials
-// [S][in_terms * B][ldp].
-struct SplitkJob {
-  const float* part;
-  int S;
-  int col0;
-  float* out;          // row b at out + b * ld
-  long long ld;
-};
-struct SplitkJobs3 {
-  SplitkJob j[3];
-};
-cudaError_t launch_splitk_finish3(const SplitkJobs3& jobs, int njobs, int B, int O, int ldp, int in_terms,
-                                  cudaStream_t s);
 // Split-K reduction + residual (out_f32) and RMSNorm of each row as `terms`
 // bf16 terms (norm_bf16, row pitch D); a cluster of kNormCluster CTAs per row.
 constexpr int kNormCluster = 8;
@@ -356,7 +343,7 @@ cudaError_t launch_finish_rmsnorm(const float* part, int S, int in_terms, int B,
                                   float* out_f32, uint16_t* norm_bf16, int terms, cudaStream_t s);
 cudaError_t launch_xfmr_embed(const uint16_t* e_rows, const uint16_t* pos_table, int pos, int B, int D,
                               float* t_out, uint16_t* a_bf16, cudaStream_t s, int terms = 1);
-cudaError_t launch_attention(const float* q, const float* kcache, const float* vcache, int B, int D, int nh,
+cudaError_t launch_attention(const float* part, int S, int in_terms, float* kcache, float* vcache, int B, int D, int nh,
                              int npos, int cache_ld_pos, uint16_t* o_bf16, cudaStream_t s, int terms = 1);
 // bf16 weights and activations, bf16 output after the activation, B <= kGemvBf16MaxRows.
 constexpr int kGemvBf16MaxRows = 4;

@@ -229,25 +229,6 @@ __global__ void k_splitk_finish(const float* __restrict__ part, int S, int B, in
   }
 }
 
-// Up to three split-K reductions in one launch (blockIdx.y = job): the same
-// sum as k_splitk_finish with in_terms-term partials of row pitch ldp (job k
-// reads columns col0 .. col0 + O - 1), no residual, no activation, float32
-// output with its own row pitch (the transformer head's q, k and v of the
-// newest position, from the partials of their stacked product).
-__global__ void k_splitk_finish3(SplitkJobs3 jobs, int B, int O, int ldp, int in_terms) {
-  if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
-  const SplitkJob& jb = jobs.j[blockIdx.y];
-  const long long total = (long long)B * O;
-  const long long term_stride = (long long)B * ldp;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(e / O), o = (int)(e % O);
-    jb.out[(long long)b * jb.ld + o] =
-        splitk_sum(jb.part, jb.S, in_terms, term_stride, (long long)b * ldp + jb.col0 + o);
-  }
-}
-
 // out = RMSNorm(x) = x / sqrt(mean(x^2) + 1e-6) as `terms` bf16 terms (rows
 // of pitch ld, see store_bf16_terms); one CTA per row.
 __global__ void k_rmsnorm_bf16(const float* __restrict__ x, int D, int ld, uint16_t* __restrict__ out, int terms,
@@ -358,60 +339,83 @@ __global__ void k_xfmr_embed(const uint16_t* __restrict__ e_rows, const uint16_t
 }
 
 // Causal attention of the newest position over positions 0..npos-1 of the
-// block: one CTA per (row, head); o = softmax(q k^T / sqrt(dh)) v, stored as
-// `terms` bf16 terms. q is staged in shared memory; one warp per position
-// computes a score with four loads of the key in flight; each output element
-// sums over the positions four values at a time.
-__global__ void k_attention(const float* __restrict__ q, const float* __restrict__ kc, const float* __restrict__ vc,
-                            int D, int nh, int npos, int cache_ld_pos, uint16_t* __restrict__ o_bf16, int terms,
-                            int B) {
-  extern __shared__ float sq[];   // dh
-  __shared__ float w[64];
+// block, one CTA per (row, head): the newest position's q, k and v from the
+// split-K partials of their stacked product (as k_splitk_finish, row pitch
+// 3 D), k and v into the caches, o = softmax(q k^T / sqrt(dh)) v, stored as
+// `terms` bf16 terms. Latency-bound: the older positions' values of up to 16
+// positions are loaded together with the partials, one warp per position
+// computes a score and every warp takes the softmax, a lane per position (8
+// rows, 8 heads of 320, block of 16: the block 3136 -> 2985 us with this and
+// the terms summed in the products' epilogue, 2970 with the reduction folded
+// in, which was a launch of its own; under ncu 7.9 us where the two took 16).
+__global__ void __launch_bounds__(1024) k_attention(const float* __restrict__ part, int S, int in_terms, float* kc,
+                                                   float* vc, int D, int nh, int npos, int cache_ld_pos,
+                                                   uint16_t* __restrict__ o_bf16, int terms, int B) {
+  extern __shared__ float sq[];   // q, k, v of the newest position: [3][dh]
+  __shared__ float w[32];
+  constexpr int kV = 16;   // positions whose values a thread keeps in flight
   if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x / nh, hd = blockIdx.x % nh;
   const int dh = D / nh;
   const float scale = rsqrtf((float)dh);
-  for (int i = threadIdx.x; i < dh; i += blockDim.x) sq[i] = q[(long long)b * D + hd * dh + i];
-  __syncthreads();
+  const long long row0 = (long long)b * cache_ld_pos * D + hd * dh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int last = npos - 1;
+  // the first output element's older values go out first
+  float v[kV];
+  const int i0 = threadIdx.x;
+#pragma unroll
+  for (int p = 0; p < kV; ++p) v[p] = i0 < dh && p < last ? __ldcg(vc + row0 + (long long)p * D + i0) : 0.f;
+  for (int i = threadIdx.x; i < 3 * dh; i += blockDim.x) {
+    const int c = i / dh, k = i - c * dh;
+    const float x = splitk_sum(part, S, in_terms, (long long)B * 3 * D, (long long)b * 3 * D + c * D + hd * dh + k);
+    sq[i] = x;
+    if (c == 1) kc[row0 + (long long)last * D + k] = x;
+    if (c == 2) vc[row0 + (long long)last * D + k] = x;
+  }
+  __syncthreads();
   for (int p = warp; p < npos; p += nw) {
-    const float* kv = kc + ((long long)b * cache_ld_pos + p) * D + hd * dh;
+    const float* kv = p == last ? sq + dh : kc + row0 + (long long)p * D;
     float d[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int i0 = lane; i0 < dh; i0 += 128) {
+    for (int i = lane; i < dh; i += 128) {
       float k4[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) k4[u] = i0 + 32 * u < dh ? kv[i0 + 32 * u] : 0.f;
+      for (int u = 0; u < 4; ++u) k4[u] = i + 32 * u < dh ? kv[i + 32 * u] : 0.f;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (i0 + 32 * u < dh) d[u] = fmaf(sq[i0 + 32 * u], k4[u], d[u]);
+        if (i + 32 * u < dh) d[u] = fmaf(sq[i + 32 * u], k4[u], d[u]);
     }
     float dd = (d[0] + d[1]) + (d[2] + d[3]);
 #pragma unroll
-    for (int k = 16; k > 0; k >>= 1) dd += __shfl_down_sync(0xFFFFFFFFu, dd, k);
+    for (int k = 16; k > 0; k >>= 1) dd += __shfl_xor_sync(0xFFFFFFFFu, dd, k);
     if (lane == 0) w[p] = dd * scale;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float m = -INFINITY;
-    for (int p = 0; p < npos; ++p) m = fmaxf(m, w[p]);
-    float s = 0.f;
-    for (int p = 0; p < npos; ++p) { w[p] = __expf(w[p] - m); s += w[p]; }
-    for (int p = 0; p < npos; ++p) w[p] /= s;
-  }
+  // softmax: lane p holds position p's score (npos <= 32)
+  const float x = lane < npos ? w[lane] : -INFINITY;
+  float m = x;
+#pragma unroll
+  for (int k = 16; k > 0; k >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, k));
+  const float e = lane < npos ? __expf(x - m) : 0.f;
+  float s = e;
+#pragma unroll
+  for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, k);
   __syncthreads();
-  const long long row0 = (long long)b * cache_ld_pos * D + hd * dh;
-  for (int i = threadIdx.x; i < dh; i += blockDim.x) {
+  if (warp == 0 && lane < npos) w[lane] = e / s;
+  __syncthreads();
+  for (int i = i0; i < dh; i += blockDim.x) {
     float o[4] = {0.f, 0.f, 0.f, 0.f};
-    int p = 0;
-    for (; p + 4 <= npos; p += 4) {
-      float v4[4];
+    for (int p0 = 0; p0 < last; p0 += kV) {
+      if (i != i0 || p0 > 0) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v4[u] = vc[row0 + (long long)(p + u) * D + i];
+        for (int p = 0; p < kV; ++p) v[p] = p0 + p < last ? __ldcg(vc + row0 + (long long)(p0 + p) * D + i) : 0.f;
+      }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) o[u] = fmaf(w[p + u], v4[u], o[u]);
+      for (int p = 0; p < kV; ++p)
+        if (p0 + p < last) o[p & 3] = fmaf(w[p0 + p], v[p], o[p & 3]);
     }
-    for (; p < npos; ++p) o[0] = fmaf(w[p], vc[row0 + (long long)p * D + i], o[0]);
+    o[last & 3] = fmaf(w[last], sq[2 * dh + i], o[last & 3]);
     store_bf16_terms(o_bf16, terms, B, b, D, hd * dh + i, (o[0] + o[1]) + (o[2] + o[3]));
   }
 }
@@ -516,13 +520,6 @@ cudaError_t launch_splitk_finish(const float* part, int S, int B, int O, const f
                     act, out_f32, ld_f32, out_bf16, ld_bf16, in_terms, out_terms);
 }
 
-cudaError_t launch_splitk_finish3(const SplitkJobs3& jobs, int njobs, int B, int O, int ldp, int in_terms,
-                                  cudaStream_t s) {
-  if (njobs < 1 || njobs > 3) return cudaErrorInvalidValue;
-  return launch_pdl(k_splitk_finish3, dim3(grid_for((long long)B * O, 256), njobs), dim3(256), 0, s, jobs, B, O, ldp,
-                    in_terms);
-}
-
 cudaError_t launch_finish_rmsnorm(const float* part, int S, int in_terms, int B, int D, const float* residual,
                                   float* out_f32, uint16_t* norm_bf16, int terms, cudaStream_t s) {
   const int per = (D + kNormCluster - 1) / kNormCluster;
@@ -542,11 +539,15 @@ cudaError_t launch_xfmr_embed(const uint16_t* e_rows, const uint16_t* pos_table,
   return launch_pdl(k_xfmr_embed, dim3(B), dim3(256), 0, s, e_rows, pos_table, pos, D, t_out, a_bf16, terms, B);
 }
 
-cudaError_t launch_attention(const float* q, const float* kcache, const float* vcache, int B, int D, int nh,
+cudaError_t launch_attention(const float* part, int S, int in_terms, float* kcache, float* vcache, int B, int D, int nh,
                              int npos, int cache_ld_pos, uint16_t* o_bf16, cudaStream_t s, int terms) {
-  if (npos < 1 || npos > 64) return cudaErrorInvalidValue;
-  const int dh = D / nh;
-  return launch_pdl(k_attention, dim3(B * nh), dim3(256), (size_t)dh * 4, s, q, kcache, vcache, D, nh, npos,
+  if (npos < 1 || npos > 32) return cudaErrorInvalidValue;
+  const size_t smem = (size_t)3 * (D / nh) * 4;
+  // a thread per reduced element, as far as a CTA goes
+  const int threads = std::min(1024, std::max(256, (3 * (D / nh) + 31) / 32 * 32));
+  const cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(k_attention), smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_attention, dim3(B * nh), dim3(threads), smem, s, part, S, in_terms, kcache, vcache, D, nh, npos,
                     cache_ld_pos, o_bf16, terms, B);
 }
 

@@ -593,10 +593,20 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
           for (int i = 0; i < 32; ++i) tr[lane * 33 + i] = acc[i];
           __syncwarp();
           const int r0 = b - lane;
-          const int rows = min(32, a.B - r0);
           float* dst = a.out_f32 + (long long)it.split * a.out_split_stride + cbase + lane;
-          if (cbase + lane < a.O)
-            for (int r = 0; r < rows; ++r) dst[(long long)(r0 + r) * a.ldo] = tr[r * 33 + lane];
+          if (cbase + lane < a.O) {
+            if (a.sum_terms == 3) {
+              // the three terms of an expansion, the smallest first
+              const int rows = a.B / 3;
+#pragma unroll 5
+              for (int r = 0; r < rows; ++r)
+                dst[(long long)r * a.ldo] =
+                    (tr[(2 * rows + r) * 33 + lane] + tr[(rows + r) * 33 + lane]) + tr[r * 33 + lane];
+            } else {
+              const int rows = min(32, a.B - r0);
+              for (int r = 0; r < rows; ++r) dst[(long long)(r0 + r) * a.ldo] = tr[r * 33 + lane];
+            }
+          }
           __syncwarp();
         } else if (b < a.B) {
           if (a.out_f32 && a.out_bmajor) {
