@@ -146,22 +146,6 @@ __device__ __forceinline__ RowAcc rowacc_merge(const RowAcc& a, const RowAcc& b)
   return r;
 }
 
-__device__ __forceinline__ RowAcc rowacc_shfl_down(const RowAcc& a, int delta) {
-  RowAcc r;
-  r.m = __shfl_down_sync(0xFFFFFFFFu, a.m, delta);
-  r.s = __shfl_down_sync(0xFFFFFFFFu, a.s, delta);
-  r.second = __shfl_down_sync(0xFFFFFFFFu, a.second, delta);
-  r.idx = __shfl_down_sync(0xFFFFFFFFu, a.idx, delta);
-  return r;
-}
-
-// Warp-level merge in a fixed tree order; lane 0 holds the result.
-__device__ __forceinline__ RowAcc rowacc_warp_reduce(RowAcc a) {
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) a = rowacc_merge(a, rowacc_shfl_down(a, d));
-  return a;
-}
-
 // Floats as integers of the same order (no NaN), for integer maxima.
 __device__ __forceinline__ int ordered_bits(float x) {
   const int i = __float_as_int(x);
@@ -171,6 +155,50 @@ __device__ __forceinline__ float from_ordered_bits(int i) { return __int_as_floa
 // Largest x of a whole warp (no NaN).
 __device__ __forceinline__ float warp_max(float x) {
   return from_ordered_bits(__reduce_max_sync(0xFFFFFFFFu, ordered_bits(x)));
+}
+
+// A record's sum of exponentials relative to a maximum M >= its own; a NaN
+// stays one.
+__device__ __forceinline__ float rowacc_scaled(float m, float s, float M) {
+  return m == -INFINITY ? (s != s ? NAN : 0.f) : s * ex2_approx((m - M) * kLog2e);
+}
+
+// N records of one lane (x: max, y: sum, z: runner-up, w: index) merged: the
+// maximum first, then every sum scaled at once, where a chain of rowacc_merge
+// would wait for one pair of exponentials after another.
+template <int N>
+__device__ __forceinline__ RowAcc rowacc_merge_many(const float4 (&v)[N]) {
+  RowAcc r;
+  r.m = v[0].x;
+#pragma unroll
+  for (int i = 1; i < N; ++i) r.m = fmaxf(r.m, v[i].x);
+  r.idx = 0x7FFFFFFF;
+  r.s = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    r.idx = v[i].x == r.m ? min(r.idx, __float_as_int(v[i].w)) : r.idx;
+    r.s += rowacc_scaled(v[i].x, v[i].y, r.m);
+  }
+  r.second = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    r.second = fmaxf(r.second, v[i].x == r.m && __float_as_int(v[i].w) == r.idx ? v[i].z : v[i].x);
+  return r;
+}
+
+// Warp-level merge (all lanes converged), the result in every lane: three
+// integer reductions and one sum, in a fixed order. (A tree of five
+// rowacc_merge steps, each with its shuffles and exponentials in line, took
+// about three times as long.)
+__device__ __forceinline__ RowAcc rowacc_warp_reduce(const RowAcc& a) {
+  RowAcc r;
+  r.m = warp_max(a.m);
+  r.idx = __reduce_min_sync(0xFFFFFFFFu, a.m == r.m ? a.idx : 0x7FFFFFFF);
+  r.second = warp_max(a.m == r.m && a.idx == r.idx ? a.second : a.m);
+  r.s = rowacc_scaled(a.m, a.s, r.m);
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) r.s += __shfl_xor_sync(0xFFFFFFFFu, r.s, d);
+  return r;
 }
 
 // One row scanned by a whole warp, all lanes together: each lane keeps the

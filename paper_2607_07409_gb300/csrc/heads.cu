@@ -118,12 +118,8 @@ __global__ void __launch_bounds__(kGatesThreads) k_gru_gates_table(GatesTableArg
         const int k = k0 + u * 32 + lane;
         v[u] = k < a.count ? __ldcg(rec + k) : make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(INT_MAX));
       }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        RowAcc y;
-        y.m = v[u].x; y.s = v[u].y; y.second = v[u].z; y.idx = __float_as_int(v[u].w);
-        x = rowacc_merge(x, y);
-      }
+      const RowAcc y = rowacc_merge_many<8>(v);
+      x = k0 == 0 ? y : rowacc_merge(x, y);
     }
     x = rowacc_warp_reduce(x);
     if (lane == 0) {

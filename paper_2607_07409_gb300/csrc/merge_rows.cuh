@@ -16,19 +16,7 @@ __device__ __forceinline__ void merge_requests(const MergeArgs& m, int b0, int n
     const int b = b0 + q;
     const float4* rec = reinterpret_cast<const float4*>(m.partials) + (long long)b * m.partial_ld;
     RowAcc x = rowacc_init();
-    for (int k0 = lane; k0 < m.count; k0 += 4 * 32) {   // four records in flight
-      float4 v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (k0 + u * 32 < m.count) v[u] = __ldcg(rec + k0 + u * 32);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (k0 + u * 32 < m.count) {
-          RowAcc y;
-          y.m = v[u].x; y.s = v[u].y; y.second = v[u].z; y.idx = __float_as_int(v[u].w);
-          x = rowacc_merge(x, y);
-        }
-    }
+    for (int k = lane; k < m.count; k += 32) x = rowacc_merge(x, ld_rowacc_cg(rec, k));   // mostly one
     x = rowacc_warp_reduce(x);
     if (lane == 0) {
       s_tok[q] = (m.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
