@@ -668,9 +668,12 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
     }
     named_bar_sync<1>(kEpiWarps * 32);
     if (worker == 0 && quad_live && b < a.B && !*c.abort_flag) {
-      RowAcc r = rowacc_init();
-      if (p.count > 0)
-        for (int w = 0; w < workers; ++w) r = rowacc_merge(r, c.red[w * rpc + b]);
+      const float4 none = make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(0x7FFFFFFF));
+      float4 v[8];   // workers: 2, 4 or 8
+#pragma unroll
+      for (int w = 0; w < 8; ++w)
+        v[w] = w < workers && p.count > 0 ? *reinterpret_cast<const float4*>(&c.red[w * rpc + b]) : none;
+      const RowAcc r = rowacc_merge_many<8>(v);
       reinterpret_cast<float4*>(a.partials)[(long long)b * a.partial_ld + cta] =
           make_float4(r.m, r.s, r.second, __int_as_float(r.idx));
     }
