@@ -294,17 +294,13 @@ __device__ __forceinline__ ArgAcc argacc_merge(const ArgAcc& a, const ArgAcc& b)
   r.nan = a.nan | b.nan;
   return r;
 }
-__device__ __forceinline__ ArgAcc argacc_shfl_down(const ArgAcc& a, int d) {
+// All lanes converged; the result in every lane.
+__device__ __forceinline__ ArgAcc argacc_warp_reduce(const ArgAcc& a) {
   ArgAcc r;
-  r.best = __shfl_down_sync(0xFFFFFFFFu, a.best, d);
-  r.idx = __shfl_down_sync(0xFFFFFFFFu, a.idx, d);
-  r.nan = __shfl_down_sync(0xFFFFFFFFu, a.nan, d);
+  r.best = warp_max(a.best);
+  r.idx = __reduce_min_sync(0xFFFFFFFFu, a.best == r.best ? a.idx : INT_MAX);
+  r.nan = __any_sync(0xFFFFFFFFu, a.nan);
   return r;
-}
-__device__ __forceinline__ ArgAcc argacc_warp_reduce(ArgAcc a) {
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) a = argacc_merge(a, argacc_shfl_down(a, d));
-  return a;
 }
 
 template <typename T, bool VEC>
