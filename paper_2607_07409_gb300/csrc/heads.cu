@@ -108,8 +108,8 @@ __global__ void __launch_bounds__(kGatesThreads) k_gru_gates_table(GatesTableArg
   }
   // merge of request b's records: warp 0 alone, every record load in flight at once
   __shared__ int s_tok;
+  RowAcc x = rowacc_init();
   if (warp == 0) {
-    RowAcc x = rowacc_init();
     const float4* rec = reinterpret_cast<const float4*>(a.partials) + (long long)b * a.partial_ld;
     for (int k0 = 0; k0 < a.count; k0 += 8 * 32) {
       float4 v[8];
@@ -122,21 +122,21 @@ __global__ void __launch_bounds__(kGatesThreads) k_gru_gates_table(GatesTableArg
       x = k0 == 0 ? y : rowacc_merge(x, y);
     }
     x = rowacc_warp_reduce(x);
-    if (lane == 0) {
-      if (!a.smp.on) {
-        s_tok = rowacc_valid(x) ? x.idx : -1;
-        if (blockIdx.y == 0) write_decode(x, (long long)b * a.n + a.jprev, a.tokens, a.out_lp, a.out_gap, a.status);
-      } else if (blockIdx.y == 0) {
-        s_tok = decode_record(x, a.smp, b, a.n, a.jprev, a.tokens, a.out_lp, a.out_gap, a.status);
-      } else {
-        s_tok = rowacc_valid_sampled(x) ? x.idx : -1;
-      }
-    }
+    if (lane == 0) s_tok = (a.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
   }
-  // temperature 1: keep r_{jprev} (not yet overwritten: the next products launch follows this one)
-  if (blockIdx.y == 0) keep_draft_input(a.smp, b, a.n, a.jprev);
   __syncthreads();
-  if (!live) return;
+  // the outputs are written last, off the path to the new state
+  auto outputs = [&] {
+    if (blockIdx.y != 0) return;
+    if (threadIdx.x == 0)
+      decode_record(x, a.smp, b, a.n, a.jprev, a.tokens, a.out_lp, a.out_gap, a.status);
+    // temperature 1: keep r_{jprev} (not yet overwritten: the next products launch follows this one)
+    keep_draft_input(a.smp, b, a.n, a.jprev);
+  };
+  if (!live) {
+    outputs();
+    return;
+  }
   const int tok = s_tok;
   float gir = 0.f, giz = 0.f, gin = 0.f;
   if (tok >= 0 && tok < a.V) {
@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(kGatesThreads) k_gru_gates_table(GatesTableArg
   const long long e = (long long)b * H + i;
   a.h[e] = hn;
   a.h_bf16[e] = f32_to_bf16_rne(hn);
+  outputs();
 }
 
 // sum_s sum_t part[s * split_stride + t * total + e] over S splits and

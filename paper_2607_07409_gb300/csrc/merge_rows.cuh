@@ -8,22 +8,21 @@
 
 namespace dels {
 
-// Tokens of requests b0 .. b0 + nb - 1 at position m.j into s_tok (valid after
-// the __syncthreads that ends the call).
+// Tokens of requests b0 .. b0 + nb - 1 (at most one per warp) at position m.j
+// into s_tok; the writer's outputs follow the barrier, off the other warps' path.
 __device__ __forceinline__ void merge_requests(const MergeArgs& m, int b0, int nb, bool writer, int* s_tok) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int q = warp; q < nb; q += nw) {
-    const int b = b0 + q;
-    const float4* rec = reinterpret_cast<const float4*>(m.partials) + (long long)b * m.partial_ld;
-    RowAcc x = rowacc_init();
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+  RowAcc x = rowacc_init();
+  if (q < nb) {
+    const float4* rec = reinterpret_cast<const float4*>(m.partials) + (long long)(b0 + q) * m.partial_ld;
     for (int k = lane; k < m.count; k += 32) x = rowacc_merge(x, ld_rowacc_cg(rec, k));   // mostly one
+    __syncwarp();
     x = rowacc_warp_reduce(x);
-    if (lane == 0) {
-      s_tok[q] = (m.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
-      if (writer) decode_record(x, m.smp, b, m.n, m.j, m.tokens, m.out_lp, m.out_gap, m.status);
-    }
+    if (lane == 0) s_tok[q] = (m.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
   }
   __syncthreads();
+  if (writer && q < nb && lane == 0)
+    decode_record(x, m.smp, b0 + q, m.n, m.j, m.tokens, m.out_lp, m.out_gap, m.status);
 }
 
 // 16-byte vector v of request b0 + q's head input (the embedding rows of its

@@ -457,9 +457,11 @@ __global__ void __launch_bounds__(256) k_draft_merge(MergeArgs a) {
   if (warp == 0) {
     x = lane < (int)(blockDim.x >> 5) ? red[lane] : rowacc_init();
     x = rowacc_warp_reduce(x);
-    if (lane == 0) s_tok = decode_record(x, a.smp, b, a.n, a.j, a.tokens, a.out_lp, a.out_gap, a.status);
+    if (lane == 0) s_tok = (a.smp.on ? rowacc_valid_sampled(x) : rowacc_valid(x)) ? x.idx : -1;
   }
   __syncthreads();
+  // the outputs are written while the other threads gather
+  if (warp == 0 && lane == 0) decode_record(x, a.smp, b, a.n, a.j, a.tokens, a.out_lp, a.out_gap, a.status);
   if (a.table == nullptr) return;
   const int es = a.table_f32 ? 4 : 2;
   const int vec_per_row = a.D * es / 16;                 // D * es is a multiple of 16
