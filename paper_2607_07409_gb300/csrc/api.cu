@@ -1585,6 +1585,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         const float* Wr = static_cast<const float*>(head->w[2]);
         float* feat = static_cast<float*>(rr);
         GemvF32Jobs gates{}, rank{};
+        gates.late = rank.late = mb.late = !fused;   // (few records: small calls)
         gates.j[0] = GemvF32Job{E, Wih, gpart, D, D};
         gates.j[1] = GemvF32Job{h, Whh, gpart + (size_t)B * 3 * H, H, H};
         rank.j[0] = GemvF32Job{h, Wr, feat, H, H};
@@ -1674,6 +1675,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         }
       } else {
         GemvF32Jobs l1{}, l2{};
+        l1.late = l2.late = mb.late = !fused;
         l1.j[0] = GemvF32Job{static_cast<const float*>(u), static_cast<const float*>(head->w[0]),
                              static_cast<float*>(h1), K1, K1};
         l2.j[0] = GemvF32Job{static_cast<const float*>(h1), static_cast<const float*>(head->w[1]),

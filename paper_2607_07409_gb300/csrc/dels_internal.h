@@ -188,6 +188,7 @@ struct MergeArgs {
   int table_f32;
   int D, window;
   void* dest;                    // [B, window*D] same dtype as table
+  int late;                      // let the next launch start after the wait for this one's predecessor, not at once
   SampleArgs smp;
 };
 cudaError_t launch_draft_merge(const MergeArgs& a, cudaStream_t s);
@@ -363,6 +364,7 @@ struct GemvF32Job {
 };
 struct GemvF32Jobs {
   GemvF32Job j[2];
+  int late;                      // as MergeArgs::late
 };
 // merge: decode position merge->j and take job 0's input from the gathered
 // head input (job 0's X is not read); allowed when gemv_f32_merges.

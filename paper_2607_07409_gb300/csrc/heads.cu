@@ -40,8 +40,8 @@ __device__ __forceinline__ void sum_gates(const float* p, int S, long long strid
 
 __global__ void __launch_bounds__(256) k_gru_gates(const float* gi, int Si, const float* gh, int Sh, int B, int H,
                                                    float* __restrict__ h, uint16_t* __restrict__ h_bf16) {
-  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
+  if (threadIdx.x == 0) pdl_trigger();
   const long long total = (long long)B * H;
   const long long split_stride = (long long)B * 3 * H;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -69,7 +69,9 @@ __global__ void __launch_bounds__(256) k_gru_gates(const float* gi, int Si, cons
 // no launch of its own. gh is the sum of S recurrent partials [S][B][3H];
 // S = 0 means gh = 0 (the step from h = 0). A row that decoded to no token
 // (non-finite logits, already flagged) takes gi = 0.
-constexpr int kGatesThreads = 256;
+// CTAs of 128 units, the successor let in after the wait: 64 requests 463 -> 457
+// us per block of 16 (256 units 459, let in at once 461).
+constexpr int kGatesThreads = 128;
 
 __device__ __forceinline__ float ld_cg_f32(const float* p) {
   float v;
@@ -78,8 +80,8 @@ __device__ __forceinline__ float ld_cg_f32(const float* p) {
 }
 
 __global__ void __launch_bounds__(kGatesThreads) k_gru_gates_table(GatesTableArgs a) {
-  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
+  if (threadIdx.x == 0) pdl_trigger();
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int H = a.H;

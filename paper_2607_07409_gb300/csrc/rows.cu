@@ -439,8 +439,9 @@ __global__ void __launch_bounds__(kRowsThreads) k_verify_rows(RowsArgs a) {
 // local head's next input rows
 // ----------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_draft_merge(MergeArgs a) {
-  if (threadIdx.x == 0) pdl_trigger();
+  if (threadIdx.x == 0 && !a.late) pdl_trigger();
   pdl_wait();
+  if (threadIdx.x == 0 && a.late) pdl_trigger();
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ RowAcc red[8];
