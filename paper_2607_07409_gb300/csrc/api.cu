@@ -180,6 +180,19 @@ bool map_w(CUtensorMap* m, const void* W, int O, int K, int n_tile) {
                         (uint32_t)n_tile, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// Share of the vocabulary weights that a temperature-0 block keeps in L2 from
+// one position to the next (the whole matrix is read at every position; the
+// rest streams through): 32 MB of the 126. Measured, none kept -> 32 MB: one
+// request, 311 MB of weights 945 -> 897 us; 8 requests, 778 MB 2934 -> 2903;
+// 64 requests, 78 MB 467 -> 449; 32 requests of a Markov head, 131 MB 222 ->
+// 211. 24 and 40 MB measure the same within 6 us; 56 and 64 MB push the block's
+// other data out (64 requests 463 and 479, one request 949, 8 requests 3033).
+// Below 30 MB the matrix stays there anyway (25 MB: 344 us, kept 346).
+// Temperature-1 launches are bound by their variates (586 -> 587) and keep none.
+float keep_share(size_t bytes) {
+  return bytes <= 30000000 ? 0.f : std::min(1.f, 32e6f / (float)bytes);
+}
+
 // W as [K / 64][O][64], boxes of two K chunks (K a multiple of 64).
 bool map_w_pairs(CUtensorMap* m, const void* W, int O, int K, int n_tile) {
   return encode_tmap_3d(m, W, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, 64, (uint64_t)O, (uint64_t)(K / 64),
@@ -351,6 +364,7 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
                       es, (uint64_t)V, (uint64_t)n, (uint64_t)B, (uint64_t)V * es, (uint64_t)n * V * es,
                       (uint32_t)a.l_box_cols, 1, (uint32_t)a.l_box_rows, CU_TENSOR_MAP_SWIZZLE_128B))
     return false;
+  a.w_keep = keep_share((size_t)V * K * 2);
   g.mA1 = g.mA0;
   g.mB1 = g.mB0;
   g.grid = grid;
@@ -1321,6 +1335,19 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
     PROF(DELS_KCLASS_VOCAB_COMBINE);
     return launch_vocab_combine_f32(vf, vf_chunks, s);
   };
+  // bf16 heads: the vocabulary launch of position j. The last position streams
+  // all its weights, which gives the kept share of L2 back.
+  float keep = -1.f;
+  auto at_position = [&](Gemm& gv, int j) {
+    if (keep < 0.f) keep = gv.a.w_keep;
+    gv.a.j = j;
+    gv.a.sample = sm.on;
+    gv.a.seed = sm.seed;
+    gv.a.step = sm.step;
+    gv.a.alpha = aw(j);
+    gv.a.beta = bw(j);
+    gv.a.w_keep = j + 1 < n && !sm.on ? keep : 0.f;
+  };
   // The first product of a float32 head decodes position j - 1 and gathers its
   // input itself when each request has few records (every CTA merges them: one
   // request, V 1024, 16 records, 73 -> 62 us per block of 8; 8 requests with
@@ -1524,12 +1551,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           ga.S = j == 1 ? 0 : gh.a.total_splits;
           { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates_table(ga, s)); }
           { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rank_hh(gr, j + 1 < n ? &gh : nullptr, s)); }
-          gv.a.j = j;
-          gv.a.sample = sm.on;
-          gv.a.seed = sm.seed;
-          gv.a.step = sm.step;
-          gv.a.alpha = aw(j);
-          gv.a.beta = bw(j);
+          at_position(gv, j);
           { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
         }
         MergeArgs m = mb;
@@ -1565,12 +1587,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           { PROF(DELS_KCLASS_HEAD_MISC);
             DELS_CUDA(launch_gru_gates(gpart, gi.a.total_splits, hh_part, j == 1 ? 0 : gh.a.total_splits, B, H, h, hb, s)); }
           { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rank_hh(gr, j + 1 < n ? &gh : nullptr, s)); }
-          gv.a.j = j;
-          gv.a.sample = sm.on;
-          gv.a.seed = sm.seed;
-          gv.a.step = sm.step;
-          gv.a.alpha = aw(j);
-          gv.a.beta = bw(j);
+          at_position(gv, j);
           { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
           MergeArgs m = mb;
           m.count = gv.grid;
@@ -1660,12 +1677,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
                                              static_cast<uint16_t*>(h2), Hd, s)); }
             }
           }
-          gv.a.j = j;
-          gv.a.sample = sm.on;
-          gv.a.seed = sm.seed;
-          gv.a.step = sm.step;
-          gv.a.alpha = aw(j);
-          gv.a.beta = bw(j);
+          at_position(gv, j);
           { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
           MergeArgs m = mb;
           m.count = gv.grid;
@@ -1748,12 +1760,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_splitk_finish(xpart, S1, B, F, nullptr, ACT_GELU, nullptr, 0, fb, F, s, g1.terms, T)); }
         { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run_rows(g2, s)); }
         { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_finish_rmsnorm(xpart, S2, g2.terms, B, D, uu, y, feat, 1, s)); }
-        gv.a.j = j;
-          gv.a.sample = sm.on;
-          gv.a.seed = sm.seed;
-          gv.a.step = sm.step;
-        gv.a.alpha = aw(j);
-        gv.a.beta = bw(j);
+        at_position(gv, j);
         { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
         MergeArgs m = mb;
         m.count = gv.grid;
@@ -1778,12 +1785,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       for (int j = 1; j < n; ++j) {
         int count;
         if (bf) {
-          gv.a.j = j;
-          gv.a.sample = sm.on;
-          gv.a.seed = sm.seed;
-          gv.a.step = sm.step;
-          gv.a.alpha = aw(j);
-          gv.a.beta = bw(j);
+          at_position(gv, j);
           { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(run(gv, s)); }
           count = gv.grid;
         } else {

@@ -685,6 +685,14 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+// Evict last for `share` of the lines (by address), evict first for the rest.
+__device__ __forceinline__ uint64_t l2_policy_keep(float share) {
+  if (share <= 0.f) return l2_policy_evict_first();
+  if (share >= 1.f) return l2_policy_evict_last();
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_last.L2::evict_first.b64 %0, %1;" : "=l"(p) : "f"(share));
+  return p;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_normal() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(threads_for(MODE), MODE != 0 ? 1 : 2)
   if (warp == 0) {
     if (lane == 0) {
       if (!a.debug_skip_producer) {
-        const uint64_t pol_w = l2_policy_evict_first();    // streamed once per launch
+        const uint64_t pol_w = l2_policy_keep(a.w_keep);
         const uint64_t pol_act = l2_policy_evict_last();   // small, re-read by every CTA
         ProdState st;
         prod_prefetch(c, p, st, pol_w);                     // weights: independent of the predecessor
