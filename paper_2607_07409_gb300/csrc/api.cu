@@ -296,7 +296,7 @@ int splits_for(int O, int n_tile, int K, int sms) {
 // Vocabulary projection fused with the combine (l_L tile of position j).
 bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void* Wv, const void* longp,
                   dels_dtype ldt, const float* prior, float alpha, float beta, void* partials, int partial_ld,
-                  int* status, int sms, bool pair_stages) {
+                  int* status, int sms, bool pair_stages, bool sample) {
   TcGemmArgs& a = g.a;
   const int n_tile = 128;
   a.B = B;
@@ -324,35 +324,54 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
   const int grid = std::min(a.num_o_tiles, std::max(1, sms));
   a.max_items_per_cta = (a.num_o_tiles + grid - 1) / grid;
   const int l_fixed = 2 * a.l_boxes * a.l_box_rows * 128 + a.max_items_per_cta * n_tile * 4;
-  a.a_resident = (a.seg_chunks[0] <= 4) ? 1 : 0;
   const int es = a.long_f32 ? 4 : 2;
   // Rows of the A tile: the B requests rounded up to whole TMEM lane
   // quadrants; when that is 32 or 64 rows, 4 or 2 copies fill the tile so
   // every epilogue warp owns live rows (the copies split the columns).
   const int rpc = (B + 31) / 32 * 32;
-  a.a_box_rows = rpc;
-  a.a_copies = (rpc == 32) ? 4 : (rpc == 64 ? 2 : 1);
-  if (!a.a_resident && B <= 32) {
-    // Activations staged with every K chunk: load only the live rows, once.
-    // The copies (and a 32-row box for a handful of requests) would make
-    // every CTA fetch the same few L2 lines four times per stage, while a
-    // long K leaves the epilogue ample time for the rows of one quadrant.
-    a.a_box_rows = (B + 7) / 8 * 8;
-    a.a_copies = 1;
-  }
+  const int w_chunk = n_tile * 128;
+  const int a_all = a.seg_chunks[0] * 128 * 128;
+  const int smem = device_max_smem_optin() - kSmemReserve - l_fixed;
+  a.a_resident = (a.seg_chunks[0] <= 4 && smem - a_all >= 2 * w_chunk) ? 1 : 0;
+  int stage;
   if (a.a_resident) {
-    a.stages = pick_stages(a, n_tile * 128, a.seg_chunks[0] * 128 * 128 + l_fixed);
+    a.a_box_rows = rpc;
+    a.a_copies = (rpc == 32) ? 4 : (rpc == 64 ? 2 : 1);
+    stage = w_chunk;
+    a.stages = pick_stages(a, stage, a_all + l_fixed);
   } else {
-    a.stages = pick_stages(a, 128 * 128 + n_tile * 128, l_fixed);
+    // Activations staged with every K chunk: only the live rows, once, packed
+    // at their own pitch. Copies (and whole quadrants of rows) would make
+    // every CTA fetch the same L2 lines several times per stage, while a long
+    // K leaves the epilogue ample time for the rows of its quadrants; and at
+    // a pitch of 128 rows more than 48 requests leave room for two paired
+    // stages only. V 151936, K 1024, bf16 logits, 7 positions, whole
+    // quadrants in copies at the full pitch -> packed: 64 requests 429 -> 376
+    // us, 96: 435 -> 388, 48: 405 -> 364, 32: 360 -> 354, 1: 346 -> 341, 128:
+    // 450 -> 451; 64 requests, K 384: 205 -> 192, K 4096: 1580 -> 1381.
+    // Temperature 1, where the epilogue's and the noise warps' work per tile
+    // outlasts a short K, keeps the copies up to the K where both take the
+    // same (one copy / copies: 64 requests, K 320 345 / 274, K 512 349 / 303,
+    // K 768 395 / 394, K 1024 451 / 484; 8 requests, K 320 338 / 293, K 384
+    // 321 / 308, K 512 326 / 350).
+    const bool copies = sample && rpc <= 64 && K <= (B > 32 ? 768 : 384);
+    a.a_box_rows = copies ? rpc : (B + 7) / 8 * 8;
+    a.a_copies = copies ? (rpc == 32 ? 4 : 2) : 1;
+    a.a_pitch = a.a_copies * a.a_box_rows * 128;
+    stage = a.a_pitch + w_chunk;
+    a.stages = pick_stages(a, stage, l_fixed);
   }
   // K in whole pairs of chunks: each pipeline stage holds two consecutive
   // chunks, the weights' as one 3-D box, whose view of K has no ragged tail
   // (8B-shaped launch 29.2 -> 26.8 us;
   // with staged activations, 0.6B-shaped 59.6 -> 53.9 us, 4B-shaped
-  // 130.9 -> 126.5 us).
-  if (pair_stages && K % 128 == 0) {
+  // 130.9 -> 126.5 us). Where only two such stages fit, single chunks keep
+  // more in flight and win on a long K (128 requests, K 1024: pairs 450 us,
+  // single 457; K 1536: 637 and 631; K 4096: 1592 and 1494).
+  const int pairs = std::min(a.stages / 2, (smem - (a.a_resident ? a_all : 0)) / (2 * stage));
+  if (pair_stages && K % 128 == 0 && pairs >= (a.a_resident || a.seg_chunks[0] <= 16 ? 2 : 3)) {
     a.b_chunks = 2;
-    a.stages = std::max(2, a.stages / 2);
+    a.stages = pairs;
   }
   if (!map_x(&g.mA0, X, B, K, a.a_box_rows)) return false;
   if (a.b_chunks == 2) {
@@ -1380,7 +1399,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
             !plan_store(gr, B, R, hb, head->w[2], H, nullptr, nullptr, 0, 32, 1, 0, ACT_SILU, nullptr,
                         static_cast<uint16_t*>(rr), R, status, sms) ||
             !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                          partials, L.partial_ld, status, sms, false))
+                          partials, L.partial_ld, status, sms, false, sm.on))
           return DELS_ERR_CUDA;
         PersistGruArgs P{};
         P.B = B; P.n = n; P.V = V; P.D = D; P.H = H; P.R = R;
@@ -1449,7 +1468,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
             !plan_store(gh, B, 3 * H, hb, head->w[1], H, nullptr, nullptr, 0, kHhTile, L.hh_splits, 0, ACT_NONE,
                         gpart, nullptr, 0, status, sms) ||
             !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                          partials, L.partial_ld, status, sms, false))
+                          partials, L.partial_ld, status, sms, false, sm.on))
           return DELS_ERR_CUDA;
         // the rank product's K splits form one cluster per output tile
         gr.a.cluster_k = gr.a.total_splits;
@@ -1527,7 +1546,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         Gemm gr, gh, gv;
         if (!plan_rank_hh(gr, gh, head, L, B, hb, static_cast<uint16_t*>(rr), gpart, status) ||
             !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                          partials, L.partial_ld, status, sms, true))
+                          partials, L.partial_ld, status, sms, true, sm.on))
           return DELS_ERR_CUDA;
         GatesTableArgs ga{};
         ga.partials = partials;
@@ -1580,7 +1599,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
                         nullptr, 0, status, sms) ||
             !plan_rank_hh(gr, gh, head, L, B, hb, static_cast<uint16_t*>(rr), hh_part, status) ||
             !plan_combine(gv, B, V, n, rr, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                          partials, L.partial_ld, status, sms, true))
+                          partials, L.partial_ld, status, sms, true, sm.on))
           return DELS_ERR_CUDA;
         for (int j = 1; j < n; ++j) {
           { PROF(DELS_KCLASS_HEAD_GEMM); DELS_CUDA(run(gi, s)); }
@@ -1656,7 +1675,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
                         nullptr, 0, status, sms))
           return DELS_ERR_CUDA;
         if (!plan_combine(gv, B, V, n, feat, Hd, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                          partials, L.partial_ld, status, sms, true))
+                          partials, L.partial_ld, status, sms, true, sm.on))
           return DELS_ERR_CUDA;
         for (int j = 1; j < n; ++j) {
           if (gemv) {
@@ -1744,7 +1763,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
                 plan_store_rows(g1, B, T, F, anb, head->w[5], D, L.xs_1, xpart, status, sms) &&
                 plan_store_rows(g2, B, T, D, fb, head->w[6], F, L.xs_2, xpart, status, sms) &&
                 plan_combine(gv, B, V, n, feat, D, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                             partials, L.partial_ld, status, sms, true);
+                             partials, L.partial_ld, status, sms, true, sm.on);
       if (!ok) return DELS_ERR_CUDA;
       const int Sqkv = gqkv.g[0].a.total_splits;
       const int So = go.g[0].a.total_splits, S1 = g1.g[0].a.total_splits, S2 = g2.g[0].a.total_splits;
@@ -1780,7 +1799,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
       if (r != DELS_OK || n == 1) return r;
       Gemm gv;
       if (bf && !plan_combine(gv, B, V, n, feat, R, head->w_vocab, long_logits, logit_dtype, log_prior, alpha, beta,
-                              partials, L.partial_ld, status, sms, true))
+                              partials, L.partial_ld, status, sms, true, sm.on))
         return DELS_ERR_CUDA;
       for (int j = 1; j < n; ++j) {
         int count;

@@ -238,7 +238,7 @@ __device__ __forceinline__ bool prod_run_c(const Ctx& c, const Phase& p, ProdSta
     for (int i = 0; i < it.ke - it.kb; i += C, ++f) {
       const int kc = it.chunk(i);
       const int s = f % c.S;
-      // staged activations: chunk kc + cc of the stage at sA + s * a_stage_bytes + cc * kATileBytes
+      // staged activations: chunk kc + cc of the stage at sA + s * a_stage_bytes + cc * (a_stage_bytes / C)
       if (f < st.pre_end) {
         if (a.a_resident) {
           mbar_arrive(&c.full[s]);
@@ -247,7 +247,7 @@ __device__ __forceinline__ bool prod_run_c(const Ctx& c, const Phase& p, ProdSta
 #pragma unroll
           for (int cc = 0; cc < C; ++cc)
             for (int cp = 0; cp < a.a_copies; ++cp)
-              tma_load_2d(c.sA + s * c.a_stage_bytes + cc * kATileBytes + cp * a_copy_bytes, mA, &c.full[s],
+              tma_load_2d(c.sA + s * c.a_stage_bytes + cc * (c.a_stage_bytes / C) + cp * a_copy_bytes, mA, &c.full[s],
                           (kc + cc) * kBlockK, 0, pol_act);
         }
         continue;
@@ -261,7 +261,7 @@ __device__ __forceinline__ bool prod_run_c(const Ctx& c, const Phase& p, ProdSta
 #pragma unroll
         for (int cc = 0; cc < C; ++cc)
           for (int cp = 0; cp < a.a_copies; ++cp)
-            tma_load_2d(c.sA + s * c.a_stage_bytes + cc * kATileBytes + cp * a_copy_bytes, mA, &c.full[s],
+            tma_load_2d(c.sA + s * c.a_stage_bytes + cc * (c.a_stage_bytes / C) + cp * a_copy_bytes, mA, &c.full[s],
                         (kc + cc) * kBlockK, 0, pol_act);
       }
       load_w<C>(c, p, it, i, s, pol_w);
@@ -335,7 +335,7 @@ __device__ __forceinline__ bool mma_run_c(const Ctx& c, const Phase& p, MmaState
       for (int cc = 0; cc < C; ++cc) {
         const int kc = it.chunk(i + cc);
         const uint32_t a_addr =
-            smem_u32(a.a_resident ? c.sA + kc * kATileBytes : c.sA + s * c.a_stage_bytes + cc * kATileBytes);
+            smem_u32(a.a_resident ? c.sA + kc * kATileBytes : c.sA + s * c.a_stage_bytes + cc * (c.a_stage_bytes / C));
         const uint32_t b_addr = smem_u32(c.sB + s * c.b_stage_bytes + cc * a.n_tile * 128);
 #pragma unroll
         for (int kk = 0; kk < kBlockK / kUmmaK; ++kk) {

@@ -16,9 +16,10 @@
 // Programmatic dependent launch: a store launch lets its successor launch at
 // once, a combine launch once its own predecessor has finished (the small
 // kernels that follow it would otherwise sit on its SMs through the wait: 64
-// requests at temperature 1 590 -> 585 us, one MLP request 941 -> 935). Before waiting for its own predecessor it already allocates TMEM,
-// stages the prior, starts the DFlash-logit tiles and the first weight
-// stages — everything that does not depend on the previous kernel.
+// requests at temperature 1 590 -> 585 us, one MLP request 941 -> 935). Before
+// waiting for its own predecessor it already allocates TMEM, stages the prior,
+// starts the DFlash-logit tiles and the first weight stages — everything that
+// does not depend on the previous kernel.
 #include <algorithm>
 
 #include "tc_engine.cuh"
@@ -46,17 +47,23 @@ __host__ __device__ inline bool store_transposes(const TcGemmArgs& a) {
   return a.epi == EPI_STORE && a.out_f32 && !a.out_bmajor && !a.out_bf16;
 }
 
+__host__ __device__ inline uint32_t a_pitch(const TcGemmArgs& a) {
+  return a.a_pitch ? (uint32_t)a.a_pitch : (uint32_t)kATileBytes;
+}
+
 __host__ __device__ inline Smem smem_layout(const TcGemmArgs& a) {
   Smem s{};
   const int b_tile = a.n_tile * 128;
   const bool comb = a.epi == EPI_COMBINE;
   const int l_tile = comb ? a.l_boxes * a.l_box_rows * 128 : 0;
-  const int a_tiles = a.a_resident ? a.seg_chunks[0] : a.stages * (a.b_chunks > 1 ? a.b_chunks : 1);
+  const int chunks = a.b_chunks > 1 ? a.b_chunks : 1;
   uint32_t off = 0;
   s.a_off = off;
-  off += (uint32_t)a_tiles * kATileBytes;
+  // staged chunks may be packed closer than the 128 rows the MMA reads: the
+  // last one's dead rows are then read from the weight stages
+  off += a.a_resident ? (uint32_t)a.seg_chunks[0] * kATileBytes : (uint32_t)(a.stages * chunks) * a_pitch(a);
   s.b_off = off;
-  off += (uint32_t)a.stages * b_tile * (uint32_t)(a.b_chunks > 1 ? a.b_chunks : 1);
+  off += (uint32_t)(a.stages * chunks * b_tile);
   s.l_off = off;
   off += 2u * l_tile;
   s.p_off = off;
@@ -190,7 +197,7 @@ __global__ void __launch_bounds__(threads_for(MODE), MODE != 0 ? 1 : 2)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mmadone + 1);
   c.abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   c.S = a.stages;
-  c.a_stage_bytes = kATileBytes * (uint32_t)(a.b_chunks > 1 ? a.b_chunks : 1);
+  c.a_stage_bytes = a_pitch(a) * (uint32_t)(a.b_chunks > 1 ? a.b_chunks : 1);
   c.b_stage_bytes = (uint32_t)a.n_tile * 128u * (uint32_t)(a.b_chunks > 1 ? a.b_chunks : 1);
   c.l_buf_bytes = comb ? (uint32_t)(a.l_boxes * a.l_box_rows * 128) : 0u;
   c.deadline = globaltimer_ns() + budget_ns;

@@ -274,6 +274,23 @@ def test_draft_ragged_feature_width(head, r, h):
     check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
 
 
+@pytest.mark.parametrize("B,r,ldt", [
+    (1, 1024, "bf16"), (7, 336, "f32"),         # one block of eight rows per stage; a ragged chunk
+    (33, 384, "bf16"), (64, 1024, "f32"),       # two lane quadrants
+    (65, 320, "bf16"), (96, 1024, "bf16"),      # three; an odd number of chunks
+    (96, 256, "f32"), (128, 256, "f32"),        # float32 logit tiles: single chunks / nothing resident
+    (104, 512, "f32"), (128, 1152, "bf16"),     # two stages of pairs do not fit / are too few for a long K
+])
+def test_draft_staged_activation_edges(B, r, ldt):
+    """Vocabulary launches whose activations are packed at their own pitch, more
+    tiles than CTAs, at the edges of the stage plan."""
+    w = synth.stress(synth.Workload("staged", B=B, n=3, V=24008, logit_dtype=ldt,
+                                    head=synth.HeadSpec("markov", "bf16", 0, 0, r), weight=1.0, seed=B))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    tok, lp, gap, W, prior = _draft(w, d)
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 @pytest.mark.parametrize("head,B,V,d,h,r", [
     ("gru", 1, 1000, 132, 36, 20),          # one request; widths just past and below a 128-wide step
     ("gru", 2, 72, 8, 4, 4),                # two requests, the smallest widths

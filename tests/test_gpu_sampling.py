@@ -52,6 +52,24 @@ def test_sampled_draft_matches_oracle(name, seed, step):
     print(name, record(f"sampled draft {name}", info))
 
 
+@pytest.mark.parametrize("B,r,ldt", [(32, 384, "bf16"), (33, 768, "f32"), (64, 512, "bf16"), (40, 896, "bf16"),
+                                     (9, 400, "bf16"), (96, 512, "f32"), (128, 256, "f32")])
+def test_sampled_draft_staged_activation_edges(B, r, ldt):
+    """Both sides of the lines between copied and packed activations, and
+    float32 logit tiles that leave no room for resident ones."""
+    w = synth.stress(synth.Workload("staged", B=B, n=3, V=24008, logit_dtype=ldt,
+                                    head=synth.HeadSpec("markov", "bf16", 0, 0, r), weight=0.5, seed=B))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    a, b = _learned_weights(w.n)
+    W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+    dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+    tok, lp, gap, _ = dr.sample(d["long"], dels.dels_prior_from_counts(d["counts"]).to(DEV), a, b, 17, 3)
+    torch.cuda.synchronize()
+    assert dr.status() == 0
+    check_draft(tok.cpu().numpy(), lp.cpu().numpy(), gap.cpu().numpy(), _oracle_head(w, W), d["long"].cpu(),
+                oracle.log_prior(d["counts"]), np.array(a), np.array(b), LP_TOL_BF16, sample=(17, 3))
+
+
 def test_sampled_calls_reject_a_step_outside_the_counter_word():
     w = synth.stress(SMALL["gru"])
     d = synth.make_inputs(w, device=DEV, target=False)
