@@ -368,7 +368,12 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
   // 130.9 -> 126.5 us). Where only two such stages fit, single chunks keep
   // more in flight and win on a long K (128 requests, K 1024: pairs 450 us,
   // single 457; K 1536: 637 and 631; K 4096: 1592 and 1494).
-  const int pairs = std::min(a.stages / 2, (smem - (a.a_resident ? a_all : 0)) / (2 * stage));
+  int pairs = std::min(a.stages / 2, (smem - (a.a_resident ? a_all : 0)) / (2 * stage));
+  // Few packed rows would leave room for six pairs; the last ones only keep
+  // the neighbouring launches' CTAs off the SM (3 / 4 / 5 / 6 pairs: one MLP
+  // request, K 1024 899 / 885 / 895 / 907 us; 8 transformer requests, K 2560
+  // 2928 / 2878 / 2865 / 2904).
+  if (!a.a_resident) pairs = std::min(pairs, a.seg_chunks[0] <= 16 ? 4 : 5);
   if (pair_stages && K % 128 == 0 && pairs >= (a.a_resident || a.seg_chunks[0] <= 16 ? 2 : 3)) {
     a.b_chunks = 2;
     a.stages = pairs;

@@ -8,7 +8,7 @@
 // keep up: token frequencies are Zipf-like, and the adds to the most frequent
 // id (about 13% of positions) serialise at one L2 address. So the counts are
 // kept per CTA in shared memory, which holds 227 KB: about 57K 32-bit bins,
-// a third of a 152K vocabulary. Two pieces:
+// a third of a 152K vocabulary. Three schemes:
 //
 // * Half-word slices (k_prior_halves): the vocabulary is cut into P slices of
 //   16-bit bins, two to a word, that each fit (115K ids a slice); P groups of
