@@ -206,7 +206,7 @@ struct TcGemmArgs {
   int seg_splits[2];             // K splits per segment (0 splits: unused segment)
   int seg_per[2];                // K chunks per split (the last may have fewer)
   int a_pitch;                   // bytes of one staged activation chunk (0: a full 128-row tile)
-  float w_keep;                  // share of the weights to keep in L2 (evict last) for the next position; the rest
+  float w_keep;                  // share of the weights kept in L2 (evict last) for the next position; the rest
                                  // is streamed (evict first)
   int sum_terms;                 // EPI_STORE f32 rows: 3: the B rows are three groups of B / 3, stored as the sum of
                                  // the groups (all in one TMEM quadrant: B <= 32); otherwise stored as they are
