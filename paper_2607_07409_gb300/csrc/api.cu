@@ -349,15 +349,20 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
     // quadrants in copies at the full pitch -> packed: 64 requests 429 -> 376
     // us, 96: 435 -> 388, 48: 405 -> 364, 32: 360 -> 354, 1: 346 -> 341, 128:
     // 450 -> 451; 64 requests, K 384: 205 -> 192, K 4096: 1580 -> 1381.
-    // Temperature 1, where the epilogue's and the noise warps' work per tile
-    // outlasts a short K, keeps the copies up to the K where both take the
-    // same (one copy / copies: 64 requests, K 320 345 / 274, K 512 349 / 303,
-    // K 768 395 / 394, K 1024 451 / 484; 8 requests, K 320 338 / 293, K 384
-    // 321 / 308, K 512 326 / 350).
-    const bool copies = sample && rpc <= 64 && K <= (B > 32 ? 768 : 384);
-    a.a_box_rows = copies ? rpc : (B + 7) / 8 * 8;
+    // Copies (of the live rows, one per lane quadrant or pair of quadrants)
+    // share out the epilogue's and, at temperature 1, the noise warps' work per
+    // tile, which outlasts a short K. One copy / copies, temperature 1: 1
+    // request, K 384 306 / 253, K 512 311 / 290, K 768 338 / 361; 32 requests,
+    // K 512 330 / 308, K 768 360 / 382; 64 requests, K 320 345 / 272, K 768 396
+    // / 396, K 1024 454 / 485. Temperature 0, 40 requests, K 384 189 / 179, K
+    // 512 218 / 213, K 1024 360 / 363; not where a 128-row pitch leaves only
+    // two paired stages (64 requests, K 384 192 / 206), nor for one quadrant (8
+    // requests, K 384 164 / 190).
+    const bool copies = rpc <= 64 && (sample ? K <= (B > 32 ? 768 : 512)
+                                             : B > 32 && K <= 512 && smem >= 6 * (128 * 128 + w_chunk));
+    a.a_box_rows = (B + 7) / 8 * 8;
     a.a_copies = copies ? (rpc == 32 ? 4 : 2) : 1;
-    a.a_pitch = a.a_copies * a.a_box_rows * 128;
+    a.a_pitch = copies ? 128 * 128 : a.a_box_rows * 128;
     stage = a.a_pitch + w_chunk;
     a.stages = pick_stages(a, stage, l_fixed);
   }

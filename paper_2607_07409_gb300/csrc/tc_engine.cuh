@@ -218,8 +218,8 @@ __device__ __forceinline__ bool prod_run_c(const Ctx& c, const Phase& p, ProdSta
                                            uint64_t pol_act) {
   const TcGemmArgs& a = *p.a;
   const uint32_t b_bytes = (uint32_t)a.n_tile * 128u * (uint32_t)C;
-  const uint32_t a_copy_bytes = (uint32_t)a.a_box_rows * 128u;
-  const uint32_t a_bytes = a_copy_bytes * (uint32_t)a.a_copies;
+  const uint32_t a_copy_bytes = (uint32_t)((a.a_box_rows + 31) / 32) * 32u * 128u;   // copies start on whole lane quadrants
+  const uint32_t a_bytes = (uint32_t)(a.a_box_rows * a.a_copies) * 128u;
   if (a.a_resident && p.count > 0) {
     // every CTA loads the same activations here: start at a CTA-dependent chunk
     const int nch = a.seg_chunks[0];
@@ -502,7 +502,7 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
   const int g = (warp - 2) >> 2;               // column-chunk parity
   const int nchunk = a.n_tile / 32;
   // The A tile holds a_copies stacked copies of the activation rows (each
-  // a_box_rows rows, a multiple of 32 for the combine): quadrant q holds copy
+  // a_box_rows rows, starting on a whole quadrant): quadrant q holds copy
   // cpy, rows 32*(q % qpc)..; the copies split the tile's 32-column chunks
   // between them, so every row's columns are covered exactly once.
   const int qpc = comb ? (a.a_box_rows + 31) / 32 : 4;

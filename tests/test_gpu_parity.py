@@ -276,7 +276,8 @@ def test_draft_ragged_feature_width(head, r, h):
 
 @pytest.mark.parametrize("B,r,ldt", [
     (1, 1024, "bf16"), (7, 336, "f32"),         # one block of eight rows per stage; a ragged chunk
-    (33, 384, "bf16"), (64, 1024, "f32"),       # two lane quadrants
+    (33, 384, "bf16"), (48, 512, "bf16"),       # two lane quadrants, twice
+    (40, 576, "bf16"), (64, 1024, "f32"),       # and once
     (65, 320, "bf16"), (96, 1024, "bf16"),      # three; an odd number of chunks
     (96, 256, "f32"), (128, 256, "f32"),        # float32 logit tiles: single chunks / nothing resident
     (104, 512, "f32"), (128, 1152, "bf16"),     # two stages of pairs do not fit / are too few for a long K

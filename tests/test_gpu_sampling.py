@@ -53,7 +53,8 @@ def test_sampled_draft_matches_oracle(name, seed, step):
 
 
 @pytest.mark.parametrize("B,r,ldt", [(32, 384, "bf16"), (33, 768, "f32"), (64, 512, "bf16"), (40, 896, "bf16"),
-                                     (9, 400, "bf16"), (96, 512, "f32"), (128, 256, "f32")])
+                                     (9, 400, "bf16"), (32, 576, "f32"), (1, 512, "bf16"), (96, 512, "f32"),
+                                     (128, 256, "f32")])
 def test_sampled_draft_staged_activation_edges(B, r, ldt):
     """Both sides of the lines between copied and packed activations, and
     float32 logit tiles that leave no room for resident ones."""
