@@ -205,6 +205,12 @@ int pick_stages(const TcGemmArgs& a, int per_stage, int fixed) {
   return std::max(2, std::min(st, 12));
 }
 
+// The activation bytes of a chunk, from the box and the copies.
+void set_a_bytes(TcGemmArgs& a) {
+  a.a_copy_bytes = (a.a_box_rows + 31) / 32 * 32 * 128;
+  a.a_load_bytes = a.a_box_rows * a.a_copies * 128;
+}
+
 // pair_stages: two K chunks per pipeline stage where K is whole pairs. Taken
 // for the GRU's rank and recurrent products (64 requests, block of 16: 518 ->
 // 501 us with both, 521 and 509 with one); the input product and the
@@ -245,6 +251,7 @@ bool plan_store(Gemm& g, int B, int O, const void* X0, const void* W0, int K0, c
   // only the B real rows are loaded; the tile's other rows feed unused outputs
   a.a_box_rows = std::min(128, (B + 7) / 8 * 8);
   a.a_copies = 1;
+  set_a_bytes(a);
   a.stages = pick_stages(a, a.b_chunks * (128 * 128 + n_tile * 128), (out_f32 && !out_bf16) ? kStoreTransposeBytes : 0);
   auto weights = [&](CUtensorMap* m, const void* W, int K) {
     return a.b_chunks == 2 ? map_w_pairs(m, W, O, K, n_tile) : map_w(m, W, O, K, n_tile);
@@ -366,6 +373,7 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
     stage = a.a_pitch + w_chunk;
     a.stages = pick_stages(a, stage, l_fixed);
   }
+  set_a_bytes(a);
   // K in whole pairs of chunks: each pipeline stage holds two consecutive
   // chunks, the weights' as one 3-D box, whose view of K has no ragged tail
   // (8B-shaped launch 29.2 -> 26.8 us;

@@ -218,8 +218,8 @@ __device__ __forceinline__ bool prod_run_c(const Ctx& c, const Phase& p, ProdSta
                                            uint64_t pol_act) {
   const TcGemmArgs& a = *p.a;
   const uint32_t b_bytes = (uint32_t)a.n_tile * 128u * (uint32_t)C;
-  const uint32_t a_copy_bytes = (uint32_t)((a.a_box_rows + 31) / 32) * 32u * 128u;   // copies start on whole lane quadrants
-  const uint32_t a_bytes = (uint32_t)(a.a_box_rows * a.a_copies) * 128u;
+  const uint32_t a_copy_bytes = (uint32_t)a.a_copy_bytes;
+  const uint32_t a_bytes = (uint32_t)a.a_load_bytes;
   if (a.a_resident && p.count > 0) {
     // every CTA loads the same activations here: start at a CTA-dependent chunk
     const int nch = a.seg_chunks[0];
