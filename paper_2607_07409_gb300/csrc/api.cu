@@ -1462,7 +1462,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         }
       }
       const float* G = static_cast<const float*>(head->w[3]);
-      if (bf && G && fused_products_enabled() && !sm.on && B <= 64) {
+      if (bf && G && fused_products_enabled() && !sm.on && B <= 64 && n > 1) {
         // Input-table path, fused variant (DELS_DRAFT_FUSED=1): two launches
         // per position —
         //   gates(j)        merge x_{j-1} from the previous position's records,
@@ -1473,13 +1473,6 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         //                   combine -> per-CTA records.
         // A last merge kernel decodes x_{n-1}. h_0 = 0 needs no clearing:
         // gates(1) runs with no recurrent partials and h = 0.
-        mb.table = nullptr;
-        if (n == 1) return draft_position0(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, mb, sms, s);
-        unsigned* r_ready = at<unsigned>(workspace, kRReadyOff);
-        DELS_CUDA(cudaMemsetAsync(r_ready, 0, sizeof(unsigned), s));
-        int count = 0;
-        r = position0_rows(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, sms, s, &count);
-        if (r != DELS_OK) return r;
         Gemm gr, gh, gv;
         if (!plan_store(gr, B, R, hb, head->w[2], H, nullptr, nullptr, 0, kRankTile, kRankClusterSplits, 0,
                         ACT_SILU, nullptr, static_cast<uint16_t*>(rr), R, status, sms) ||
@@ -1500,8 +1493,7 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
         // take part in the products (and publish neutral records)
         const int ck = gr.a.cluster_k;
         const int grid = std::min(sms, std::max(gv.grid, P.rank_ctas + std::min(hh_items, sms))) / ck * ck;
-        if (P.rank_ctas >= grid || grid > L.partial_ld) return DELS_ERR_UNSUPPORTED;
-        P.r_ready = r_ready;
+        P.r_ready = at<unsigned>(workspace, kRReadyOff);
         P.r = static_cast<uint16_t*>(rr);
         P.R = R;
         P.stages = kMaxStagesHost;
@@ -1510,40 +1502,50 @@ int draft_block_impl(const dels_local_head* head, const void* long_logits, dels_
           --P.stages;
           smem = prod_vocab_smem_bytes(P);
         }
-        if ((int)smem > device_max_smem_optin()) return DELS_ERR_UNSUPPORTED;
-        const CUtensorMap maps[6] = {gr.mA0, gr.mB0, gh.mB0, gv.mA0, gv.mB0, gv.mL};
-        GatesTableArgs ga{};
-        ga.partials = partials;
-        ga.partial_ld = L.partial_ld;
-        ga.tokens = out_tokens;
-        ga.out_lp = out_logprob;
-        ga.out_gap = out_top2_gap;
-        ga.n = n;
-        ga.G = G;
-        ga.V = V;
-        ga.part = gpart;
-        ga.B = B;
-        ga.H = H;
-        ga.h = h;
-        ga.h_bf16 = hb;
-        ga.status = status;
-        for (int j = 1; j < n; ++j) {
-          ga.count = j == 1 ? count : grid;
-          ga.jprev = j - 1;
-          ga.S = j == 1 ? 0 : gh.a.total_splits;
-          { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates_table(ga, s)); }
-          P.vocab.j = j;
-          P.vocab.alpha = aw(j);
-          P.vocab.beta = bw(j);
-          P.hh_ctas = j + 1 < n ? std::min(hh_items, grid - P.rank_ctas) : 0;
-          P.r_target = (unsigned)(j * gr.a.num_o_tiles);
-          { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(launch_prod_vocab(P, maps, grid, smem, s)); }
+        // What the kernel cannot run takes the three launches below: its stages
+        // hold the B activation rows once (resident activations have an area of
+        // their own), and the rank product's CTAs leave some for the others.
+        if ((gv.a.a_resident || gv.a.a_copies == 1) && P.rank_ctas < grid && grid <= L.partial_ld &&
+            (int)smem <= device_max_smem_optin()) {
+          mb.table = nullptr;
+          DELS_CUDA(cudaMemsetAsync(P.r_ready, 0, sizeof(unsigned), s));
+          int count = 0;
+          r = position0_rows(long_logits, logit_dtype, B, n, V, partials, L.partial_ld, status, sms, s, &count);
+          if (r != DELS_OK) return r;
+          const CUtensorMap maps[6] = {gr.mA0, gr.mB0, gh.mB0, gv.mA0, gv.mB0, gv.mL};
+          GatesTableArgs ga{};
+          ga.partials = partials;
+          ga.partial_ld = L.partial_ld;
+          ga.tokens = out_tokens;
+          ga.out_lp = out_logprob;
+          ga.out_gap = out_top2_gap;
+          ga.n = n;
+          ga.G = G;
+          ga.V = V;
+          ga.part = gpart;
+          ga.B = B;
+          ga.H = H;
+          ga.h = h;
+          ga.h_bf16 = hb;
+          ga.status = status;
+          for (int j = 1; j < n; ++j) {
+            ga.count = j == 1 ? count : grid;
+            ga.jprev = j - 1;
+            ga.S = j == 1 ? 0 : gh.a.total_splits;
+            { PROF(DELS_KCLASS_HEAD_MISC); DELS_CUDA(launch_gru_gates_table(ga, s)); }
+            P.vocab.j = j;
+            P.vocab.alpha = aw(j);
+            P.vocab.beta = bw(j);
+            P.hh_ctas = j + 1 < n ? std::min(hh_items, grid - P.rank_ctas) : 0;
+            P.r_target = (unsigned)(j * gr.a.num_o_tiles);
+            { PROF(DELS_KCLASS_VOCAB_COMBINE); DELS_CUDA(launch_prod_vocab(P, maps, grid, smem, s)); }
+          }
+          MergeArgs m = mb;
+          m.count = grid;
+          m.j = n - 1;
+          { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
+          return DELS_OK;
         }
-        MergeArgs m = mb;
-        m.count = grid;
-        m.j = n - 1;
-        { PROF(DELS_KCLASS_MERGE); DELS_CUDA(launch_draft_merge(m, s)); }
-        return DELS_OK;
       }
       if (bf && G) {
         // Input-table path (gi = G[x] with G = E W_ih^T precomputed): three

@@ -413,6 +413,19 @@ def test_draft_fused_products_vocab_kernel_matches_oracle(name, stress, monkeypa
     print(name, stress, info)
 
 
+@pytest.mark.parametrize("B,r", [(40, 512), (33, 320), (48, 512),   # planned with two copies of the rows: the three launches
+                                 (12, 384), (64, 512)])             # rows staged once: the cooperative launch
+def test_draft_fused_products_vocab_staged_activations(B, r, monkeypatch):
+    """Ranks whose activations are not resident in the vocabulary phase."""
+    monkeypatch.setenv("DELS_DRAFT_FUSED", "1")
+    w = synth.stress(synth.with_sizes(synth.WORKLOADS["qwen3_8b_batched"], B=B, n=4, V=24008,
+                                      head_d_model=256, head_d_hidden=128, head_d_rank=r))
+    d = _with_table(w, synth.make_inputs(w, device=DEV, target=False))
+    tok, lp, gap, W, prior = _draft(w, d)
+    W = {k: v for k, v in W.items() if k != "input_table"}
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 def _learned_weights(n):
     """Per-position (alpha_j, beta_j) from the Appendix C table (positions 2..15
     are j = 1..14; later positions keep the last printed value)."""
