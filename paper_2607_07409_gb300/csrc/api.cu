@@ -613,7 +613,10 @@ bool plan_rank_hh(Gemm& gr, Gemm& gh, const dels_local_head* hd, const DraftLayo
   if (ck > 1) {
     gr.a.cluster_k = ck;
     gr.grid = gr.a.num_o_tiles * ck;
-    gr.a.stages = std::max(2, std::min(gr.a.stages, gr.a.seg_per[0] / gr.a.b_chunks));
+    // as many stages as fit beside the area that takes the other splits' sums
+    // (it binds from a state of about 2100 on), no more than a split has
+    const int fit = pick_stages(gr.a, gr.a.b_chunks * (128 * 128 + kRankTile * 128), (ck - 1) * 128 * kRankTile * 4);
+    gr.a.stages = std::max(2, std::min(fit, gr.a.seg_per[0] / gr.a.b_chunks));
     gr.smem = tc_gemm_smem_bytes(gr.a);
   }
   // both products fit one wave next to each other; whole clusters only

@@ -274,6 +274,21 @@ def test_draft_ragged_feature_width(head, r, h):
     check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
 
 
+@pytest.mark.parametrize("table", [False, True])
+@pytest.mark.parametrize("h", [2048, 2112, 2560])   # the last with stages for all of a split's K, single chunks, pairs
+def test_draft_wide_gru_state(h, table):
+    """States whose K split fills the rank product's pipeline: its stages share
+    the CTA's memory with the cluster's sums."""
+    spec = synth.HeadSpec("gru", "bf16", 128, h, 64)
+    w = synth.stress(synth.Workload("wide", B=3, n=3, V=3000, logit_dtype="bf16", head=spec, weight=1.0, seed=h))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    if table:
+        d = _with_table(w, d)
+    tok, lp, gap, W, prior = _draft(w, d)
+    W = {k: v for k, v in W.items() if k != "input_table"}
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 @pytest.mark.parametrize("B,r,ldt", [
     (1, 1024, "bf16"), (7, 336, "f32"),         # one block of eight rows per stage; a ragged chunk
     (33, 384, "bf16"), (48, 512, "bf16"),       # two lane quadrants, twice
