@@ -479,7 +479,7 @@ constexpr int kXfmrTerms = 3;
 // Input-table GRU path: output tile widths of the rank product and of the
 // recurrent product (both split over K).
 constexpr int kRankTile = 32;
-constexpr int kRankSplits = 4;     // K splits of the rank product (grouped launch)
+constexpr int kRankSplits = 4;     // K splits of the rank product at most (grouped launch)
 constexpr int kRankClusterSplits = 2;   // ... in the cooperative products+vocabulary launch (2-CTA clusters)
 constexpr size_t kRReadyOff = 128; // workspace header: rank tiles finished in the current block
 constexpr int kHhTile = 64;
@@ -501,7 +501,8 @@ struct DraftLayout {
   // GRU
   size_t eg = 0, h = 0, hb = 0, gpart = 0, r = 0;
   int gru_s0 = 0, gru_s1 = 0;
-  int rank_grid = 0, hh_splits = 0, ih_splits = 0;   // grouped rank + recurrent product; input product alone
+  // grouped rank + recurrent product (CTAs of the second at most); input product alone
+  int rank_splits = 0, hh_ctas = 0, hh_splits = 0, ih_splits = 0;
   // MLP
   size_t u = 0, mpart = 0, h1 = 0, h2 = 0;
   int mlp_s1 = 0, mlp_s2 = 0;
@@ -513,6 +514,24 @@ struct DraftLayout {
   size_t mk = 0;
   size_t total = 0;
 };
+
+// How the GRU's rank and recurrent products share the chip: as many K splits
+// of the rank product as keep it within a quarter of the SMs (four up to rank
+// 288, two to 608, then one), the rest to the recurrent product; from rank
+// 2432 on, where less than half is left, the recurrent product gets a CTA for
+// every SM, which come in as the rank product's finish. 64 requests, block of
+// 11, V 24008, state 1024, no table; four splits throughout with what they
+// leave for the recurrent product / this rule / the recurrent product beside
+// the input product and the rank product alone: rank 512 320 / 319 / 417 us,
+// 1024 450 / 364 / 489, 1216 929 / 425 / 521, 2048 977 / 452 / 622, 4096 1296 /
+// 683 / 871.
+void share_rank_hh(int R, int sms, int& rank_splits, int& hh_ctas) {
+  const int tiles = (R + kRankTile - 1) / kRankTile;
+  rank_splits = kRankSplits;
+  while (rank_splits > 1 && tiles * rank_splits > sms / 4) rank_splits /= 2;
+  const int rest = sms - tiles * rank_splits;
+  hh_ctas = rest >= sms / 2 ? rest : sms;
+}
 
 int head_es(const dels_local_head* h) { return h->wdtype == DELS_F32 ? 4 : 2; }
 
@@ -535,8 +554,8 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
       if (bf) {
         L.gru_s0 = std::max(1, std::min((D + 63) / 64, sms / std::max(1, (3 * H + 127) / 128) - 1));
         L.gru_s1 = 1;
-        L.rank_grid = (R + kRankTile - 1) / kRankTile * kRankSplits;
-        L.hh_splits = splits_for(3 * H, kHhTile, H, std::max(1, sms - L.rank_grid));
+        share_rank_hh(R, sms, L.rank_splits, L.hh_ctas);
+        L.hh_splits = splits_for(3 * H, kHhTile, H, L.hh_ctas);
         L.ih_splits = splits_for(3 * H, 128, D, sms);
       } else {
         L.gru_s0 = 1;
@@ -604,8 +623,8 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
 bool plan_rank_hh(Gemm& gr, Gemm& gh, const dels_local_head* hd, const DraftLayout& L, int B, const uint16_t* hb,
                   uint16_t* r, float* hh_part, int* status) {
   const int H = hd->d_hidden, R = hd->d_rank, sms = L.sms;
-  if (!plan_store(gr, B, R, hb, hd->w[2], H, nullptr, nullptr, 0, kRankTile, kRankSplits, 0, ACT_SILU, nullptr, r, R,
-                  status, sms, true) ||
+  if (!plan_store(gr, B, R, hb, hd->w[2], H, nullptr, nullptr, 0, kRankTile, L.rank_splits, 0, ACT_SILU, nullptr, r,
+                  R, status, sms, true) ||
       !plan_store(gh, B, 3 * H, hb, hd->w[1], H, nullptr, nullptr, 0, kHhTile, L.hh_splits, 0, ACT_NONE, hh_part,
                   nullptr, 0, status, sms, true))
     return false;
@@ -619,8 +638,8 @@ bool plan_rank_hh(Gemm& gr, Gemm& gh, const dels_local_head* hd, const DraftLayo
     gr.a.stages = std::max(2, std::min(fit, gr.a.seg_per[0] / gr.a.b_chunks));
     gr.smem = tc_gemm_smem_bytes(gr.a);
   }
-  // both products fit one wave next to each other; whole clusters only
-  gh.grid = std::min(gh.grid, std::max(ck, sms - gr.grid));
+  // whole clusters only
+  gh.grid = std::min(gh.grid, L.hh_ctas);
   gh.grid = std::max(ck, gh.grid / ck * ck);
   return true;
 }

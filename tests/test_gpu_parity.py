@@ -289,6 +289,20 @@ def test_draft_wide_gru_state(h, table):
     check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
 
 
+@pytest.mark.parametrize("table", [False, True])
+@pytest.mark.parametrize("r", [288, 304, 608, 624, 2432, 2448])   # 4 | 2 | 1 K splits of W_rank h; W_hh h on every SM
+def test_draft_gru_rank_shares(r, table):
+    """Both sides of each line in how the rank and recurrent products share the chip."""
+    spec = synth.HeadSpec("gru", "bf16", 128, 512, r)
+    w = synth.stress(synth.Workload("rank", B=5, n=4, V=3000, logit_dtype="bf16", head=spec, weight=1.0, seed=r))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    if table:
+        d = _with_table(w, d)
+    tok, lp, gap, W, prior = _draft(w, d)
+    W = {k: v for k, v in W.items() if k != "input_table"}
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 @pytest.mark.parametrize("B,r,ldt", [
     (1, 1024, "bf16"), (7, 336, "f32"),         # one block of eight rows per stage; a ragged chunk
     (33, 384, "bf16"), (48, 512, "bf16"),       # two lane quadrants, twice
