@@ -69,6 +69,10 @@ __device__ __forceinline__ float max8(const float (&x)[8]) {
   return fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), fmaxf(fmaxf(x[4], x[5]), fmaxf(x[6], x[7])));
 }
 
+__device__ __forceinline__ float min8(const float (&x)[8]) {
+  return fminf(fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), fminf(fminf(x[4], x[5]), fminf(x[6], x[7])));
+}
+
 // Top-2 update of eight keys with maximum km: element by element only when
 // km exceeds the runner-up (smaller keys change nothing).
 __device__ __forceinline__ void push8(const float (&k)[8], float km, int c, float& best, float& second, int& idx) {
@@ -291,6 +295,17 @@ __device__ __forceinline__ void load8_row(const T* row, int c, int c1, float (&x
   }
 }
 
+// The fast weights flush p and q below 2^-126 to zero, which changes a weight
+// p - q noticeably only below 2^-102, so weights up to that are left to a second
+// pass with weights of the whole float range. A key of such a weight is at most
+// -102 ln 2 - ln(-ln(1 - 2^-24)) = -54.07, so the pass is taken by the threads
+// alone whose runner-up ends below that; and p - q <= 2^-102 is not zero only
+// for p < 2^-77 (p and q are multiples of 2^-101 above), so only where a target
+// logit is that small. (Verification of 64 requests of 151936: 118.4 us without
+// the pass, 118.8 with it.)
+constexpr float kSmallWeight = 0x1p-102f;
+constexpr float kSmallKey = -54.f;
+
 // Records of the bonus draw of request b over one chunk of the vocabulary:
 // residual keys log(max(0, p_a - q_a)) + g (a < n) and target keys t + g
 // (used after n acceptances, or when every residual weight rounded to zero).
@@ -320,26 +335,60 @@ __global__ void __launch_bounds__(kSampleThreads) k_residual_rows(VerifySampledA
   const float* prior = a.prior ? a.prior + c0 : nullptr;
   float rb = -INFINITY, rs = -INFINITY, pb = -INFINITY, ps = -INFINITY;
   int ri = 0x7FFFFFFF, pi = 0x7FFFFFFF;
-  for (int c = 8 * (int)threadIdx.x; c < cols; c += 8 * kSampleThreads) {
-    float t[8], l[8], sl[8], pr[8];
-    load8_row<TT, VEC>(trow, c, cols, t);
+  float lo = INFINITY;                      // the smallest target logit met
+  auto load_pair = [&](int c, float (&l)[8], float (&sl)[8], float (&pr)[8]) {
     if (resid) load8_row<TL, VEC>(lrow, c, cols, l);
     if (head) {
       load8_row<float, VEC>(ls, c, cols, sl);
       if (prior) load8_row<float, VEC>(prior, c, cols, pr);
     }
+  };
+  auto fused = [&](float l, float sl, float pr) {
+    return head ? fmaf(nbe, prior ? pr : 0.f, fmaf(al, sl, l)) : l;
+  };
+  auto weight = [&](float t, float x) {
+    return ex2_approx((t - lse_t) * kLog2e) - ex2_approx((x - lse_q) * kLog2e);
+  };
+  for (int c = 8 * (int)threadIdx.x; c < cols; c += 8 * kSampleThreads) {
+    float t[8], l[8], sl[8], pr[8];
+    load8_row<TT, VEC>(trow, c, cols, t);
+    load_pair(c, l, sl, pr);
     float g[8], k[8];
     gumbel8(a.seed, a.step, b, acc, kStreamResidual, (c0 + c) >> 3, g);
 #pragma unroll
     for (int i = 0; i < 8; ++i) k[i] = t[i] + g[i];
     push8(k, max8(k), (int)(c0 + c), pb, ps, pi);
     if (resid) {
+      lo = fminf(lo, min8(t));
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        float x = l[i];
-        if (head) x = fmaf(nbe, prior ? pr[i] : 0.f, fmaf(al, sl[i], x));
-        const float w = ex2_approx((t[i] - lse_t) * kLog2e) - ex2_approx((x - lse_q) * kLog2e);
-        k[i] = w > 0.f && (VEC || c + i < cols) ? fmaf(lg2_approx(w), kLn2, g[i]) : -INFINITY;
+        const float w = weight(t[i], fused(l[i], sl[i], pr[i]));
+        k[i] = w > kSmallWeight && (VEC || c + i < cols) ? fmaf(lg2_approx(w), kLn2, g[i]) : -INFINITY;
+      }
+      push8(k, max8(k), (int)(c0 + c), rb, rs, ri);
+    }
+  }
+  // the small weights, where they may count (kSmallWeight)
+  if (resid && rs < kSmallKey && (lo - lse_t) * kLog2e < -77.f) {
+#pragma unroll 1
+    for (int c = 8 * (int)threadIdx.x; c < cols; c += 8 * kSampleThreads) {
+      float t[8], l[8], sl[8], pr[8];
+      load8_row<TT, VEC>(trow, c, cols, t);
+      bool small = false;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float p = (t[i] - lse_t) * kLog2e;
+        small |= p < -77.f && p > -151.f;
+      }
+      if (!small) continue;
+      load_pair(c, l, sl, pr);
+      float g[8], k[8];
+      gumbel8(a.seed, a.step, b, acc, kStreamResidual, (c0 + c) >> 3, g);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float x = fused(l[i], sl[i], pr[i]);
+        const float w = __expf(t[i] - lse_t) - __expf(x - lse_q);
+        k[i] = w > 0.f && !(weight(t[i], x) > kSmallWeight) && (VEC || c + i < cols) ? __logf(w) + g[i] : -INFINITY;
       }
       push8(k, max8(k), (int)(c0 + c), rb, rs, ri);
     }

@@ -227,6 +227,30 @@ def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
         assert st & dels.DELS_STATUS_NONFINITE
 
 
+@pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("V", [72, 20000])
+def test_sampled_verify_denormal_residual(target_dtype, V):
+    """A residual whose every weight is a denormal float32 is drawn from, not
+    taken for zero: p and q agree on token 0 and only token 5 has p > q, by
+    e^-90 (a draft log-probability set far too high rejects token 0)."""
+    w = synth.stress(synth.Workload("denormal", B=2, n=1, V=V, logit_dtype="f32",
+                                    head=synth.HeadSpec("markov", "bf16", 0, 0, 64), weight=0.5, seed=3))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    d["long"].fill_(-200.0)
+    d["long"][:, :, 0] = 0.0
+    W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+    tok, lp, gap, state = dr.sample(d["long"], prior, [0.0], [0.0], 23, 7)
+    assert tok.tolist() == [[0], [0]]
+    target = torch.full((w.B, 2, V), -200.0, device=DEV)
+    target[:, :, 0] = 0.0
+    target[:, :, 5] = -90.0
+    acc, bonus, bgap, st = _verify_raw(w, d, W, [0.0], [0.0], tok, lp + 60.0, state, target.to(target_dtype), prior)
+    assert st == 0 and acc.tolist() == [0, 0]
+    assert bonus.tolist() == [5, 5] and np.all(np.isinf(bgap))
+
+
 @pytest.mark.parametrize("name", ["gru", "markov", "tiny"])
 def test_sampled_verify_rejection_at_position_zero(name):
     """The target rules out every x_0 (p_0(x_0) = 0): every request rejects at
