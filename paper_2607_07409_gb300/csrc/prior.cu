@@ -675,21 +675,24 @@ __global__ void __launch_bounds__(kMapThreads) k_prior_total(PriorLogArgs a) {
 
 // ln x of a positive, normal double by table lookup and a short series (Tang,
 // "Table-driven implementation of the logarithm function in IEEE
-// floating-point arithmetic", 1990): x = 2^e m, c the middle of the 1/128-wide
-// interval that holds m, r = m / c - 1 (|r| <= 2^-8), ln x = e ln 2 + ln c +
-// ln(1 + r); the series stops at r^4, an error below |r|^5 / 5 = 2e-13.
-// Float64 units are few here (two operations per cycle and SM): this is about
-// a quarter of log()'s operations. x outside [1e-300, 1e300] takes log().
+// floating-point arithmetic", 1990): x = 2^e m, c the middle of the 1/256-wide
+// interval that holds m, r = m / c - 1 (|r| <= 2^-9), ln x = e ln 2 + (ln c +
+// ln(1 + r)); the series stops at r^5, an error below |r|^6 / 6 = 1e-17, so
+// that the last rounding is what is left: at most 2.9e-15 for x < 2^40 (under
+// one unit in the last place). Float64 units are few here (two operations per
+// cycle and SM): this is about a quarter of log()'s operations. x outside
+// [1e-300, 1e300] takes log().
+constexpr int kLogIntervals = 256;
 struct LogEntry {
-  double inv, ln;   // 1 / c and ln c of interval i, c = 1 + (i + 1/2) / 128
+  double inv, ln;   // 1 / c and ln c of interval i, c = 1 + (i + 1/2) / 256
 };
 struct LogTable {
-  LogEntry e[128];
+  LogEntry e[kLogIntervals];
 };
 constexpr LogTable make_log_table() {
   LogTable t{};
-  for (int i = 0; i < 128; ++i) {
-    const double c = 1.0 + (i + 0.5) / 128.0;
+  for (int i = 0; i < kLogIntervals; ++i) {
+    const double c = 1.0 + (i + 0.5) / kLogIntervals;
     // ln c = 2 artanh z, z = (c - 1) / (c + 1) <= 1/3: terms below 3^-41 left out
     const double z = (c - 1.0) / (c + 1.0);
     double sum = 0.0;
@@ -704,34 +707,43 @@ __device__ __forceinline__ double log_table(double x, const LogEntry* tab) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) - 1023;
   const double m = __hiloint2double((hi & 0x000FFFFF) | 0x3FF00000, __double2loint(x));
-  const LogEntry t = tab[(hi >> 13) & 127];
+  const LogEntry t = tab[(hi >> 12) & (kLogIntervals - 1)];
   const double r = fma(m, t.inv, -1.0);
-  double p = fma(r, -0.25, 1.0 / 3.0);
+  double p = fma(r, 0.2, -0.25);
+  p = fma(r, p, 1.0 / 3.0);
   p = fma(r, p, -0.5);
   p = fma(r * r, p, r);
-  return fma((double)e, 0.693147180559945309417, t.ln) + p;
+  return fma((double)e, 0.693147180559945309417, t.ln + p);
 }
 
 // l_P(v) = log(c(v) + lambda) - log(sum_u c(u) + V lambda), in float64,
-// stored as float32. Optionally copies the counts and the tally out (the
-// one-call estimate keeps both in its workspace).
+// stored as float32. The one id that may hold more than half of the sum takes
+// log1p of the others' share instead: there the two logarithms cancel.
+// Optionally copies the counts and the tally out (the one-call estimate keeps
+// both in its workspace).
 __global__ void __launch_bounds__(kThreads) k_prior_log(PriorLogArgs a) {
-  __shared__ LogEntry tab[128];
-  __shared__ double log_s_sh;
+  __shared__ LogEntry tab[kLogIntervals];
+  __shared__ double sum_sh, log_s_sh;
   const double lam = a.lambda;
   if (threadIdx.x == 0) pdl_trigger();
-  if (threadIdx.x < 128) tab[threadIdx.x] = kLogTable.e[threadIdx.x];
+  for (int i = threadIdx.x; i < kLogIntervals; i += blockDim.x) tab[i] = kLogTable.e[i];
   __syncthreads();
   // lambda may be any positive float64, denormal or large
   auto ln = [&](double x) { return x >= 1e-300 && x <= 1e300 ? log_table(x, tab) : log(x); };
   pdl_wait();
-  if (threadIdx.x == 0) log_s_sh = ln((double)__ldcg(a.total) + (double)a.V * lam);
+  if (threadIdx.x == 0) {
+    sum_sh = (double)__ldcg(a.total) + (double)a.V * lam;
+    log_s_sh = ln(sum_sh);
+  }
   __syncthreads();
-  const double log_s = log_s_sh;
+  const double half = 0.5 * sum_sh, log_s = log_s_sh;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.V; v += stride) {
     const unsigned long long c = __ldcg(a.counts + v);
-    a.out[v] = (float)(ln((double)c + lam) - log_s);
+    const double x = (double)c + lam;
+    double l = ln(x) - log_s;
+    if (x > half) l = log1p(-((double)(__ldcg(a.total) - c) + (a.V - 1) * lam) / sum_sh);
+    a.out[v] = (float)l;
     if (a.counts_out) a.counts_out[v] = c;
   }
   if (a.tally_out && blockIdx.x == 0 && threadIdx.x < 2) a.tally_out[threadIdx.x] = __ldcg(a.tally + threadIdx.x);
