@@ -516,19 +516,23 @@ struct DraftLayout {
 };
 
 // How the GRU's rank and recurrent products share the chip: as many K splits
-// of the rank product as keep it within a quarter of the SMs (four up to rank
-// 288, two to 608, then one), the rest to the recurrent product; from rank
-// 2432 on, where less than half is left, the recurrent product gets a CTA for
-// every SM, which come in as the rank product's finish. 64 requests, block of
-// 11, V 24008, state 1024, no table; four splits throughout with what they
-// leave for the recurrent product / this rule / the recurrent product beside
-// the input product and the rank product alone: rank 512 320 / 319 / 417 us,
-// 1024 450 / 364 / 489, 1216 929 / 425 / 521, 2048 977 / 452 / 622, 4096 1296 /
-// 683 / 871.
-void share_rank_hh(int R, int sms, int& rank_splits, int& hh_ctas) {
-  const int tiles = (R + kRankTile - 1) / kRankTile;
+// of the rank product as keep it within half of the SMs (four up to rank 608,
+// two to 1216, then one) and cost the recurrent product no further round of
+// its tiles; the rest to the recurrent product; from rank 2433 on, where less
+// than half is left, a CTA for every SM, which come in as the rank product's
+// finish. 64 requests, block of 11, V 24008, no table; four splits throughout
+// with what they leave for the recurrent product / this rule / the recurrent
+// product beside the input product and the rank product alone, as it once was:
+// state 1024, rank 512 305 / 305 / 392 us, 768 337 / 326 / 421, 1024 434 / 349 /
+// 463, 1216 910 / 411 / 503, 2048 960 / 437 / 601, 4096 1271 / 664 / 853; state
+// 2048, rank 512 423 / 357 / 541, 1024 681 / 405 / 608, 4096 2667 / 782 / 988.
+// (Within a quarter of the SMs: rank 1024 and state 1024 the same, but 8
+// requests, state 592, rank 336 51.0 -> 52.5 for a block of 3.)
+void share_rank_hh(int H, int R, int sms, int& rank_splits, int& hh_ctas) {
+  const int tiles = (R + kRankTile - 1) / kRankTile, hh_tiles = (3 * H + kHhTile - 1) / kHhTile;
+  auto rounds = [&](int s) { return (hh_tiles + sms - tiles * s - 1) / (sms - tiles * s); };
   rank_splits = kRankSplits;
-  while (rank_splits > 1 && tiles * rank_splits > sms / 4) rank_splits /= 2;
+  while (rank_splits > 1 && (tiles * rank_splits > sms / 2 || rounds(rank_splits) > rounds(1))) rank_splits /= 2;
   const int rest = sms - tiles * rank_splits;
   hh_ctas = rest >= sms / 2 ? rest : sms;
 }
@@ -554,7 +558,7 @@ DraftLayout draft_layout(const dels_local_head* hd, int B, int n, int V) {
       if (bf) {
         L.gru_s0 = std::max(1, std::min((D + 63) / 64, sms / std::max(1, (3 * H + 127) / 128) - 1));
         L.gru_s1 = 1;
-        share_rank_hh(R, sms, L.rank_splits, L.hh_ctas);
+        share_rank_hh(H, R, sms, L.rank_splits, L.hh_ctas);
         L.hh_splits = splits_for(3 * H, kHhTile, H, L.hh_ctas);
         L.ih_splits = splits_for(3 * H, 128, D, sms);
       } else {

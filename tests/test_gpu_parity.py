@@ -290,10 +290,12 @@ def test_draft_wide_gru_state(h, table):
 
 
 @pytest.mark.parametrize("table", [False, True])
-@pytest.mark.parametrize("r", [288, 304, 608, 624, 2432, 2448])   # 4 | 2 | 1 K splits of W_rank h; W_hh h on every SM
-def test_draft_gru_rank_shares(r, table):
+@pytest.mark.parametrize("h,r", [(512, 608), (512, 624), (512, 1216), (512, 1232),     # 4 | 2 | 1 K splits of W_rank h
+                                 (512, 2432), (512, 2448),                             # W_hh h on what is left | every SM
+                                 (1888, 512), (1904, 512)])                            # 4 | 2: a further round of W_hh h
+def test_draft_gru_rank_shares(h, r, table):
     """Both sides of each line in how the rank and recurrent products share the chip."""
-    spec = synth.HeadSpec("gru", "bf16", 128, 512, r)
+    spec = synth.HeadSpec("gru", "bf16", 128, h, r)
     w = synth.stress(synth.Workload("rank", B=5, n=4, V=3000, logit_dtype="bf16", head=spec, weight=1.0, seed=r))
     d = synth.make_inputs(w, device=DEV, target=False)
     if table:
