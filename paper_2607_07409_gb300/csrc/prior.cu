@@ -717,13 +717,15 @@ __device__ __forceinline__ double log_table(double x, const LogEntry* tab) {
 }
 
 // l_P(v) = log(c(v) + lambda) - log(sum_u c(u) + V lambda), in float64,
-// stored as float32. The one id that may hold more than half of the sum takes
-// log1p of the others' share instead: there the two logarithms cancel.
+// stored as float32. An id that holds all but y < 2^-10 of the sum takes
+// ln(1 - y) = -(y + y^2 / 2 + ... + y^5 / 5) (the rest is below y 2^-52) from
+// the others' share y instead: there the two logarithms cancel.
 // Optionally copies the counts and the tally out (the one-call estimate keeps
 // both in its workspace).
 __global__ void __launch_bounds__(kThreads) k_prior_log(PriorLogArgs a) {
   __shared__ LogEntry tab[kLogIntervals];
   __shared__ double sum_sh, log_s_sh;
+  __shared__ unsigned long long half_sh;
   const double lam = a.lambda;
   if (threadIdx.x == 0) pdl_trigger();
   for (int i = threadIdx.x; i < kLogIntervals; i += blockDim.x) tab[i] = kLogTable.e[i];
@@ -732,17 +734,21 @@ __global__ void __launch_bounds__(kThreads) k_prior_log(PriorLogArgs a) {
   auto ln = [&](double x) { return x >= 1e-300 && x <= 1e300 ? log_table(x, tab) : log(x); };
   pdl_wait();
   if (threadIdx.x == 0) {
+    half_sh = __ldcg(a.total) / 2;
     sum_sh = (double)__ldcg(a.total) + (double)a.V * lam;
     log_s_sh = ln(sum_sh);
   }
   __syncthreads();
-  const double half = 0.5 * sum_sh, log_s = log_s_sh;
+  const double log_s = log_s_sh;
+  const unsigned long long half = half_sh;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.V; v += stride) {
     const unsigned long long c = __ldcg(a.counts + v);
-    const double x = (double)c + lam;
-    double l = ln(x) - log_s;
-    if (x > half) l = log1p(-((double)(__ldcg(a.total) - c) + (a.V - 1) * lam) / sum_sh);
+    double l = ln((double)c + lam) - log_s;
+    if (c > half) {   // (at most one id, or two halves)
+      const double y = ((double)(__ldcg(a.total) - c) + (a.V - 1) * lam) * (1.0 / sum_sh);
+      if (y < 0x1p-10) l = -y * fma(y, fma(y, fma(y, fma(y, 0.2, 0.25), 1.0 / 3.0), 0.5), 1.0);
+    }
     a.out[v] = (float)l;
     if (a.counts_out) a.counts_out[v] = c;
   }
