@@ -14,9 +14,9 @@
 //   16-bit bins, two to a word, that each fit (115K ids a slice); P groups of
 //   CTAs read the same positions (the second reading hits L2), each counting
 //   one slice, and the bins of a group's CTAs are summed at the end
-//   (k_prior_halves_reduce). A bin that reaches 2^15 hands 2^15 to the global
-//   count, so it never carries into its neighbour. Used over long ranges for
-//   vocabularies that two slices cover.
+//   (k_prior_halves_reduce). A bin past 2^15 hands 2^15 to the global count
+//   before it can carry into its neighbour (wait_handed_off). Used over long
+//   ranges for vocabularies that two slices cover.
 // * Slice histograms (k_prior_slices): the same with 32-bit bins, added to
 //   the counts by atomics: short ranges, small vocabularies, and the prefix
 //   of the hot scheme.
@@ -48,7 +48,8 @@ constexpr int kMapThreads = 256;             // the V-sized maps (sum, log)
 constexpr int kWarpSpan = 512;               // positions a warp takes per vector step
 constexpr int kSelectBuckets = kPriorHistBuckets;   // count buckets of the hot-set choice (32 x 118)
 constexpr int kIdsPerWord = 15;              // remap word: 15 presence bits + a 17-bit slot number
-constexpr unsigned kFlush = 0x8000u;         // a 16-bit hot bin hands this to the global count
+constexpr unsigned kFlush = 0x8000u;         // a 16-bit bin hands this to the global count
+constexpr int kMaxPolls = 1 << 22;           // of a wait for a hand-off (tens of milliseconds)
 
 struct Tally {   // per thread; a thread sees far fewer than 2^32 positions per launch
   unsigned in = 0, out = 0;
@@ -125,29 +126,50 @@ __device__ __forceinline__ void visit(const PriorRange& r, long long worker, lon
   }
 }
 
-// One position of a half-word slice: adds `one` (1 or 2^16, by the bin's half)
-// to the word of id's bin if its mask byte is set and id lies in [lo, lo + nb);
-// returns the word before the add, or 0 if there was none. Written as
+// The 16-bit bins of the half-word slices, two to a word of shared memory. A
+// bin never carries into its neighbour: of the adds that meet it at 2^15 or
+// more (their old value), the one that meets 2^15 exactly hands 2^15 to the
+// global count and takes it off the bin at once; a thread whose add met more
+// waits for that at the end of its warp's round of at most four positions a
+// lane. So every thread has at most four adds in a bin past 2^15, 4096 of a
+// CTA's, where 2^15 are left; and as all of a warp's lanes have handed over
+// before any of them waits, no wait depends on another. (2^28 positions of
+// 151936 ids 375 -> 363 us against a test for the crossing and no wait, which
+// took an addition more per position.)
+__device__ __forceinline__ unsigned half_of(unsigned word, unsigned u) { return (u & 1u) ? word >> 16 : word & 0xFFFFu; }
+
+__device__ __noinline__ void wait_handed_off(const unsigned* word, unsigned u, int* status) {
+  const volatile unsigned* w = word;
+  for (int polls = 0; half_of(*w, u) > kFlush; ++polls) {
+    if (polls == kMaxPolls) {
+      raise_status(status, DELS_STATUS_TIMEOUT);
+      return;
+    }
+  }
+}
+
+// One position of a half-word slice: adds 1 to id's bin if its mask byte is set
+// and id lies in [lo, lo + nb); returns the word before the add, or 0 if there
+// was none. Written as
 // predicated instructions: as C++ conditionals the compiler branched around
 // each add (20.7 instructions per position instead of 19.8).
 template <int Q>
-__device__ __forceinline__ unsigned count_half(unsigned id, uint32_t mk, unsigned lo, unsigned nb, unsigned base2,
-                                               unsigned& one) {
+__device__ __forceinline__ unsigned count_half(unsigned id, uint32_t mk, unsigned lo, unsigned nb, unsigned base2) {
   unsigned old;
   asm volatile(
-      "{\n\t.reg .pred p, h;\n\t.reg .u32 t, v;\n\t"
-      "and.b32 t, %3, %4;\n\t"
+      "{\n\t.reg .pred p, h;\n\t.reg .u32 t, v, one;\n\t"
+      "and.b32 t, %2, %3;\n\t"
       "setp.ne.u32 p, t, 0;\n\t"
-      "sub.u32 t, %2, %5;\n\t"
-      "setp.lt.and.u32 p, t, %6, p;\n\t"
-      "mad.lo.u32 v, %2, 2, %7;\n\t"
+      "sub.u32 t, %1, %4;\n\t"
+      "setp.lt.and.u32 p, t, %5, p;\n\t"
+      "mad.lo.u32 v, %1, 2, %6;\n\t"
       "and.b32 t, v, 2;\n\t"
       "setp.ne.u32 h, t, 0;\n\t"
-      "selp.u32 %1, 65536, 1, h;\n\t"
+      "selp.u32 one, 65536, 1, h;\n\t"
       "and.b32 v, v, -4;\n\t"
       "mov.u32 %0, 0;\n\t"
-      "@p atom.shared.add.u32 %0, [v], %1;\n\t}"
-      : "=&r"(old), "=&r"(one)
+      "@p atom.shared.add.u32 %0, [v], one;\n\t}"
+      : "=&r"(old)
       : "r"(id), "r"(mk), "n"(0xFFu << (8 * Q)), "r"(lo), "r"(nb), "r"(base2)
       : "memory");
   return old;
@@ -175,40 +197,46 @@ __global__ void __launch_bounds__(kThreads, 1) k_prior_halves(PriorHalvesArgs a)
   pdl_wait();
   const int lane = threadIdx.x & 31;
   Tally t;
-  // bin u has reached 2^15: its word goes back by that much
-  auto hand_off = [&](unsigned u) {
-    atomicSub(words + (u >> 1), (u & 1u) ? 0x80000000u : 0x8000u);
-    atomicAdd(a.counts + lo + u, 1ull << 15);
-    t.in += 1u << 15;
+  // an add met `word` in id u's bin; whether a hand-off is to be waited for
+  auto met = [&](unsigned word, unsigned u) {
+    const unsigned old = half_of(word, u);
+    if (old == kFlush) {
+      atomicSub(words + (u >> 1), kFlush << ((u & 1u) << 4));
+      atomicAdd(a.counts + lo + u, (unsigned long long)kFlush);
+      t.in += kFlush;
+    }
+    return old > kFlush;
   };
   const PriorRange& r = a.range;
   const long long nworkers = (long long)members * kWarps;
   const long long steps = r.nvec / kWarpSpan;
   const int4* tv = reinterpret_cast<const int4*>(r.tokens + r.head);
   const uint32_t* mv = reinterpret_cast<const uint32_t*>(r.mask + r.head);
-  // Four positions at a time: the adds go out together, then one test for
-  // their hand-offs. (A bin has room for 2^15 more adds between reaching 2^15
-  // and the subtraction, eight from every quad of the CTA's threads.)
   const unsigned base2 = smem_u32(words) - 2u * lo;   // byte address of bin u's half word: 2 id + base2
+  // four positions at a time: the adds go out together, then one test of what
+  // they met (no add: 0)
   auto quad = [&](const int4& tk, uint32_t mk, auto tally) {
     unsigned old[4];
-    unsigned flips = 0;   // bit 15 of a bin changes only when it reaches 2^15
-    unsigned one[4];
-    old[0] = count_half<0>((unsigned)tk.x, mk, lo, nb, base2, one[0]);
-    old[1] = count_half<1>((unsigned)tk.y, mk, lo, nb, base2, one[1]);
-    old[2] = count_half<2>((unsigned)tk.z, mk, lo, nb, base2, one[2]);
-    old[3] = count_half<3>((unsigned)tk.w, mk, lo, nb, base2, one[3]);
+    old[0] = count_half<0>((unsigned)tk.x, mk, lo, nb, base2);
+    old[1] = count_half<1>((unsigned)tk.y, mk, lo, nb, base2);
+    old[2] = count_half<2>((unsigned)tk.z, mk, lo, nb, base2);
+    old[3] = count_half<3>((unsigned)tk.w, mk, lo, nb, base2);
+    if constexpr (decltype(tally)::value) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      flips |= old[q] ^ (old[q] + one[q]);
-      if constexpr (decltype(tally)::value)
+      for (int q = 0; q < 4; ++q)
         t.out += (mk & (0xFFu << (8 * q))) != 0u && (unsigned)int4_at(tk, q) >= (unsigned)a.V ? 1u : 0u;
     }
-    if (flips & 0x80008000u) {
+    if (__any_sync(0xFFFFFFFFu, ((old[0] | old[1]) | (old[2] | old[3])) & 0x80008000u)) {
+      unsigned late = 0;   // adds that met a bin past 2^15
+#pragma unroll
+      for (int q = 0; q < 4; ++q) late |= met(old[q], (unsigned)int4_at(tk, q) - lo) ? 1u << q : 0u;
+      __syncwarp();        // every lane has handed over
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        if ((old[q] ^ (old[q] + one[q])) & 0x80008000u) hand_off((unsigned)int4_at(tk, q) - lo);
+        const unsigned u = (unsigned)int4_at(tk, q) - lo;
+        if (late & (1u << q)) wait_handed_off(words + (u >> 1), u, a.status);
       }
+      __syncwarp();
     }
   };
   for (long long st = (long long)member * kWarps + (threadIdx.x >> 5); st < steps; st += nworkers) {
@@ -228,17 +256,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_prior_halves(PriorHalvesArgs a)
     }
   }
   const long long rest = r.n - r.nvec;
-  for (long long j = ((long long)member * kWarps + (threadIdx.x >> 5)) * 32 + lane; j < rest; j += nworkers * 32) {
-    const long long i = j < r.head ? j : j + r.nvec;
-    const int id = r.tokens[i];
-    if (!r.mask[i]) continue;
-    if (g == 0 && (unsigned)id >= (unsigned)a.V) ++t.out;
-    const unsigned u = (unsigned)id - lo;
-    if (u < nb) {
-      const unsigned one = (u & 1u) ? 0x10000u : 1u;
-      const unsigned old = atomicAdd(words + (u >> 1), one);
-      if ((old ^ (old + one)) & 0x80008000u) hand_off(u);
-    }
+  for (long long j0 = ((long long)member * kWarps + (threadIdx.x >> 5)) * 32; j0 < rest; j0 += nworkers * 32) {
+    const long long j = j0 + lane, i = j < r.head ? j : j + r.nvec;
+    const bool masked = j < rest && r.mask[i] != 0;
+    const unsigned id = masked ? (unsigned)r.tokens[i] : 0u, u = id - lo;
+    if (masked && g == 0 && id >= (unsigned)a.V) ++t.out;
+    const bool late = masked && u < nb && met(atomicAdd(words + (u >> 1), (u & 1u) ? 0x10000u : 1u), u);
+    __syncwarp();
+    if (late) wait_handed_off(words + (u >> 1), u, a.status);
   }
   __syncthreads();
   uint4* out = reinterpret_cast<uint4*>(a.partials + ((long long)g * members + member) * kw);
@@ -251,7 +276,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_prior_halves(PriorHalvesArgs a)
 // memory, and each thread adds one id's total.
 __global__ void __launch_bounds__(256) k_prior_halves_reduce(PriorHalvesArgs a) {
   __shared__ __align__(8) unsigned sums[8][32][9];
-  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
   const int kw4 = a.slice / 8;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
@@ -276,6 +300,7 @@ __global__ void __launch_bounds__(256) k_prior_halves_reduce(PriorHalvesArgs a) 
       }
     }
   }
+  if (threadIdx.x == 0) pdl_trigger();   // not before: two CTAs of the logarithm's map fill an SM
 #pragma unroll
   for (int i = 0; i < 8; ++i) sums[y][x][i] = s[i];
   __syncthreads();
@@ -544,9 +569,13 @@ __global__ void __launch_bounds__(kMapThreads) k_prior_place(PriorSelectArgs a) 
 }
 
 // Main pass over a long range: loss-masked hot ids are counted in 16-bit
-// shared-memory bins (two per word; a bin that reaches 2^15 hands 2^15 to the
-// global count, so it never carries into its neighbour), the others go to the
-// global counts directly. Writes the CTA's bin words to partials.
+// shared-memory bins, two per word; the thread whose add brings a bin to 2^15
+// hands 2^15 to the global count with its next instructions. That no bin
+// carries into its neighbour rests on a margin here, not on a wait: the CTA's
+// other threads would have to make 2^15 more adds to the bin in between, 32
+// each. (Waits as in k_prior_halves, a vote for every four positions, took 2^28
+// positions of 250000 ids from 473 to 598 us.) The other ids go to the global
+// counts directly. Writes the CTA's bin words to partials.
 __global__ void __launch_bounds__(kThreads, 1) k_prior_hot(PriorHotArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint32_t* ent = reinterpret_cast<uint32_t*>(smem_raw);

@@ -259,6 +259,21 @@ def test_half_word_slices_match_oracle(V, N):
     _check_log_prior(out, c_ref, 1.0)
 
 
+@pytest.mark.parametrize("V", [100000, 151936, 250000])   # one and two half-word slices, the hot scheme
+@pytest.mark.parametrize("ids", [[77776], [77777], [77776, 77777], [77776, 77777, 77776, 3]])
+def test_bins_under_one_or_two_ids(V, ids):
+    """A range of one or two ids, the two halves of one word of bins: every
+    add of a CTA meets the same word, and every bin hands over many times."""
+    N = (1 << 25) + 19
+    tok = torch.tensor(ids, dtype=torch.int32, device=DEV).repeat((N + len(ids) - 1) // len(ids))[:N].contiguous()
+    mask = torch.ones(N, dtype=torch.uint8, device=DEV)
+    ref = np.bincount(tok.cpu().numpy(), minlength=V)
+    for _ in range(3):
+        out, c, tally = _estimate(tok, mask, V)
+        np.testing.assert_array_equal(c, ref)
+        assert tally.tolist() == [N, 0]
+
+
 @pytest.mark.parametrize("lam", [5e-324, 1e-310, 1e-5, 0.3, 3e7, 1e301])
 def test_log_prior_over_smoothing_weights(lam):
     """The table-driven logarithm and, outside [1e-300, 1e300], the general one."""
