@@ -273,7 +273,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_prior_halves(PriorHalvesArgs a)
 
 // counts[v] += the sum over a group's members of bin v: a thread takes four
 // words (eight ids) of every eighth member, the eight sums meet in shared
-// memory, and each thread adds one id's total.
+// memory, and each thread adds one id's total (atomically: pieces may be counted
+// on several streams at a time).
 __global__ void __launch_bounds__(256) k_prior_halves_reduce(PriorHalvesArgs a) {
   __shared__ __align__(8) unsigned sums[8][32][9];
   pdl_wait();
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(256) k_prior_halves_reduce(PriorHalvesArgs a) 
   for (int k = 0; k < 8; ++k) total += sums[k][xi][i];
   const int u = blockIdx.x * 256 + threadIdx.x;
   const long long v = (long long)blockIdx.y * a.slice + u;
-  if (u < a.slice && v < a.V && total) a.counts[v] += total;
+  if (u < a.slice && v < a.V && total) atomicAdd(a.counts + v, (unsigned long long)total);
   if (a.tally) {
     const unsigned long long in = warp_sum_u64(total);
     __syncthreads();
@@ -667,8 +668,8 @@ __global__ void __launch_bounds__(kMapThreads) k_prior_hot_reduce(PriorHotArgs a
         hi += x[k] >> 16;
       }
     }
-    if (lo) a.counts[__ldcg(a.slot_id + 2 * w)] += lo;
-    if (hi && 2 * w + 1 < n_hot) a.counts[__ldcg(a.slot_id + 2 * w + 1)] += hi;
+    if (lo) atomicAdd(a.counts + __ldcg(a.slot_id + 2 * w), lo);
+    if (hi && 2 * w + 1 < n_hot) atomicAdd(a.counts + __ldcg(a.slot_id + 2 * w + 1), hi);
   }
 }
 

@@ -274,6 +274,27 @@ def test_bins_under_one_or_two_ids(V, ids):
         assert tally.tolist() == [N, 0]
 
 
+@pytest.mark.parametrize("V", [100000, 151936, 250000])
+def test_pieces_counted_on_several_streams(V):
+    """Pieces with workspaces of their own, counted at the same time into one
+    set of counts."""
+    N, S = (1 << 24) + 512, 3
+    g = torch.Generator(device=DEV).manual_seed(V)
+    tok = torch.randint(0, V, (N,), generator=g, device=DEV, dtype=torch.int32)
+    mask = torch.ones(N, dtype=torch.uint8, device=DEV)
+    one = torch.bincount(tok, minlength=V)
+    streams = [torch.cuda.Stream() for _ in range(S)]
+    ws = [_ws(V, N) for _ in range(S)]
+    for _ in range(5):
+        counts = torch.zeros(V, dtype=torch.int64, device=DEV)
+        tally = torch.zeros(2, dtype=torch.int64, device=DEV)
+        torch.cuda.synchronize()
+        for s, (w, nbytes) in zip(streams, ws):
+            assert dels.dels_prior_count(tok, mask, N, V, counts, tally, w, nbytes, stream=s) == 0
+        torch.cuda.synchronize()
+        assert torch.equal(counts, S * one) and tally.tolist() == [S * N, 0]
+
+
 @pytest.mark.parametrize("lam", [5e-324, 1e-310, 1e-5, 0.3, 3e7, 1e301])
 def test_log_prior_over_smoothing_weights(lam):
     """The table-driven logarithm and, outside [1e-300, 1e300], the general one."""
