@@ -108,20 +108,39 @@ __device__ __forceinline__ float lg2_approx(float x) {
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.693147180559945309f;
 
+// exp(x - ref) = 2^(x log2e - ref log2e) with the second product rounded once is
+// off by a factor of up to 2^(|ref| 2^-24): below the rounding of the row's LSE
+// up to this bound, but without one for masks such as -1e9, -1e30 or the type's
+// lowest value, where it overflows. Past the bound, where a row's largest
+// element so far is a mask, the difference is taken first, in place (a loop of
+// its own beside the hot one took 64 requests' block from 450 to 453 us; this
+// way 450, one MLP request 867 -> 873, temperature 1 572 -> 576).
+constexpr float kMaxRef = 4096.f;
+__device__ __forceinline__ bool past_ref_bound(float ref) { return !(fabsf(ref) <= kMaxRef); }
+
 // lse_chunk with the exponent pre-scaled to base 2: one FFMA + one ex2 per
 // element (exp(x - best) = 2^(x*log2e - best*log2e)). The running sum is
 // rescaled only when the maximum moved (rare after the first chunks).
 template <int K>
 __device__ __forceinline__ void lse_chunk_ex2(const float (&x)[K], float best, float& m, float& s) {
-  if (best == -INFINITY) return;
-  const float nb = -best * kLog2e;
-  if (best != m) {
+  float y[K];
+#pragma unroll
+  for (int i = 0; i < K; ++i) y[i] = x[i];
+  float nb = -best * kLog2e;
+  if (past_ref_bound(best)) {
+    if (best == -INFINITY) return;
+    s *= ex2_approx((m - best) * kLog2e);      // m == -inf -> 0 (s was 0)
+    m = best;
+    nb = 0.f;
+#pragma unroll
+    for (int i = 0; i < K; ++i) y[i] -= best;
+  } else if (best != m) {
     s *= ex2_approx(fmaf(m, kLog2e, nb));
     m = best;
   }
   float acc = 0.f;
 #pragma unroll
-  for (int i = 0; i < K; ++i) acc += ex2_approx(fmaf(x[i], kLog2e, nb));
+  for (int i = 0; i < K; ++i) acc += ex2_approx(fmaf(y[i], kLog2e, nb));
   s += acc;
 }
 
@@ -208,7 +227,8 @@ __device__ __forceinline__ RowAcc rowacc_warp_reduce(const RowAcc& a) {
 // row's top-1 nor its top-2 whichever lane holds it, so the top-2 update runs
 // only where a lane meets an element at or above T: of a warp's n-th group of
 // 256 elements about 2/n do, where a lane's own runner-up would let 64/n
-// through and some lane of the warp nearly always.
+// through and some lane of the warp nearly always. (T is -inf, and every group
+// let through, while the reference is past kMaxRef.)
 struct WarpRow {
   float best, second, s;   // per lane; s relative to the warp's reference
   int idx;
@@ -222,14 +242,16 @@ struct WarpRow {
   // While nothing finite has been met the values are -inf (0) or NaN (NaN).
   template <int G>
   __device__ __forceinline__ void push(const float (&f)[G][8], const int (&c)[G]) {
-    float vm[G], top = -INFINITY;
+    float y[G][8], vm[G], top = -INFINITY;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) y[g][i] = f[g][i];
       vm[g] = fmaxf(fmaxf(fmaxf(f[g][0], f[g][1]), fmaxf(f[g][2], f[g][3])),
                     fmaxf(fmaxf(f[g][4], f[g][5]), fmaxf(f[g][6], f[g][7])));
       top = fmaxf(top, vm[g]);
     }
-    if (__any_sync(0xFFFFFFFFu, top >= T && top > second)) {
+    if (__any_sync(0xFFFFFFFFu, top >= T)) {
 #pragma unroll
       for (int g = 0; g < G; ++g)
         if (vm[g] > second) {
@@ -240,7 +262,15 @@ struct WarpRow {
       const float old = ref;
       ref = warp_max(best);
       T = warp_max(best == ref ? second : best);
-      if (ref != old) {
+      if (past_ref_bound(ref) && ref != -INFINITY) {
+        if (old != ref && old != -INFINITY) s *= ex2_approx((old - ref) * kLog2e);
+        T = -INFINITY;
+        nb = 0.f;
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) y[g][i] -= ref;
+      } else if (ref != old) {
         nb = -ref * kLog2e;
         if (old != -INFINITY) s *= ex2_approx(fmaf(old, kLog2e, nb));
       }
@@ -249,14 +279,14 @@ struct WarpRow {
 #pragma unroll
     for (int g = 0; g < G; ++g)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i & 1] += ex2_approx(fmaf(f[g][i], kLog2e, nb));
+      for (int i = 0; i < 8; ++i) acc[i & 1] += ex2_approx(fmaf(y[g][i], kLog2e, nb));
     s += acc[0] + acc[1];
   }
   // The warp's record, in every lane.
   __device__ __forceinline__ RowAcc record() const {
     RowAcc r;
     r.m = ref;
-    r.second = T;
+    r.second = warp_max(best == ref ? second : best);
     r.idx = __reduce_min_sync(0xFFFFFFFFu, best == ref ? idx : 0x7FFFFFFF);
     // a tie for the top in two lanes: the runner-up equals the top
     if (__popc(__ballot_sync(0xFFFFFFFFu, best == ref)) > 1) r.second = ref;

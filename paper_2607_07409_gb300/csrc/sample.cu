@@ -138,13 +138,24 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
   const T* src = static_cast<const T*>(a.src) + row * a.ld + c0;
   const int cols = (int)min((long long)a.chunk_cols, a.V - c0);
   float m = -INFINITY, s = 0.f, nb = 0.f;      // nb = -m log2(e), 0 while m is -inf
+  float gate = -INFINITY;                      // m, or -inf while m is past kMaxRef
   // Eight values with maximum vm (NaN ignored). While m is -inf they are -inf
   // (0) or NaN (NaN).
-  auto push = [&](const float (&x)[8], float vm) {
-    if (vm > m) {
-      nb = -vm * kLog2e;
-      if (m != -INFINITY) s *= ex2_approx(fmaf(m, kLog2e, nb));
-      m = vm;
+  auto push = [&](float (&x)[8], float vm) {
+    if (vm > gate) {
+      const float old = m;
+      m = fmaxf(m, vm);
+      if (past_ref_bound(m)) {
+        if (old != -INFINITY) s *= ex2_approx((old - m) * kLog2e);
+        nb = 0.f;
+        gate = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] -= m;
+      } else {
+        nb = -m * kLog2e;
+        gate = m;
+        if (old != -INFINITY) s *= ex2_approx(fmaf(old, kLog2e, nb));
+      }
     }
     float e[2] = {0.f, 0.f};
 #pragma unroll

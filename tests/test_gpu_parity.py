@@ -112,6 +112,51 @@ def test_combine_masked_and_nonfinite_rows(V):
     assert tok[1] == -1 and tok[2] == -1 and tok[3] == -1
 
 
+MASKS = ["lowest", -1e30, -1e9, -65504.0]
+
+
+def _mask_value(x, mask):
+    return torch.finfo(x.dtype).min if mask == "lowest" else mask
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("mask", MASKS)
+@pytest.mark.parametrize("rows,V", [(6, 2048), (6, 2003), (6, 40000), (800, 20000)])   # row kernel, element by element, ...
+def test_combine_rows_masked_by_a_finite_value(rows, V, mask, dtype):
+    """Masks that are finite: leading stretches, most of a row, all of it but one
+    entry, all of it (uniform), and rows far from zero. The masked entries are
+    what a thread or a warp meets first."""
+    g = torch.Generator(device=DEV).manual_seed(V)
+    long = (torch.randn(rows, V, generator=g, device=DEV) * 3).to(dtype)
+    m = _mask_value(long, mask)
+    long[0::6, : 3 * V // 4] = m
+    long[1::6][torch.rand(len(long[1::6]), V, generator=g, device=DEV) < 0.95] = m
+    one = long[2::6, V - 3].clone()
+    long[2::6] = m
+    long[2::6, V - 3] = one
+    long[3::6] = m
+    long[4::6] += 1e5
+    long[5::6, : V // 2] = m                       # and a lower mask before it
+    long[5::6, : V // 4] = torch.finfo(dtype).min
+    tok, lp, gap, st = _combine(long, None, None, 0.0, 0.0)
+    assert st == 0
+    rt, rl, rg = oracle.combine_argmax(long.cpu(), None, None, 0.0, 0.0)
+    rl[3::6] = -np.log(V)                          # (the oracle's l - LSE absorbs it at 1e9 and more)
+    check_rows(tok, lp, np.minimum(gap, 1e4), rt, rl, np.minimum(rg, 1e4), exact_ties=True)
+
+
+@pytest.mark.parametrize("mask", MASKS)
+@pytest.mark.parametrize("name", ["gru", "gru_b100", "mlp2", "markov", "markov_f32", "gru_f32"])
+def test_draft_rows_masked_by_a_finite_value(name, mask):
+    w = synth.stress(SMALL[name])
+    d = synth.make_inputs(w, device=DEV, target=False)
+    d["long"][:, :, : w.V // 2] = _mask_value(d["long"], mask)
+    d["long"][0, 1, : w.V - 20] = _mask_value(d["long"], mask)
+    tok, lp, gap, W, prior = _draft(w, d)
+    tol = LP_TOL_F32 if w.head.wdtype == "f32" else LP_TOL_BF16
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, tol)
+
+
 def test_combine_nonfinite_rows_among_many():
     """A NaN, an all-masked row and an infinite entry among 400 rows each give
     token -1 and the status flag; the other rows match the oracle."""

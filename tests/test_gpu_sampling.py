@@ -227,6 +227,34 @@ def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
         assert st & dels.DELS_STATUS_NONFINITE
 
 
+@pytest.mark.parametrize("mask", ["lowest", -1e30, -1e9])
+@pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
+def test_sampled_rows_masked_by_a_finite_value(target_dtype, mask):
+    """Draft and target rows whose leading half, and nearly all of one row, hold
+    a finite mask."""
+    w = synth.stress(SMALL["gru"])
+    d = synth.make_inputs(w, device=DEV, target=False)
+    value = torch.finfo(torch.bfloat16).min if mask == "lowest" else mask
+    d["long"][:, :, : w.V // 2] = value
+    a, b = _learned_weights(w.n)
+    W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+    tok, lp, gap, state = dr.sample(d["long"], prior, a, b, 23, 7)
+    torch.cuda.synchronize()
+    assert dr.status() == 0
+    tok, lp, gap = tok.cpu().numpy(), lp.cpu().numpy(), gap.cpu().numpy()
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), oracle.log_prior(d["counts"]), np.array(a),
+                np.array(b), LP_TOL_BF16, sample=(23, 7))
+    target = synth.make_target_logits(w, d["long"], device=DEV).to(target_dtype)
+    target[:, :, : w.V // 2] = torch.finfo(target_dtype).min if mask == "lowest" else mask
+    target[1, 2, : w.V - 9] = value
+    acc, bonus, bgap, st = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+    assert st == 0
+    info = _check_verify(w, d, W, a, b, tok, acc, bonus, bgap, target, 23, 7, LP_TOL_BF16)
+    assert info["requests"] == w.B
+
+
 @pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("V", [72, 20000])
 def test_sampled_verify_denormal_residual(target_dtype, V):
