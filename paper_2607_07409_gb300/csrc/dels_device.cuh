@@ -80,7 +80,12 @@ __device__ __forceinline__ void top2_push(float x, int v, float& best, float& se
 // been pushed (so `best` is the new running max); `m` is the old max.
 template <int K>
 __device__ __forceinline__ void lse_chunk(const float (&x)[K], float best, float& m, float& s) {
-  if (best == -INFINITY) return;               // chunk and history all -inf
+  if (best == -INFINITY) {                     // chunk and history all -inf or NaN
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      if (x[i] != x[i]) s = NAN;
+    return;
+  }
   s *= __expf(m - best);                       // m == -inf -> 0 (s was 0)
   m = best;
   float acc = 0.f;
@@ -128,12 +133,13 @@ __device__ __forceinline__ void lse_chunk_ex2(const float (&x)[K], float best, f
   for (int i = 0; i < K; ++i) y[i] = x[i];
   float nb = -best * kLog2e;
   if (past_ref_bound(best)) {
-    if (best == -INFINITY) return;
-    s *= ex2_approx((m - best) * kLog2e);      // m == -inf -> 0 (s was 0)
-    m = best;
     nb = 0.f;
+    if (best != -INFINITY) {                   // else all -inf (0 each) or NaN (NaN)
+      s *= ex2_approx((m - best) * kLog2e);    // m == -inf -> 0 (s was 0)
+      m = best;
 #pragma unroll
-    for (int i = 0; i < K; ++i) y[i] -= best;
+      for (int i = 0; i < K; ++i) y[i] -= best;
+    }
   } else if (best != m) {
     s *= ex2_approx(fmaf(m, kLog2e, nb));
     m = best;

@@ -502,6 +502,24 @@ def test_draft_fused_products_vocab_staged_activations(B, r, monkeypatch):
     check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
 
 
+@pytest.mark.parametrize("name", ["gru", "gru_b100", "markov", "gru_f32"])
+@pytest.mark.parametrize("sampled", [False, True])
+def test_draft_nan_among_masked_entries(name, sampled):
+    """A NaN that a thread meets among -inf entries alone, before or without
+    anything finite, is flagged like any other."""
+    w = synth.stress(SMALL[name])
+    d = synth.make_inputs(w, device=DEV, target=False)
+    d["long"][:, :, : w.V // 2] = -float("inf")
+    d["long"][1, 2, 33] = float("nan")
+    W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+    tok = (dr.sample(d["long"], prior, w.alpha, w.beta, 5, 6) if sampled else dr(d["long"], prior, w.alpha, w.beta))[0]
+    assert dr.status() == dels.DELS_STATUS_NONFINITE
+    bad = (tok == -1).cpu().numpy()
+    assert bad[1, 2] and bad.sum() == 1
+
+
 def _learned_weights(n):
     """Per-position (alpha_j, beta_j) from the Appendix C table (positions 2..15
     are j = 1..14; later positions keep the last printed value)."""
