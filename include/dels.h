@@ -24,6 +24,9 @@
  *   and 16-byte aligned. Pointers marked [host] are ordinary host memory.
  * - Calls are asynchronous on the given stream (a cudaStream_t; NULL is the
  *   legacy default stream) and never synchronise, except dels_read_status.
+ *   They start after the work issued to the stream before them, also behind a
+ *   kernel that lets its dependents launch early: nothing that such a kernel
+ *   writes is read before it has finished.
  * - The library allocates no memory and keeps no state between calls, with
  *   one exception: dels_combine_argmax_noalloc keeps a fixed scratch array per
  *   device and caches its address (see there). Every other

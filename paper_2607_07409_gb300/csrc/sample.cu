@@ -130,8 +130,10 @@ __global__ void __launch_bounds__(kSampleThreads) k_sample_rows(SampleRowsArgs a
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_rows(SampleRowsArgs a) {
   __shared__ RowAcc red[kSampleThreads / 32];
-  if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
+  // not before: launches of this call read weights ahead of their own wait, and
+  // the weights may be the work of this launch's predecessor
+  if (threadIdx.x == 0) pdl_trigger();
   const int chunk = blockIdx.x % a.nchunks;
   const long long row = blockIdx.x / a.nchunks;
   const long long c0 = (long long)chunk * a.chunk_cols;

@@ -227,6 +227,58 @@ def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
         assert st & dels.DELS_STATUS_NONFINITE
 
 
+def test_sampled_verify_right_behind_the_launch_that_writes_its_weights():
+    """W_vocab of a float32 head written by a launch that lets its successors
+    start early (an input table, 48 wide): the verification called right behind
+    it reads the new weights."""
+    V, R, B, n = 100000, 48, 2, 3
+    g = torch.Generator(device=DEV).manual_seed(4)
+    gru = synth.HeadSpec("gru", "bf16", 4096, R // 3, 16)
+    E = torch.randn(V, 4096, generator=g, device=DEV).to(torch.bfloat16)
+    Wih = torch.randn(R, 4096, generator=g, device=DEV).to(torch.bfloat16) / 64
+    maker = dels.make_head(gru, {"emb": E, "w_ih": Wih, "w_vocab": E})
+    G = torch.empty(V, R, device=DEV)
+    ws = torch.zeros(256, dtype=torch.uint8, device=DEV)
+
+    def write_weights():
+        assert dels.dels_gru_build_input_table(maker, V, G, V * R * 4, ws, 256) == 0
+
+    write_weights()
+    w = synth.Workload("behind", B=B, n=n, V=V, logit_dtype="f32", head=synth.HeadSpec("markov", "f32", 0, 0, R),
+                       weight=1.0, seed=3)
+    W = {"emb": torch.randn(V, R, generator=g, device=DEV) * 0.3, "w_vocab": G}
+    d = {"long": torch.randn(B, n, V, generator=g, device=DEV) * 2}
+    prior = torch.full((V,), -float(np.log(V)), device=DEV)
+    a = b = [1.0] * n
+    dr = dels.Drafter(w.head, W, B, n, V)
+    tok, lp, gap, state = dr.sample(d["long"], prior, a, b, 23, 7)
+    lp = lp + torch.tensor([-50.0, 50.0, 0.0], device=DEV)       # accepted, then rejected: q is rebuilt from W_vocab
+    target = torch.randn(B, n + 1, V, generator=g, device=DEV) * 2
+    head = dels.make_head(w.head, W)
+    nbytes = dels.dels_verify_sampled_workspace_bytes(head, B, n, V, dels.DELS_F32)
+    vws = torch.zeros(nbytes, dtype=torch.uint8, device=DEV)
+    acc, bonus = (torch.empty(B, dtype=torch.int32, device=DEV) for _ in range(2))
+    bgap = torch.empty(B, dtype=torch.float32, device=DEV)
+
+    def verify():                                 # no launch but the library's in between
+        assert dels.dels_verify_block_sampled(head, tok, lp, state, d["long"], dels.DELS_F32, prior, a, b, target,
+                                              dels.DELS_F32, B, n, V, 23, 7, acc, bonus, bgap, vws, nbytes) == 0
+
+    def results():
+        assert dels.dels_read_status(vws) == 0
+        return acc.tolist(), bonus.tolist(), bgap.tolist()
+
+    verify()
+    want = results()
+    assert want[0] == [1] * B
+    for _ in range(5):
+        G.fill_(3.0)
+        torch.cuda.synchronize()
+        write_weights()
+        verify()
+        assert results() == want
+
+
 @pytest.mark.parametrize("mask", ["lowest", -1e30, -1e9])
 @pytest.mark.parametrize("target_dtype", [torch.float32, torch.bfloat16])
 def test_sampled_rows_masked_by_a_finite_value(target_dtype, mask):
