@@ -8,6 +8,7 @@
 // row split over several CTAs is finished by the last CTA to arrive (atomic
 // ticket, reset by that CTA), so no [rows, V] intermediate is ever written.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <type_traits>
 
@@ -551,7 +552,7 @@ RowsPlan plan_rows(int rows, int V, int bytes_per_col, int num_sms, bool vec, in
 int rows_slots_per_sm(bool verify, dels_dtype dt) {
   // resident CTAs per SM of the main instantiation (all four combine
   // variants use the same registers to within a few), queried once
-  static int cache[4] = {-1, -1, -1, -1};
+  static std::atomic<int> cache[4] = {{-1}, {-1}, {-1}, {-1}};
   const int k = (verify ? 2 : 0) + (dt == DELS_F32 ? 1 : 0);
   if (cache[k] < 0) {
     int n = 0;

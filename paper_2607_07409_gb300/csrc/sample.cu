@@ -13,6 +13,7 @@
 //   p_n. q_a is rebuilt from the drafting's kept state: the fused row
 //   l_L + alpha_a W_vocab r_a - beta_a l_P and its LSE.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "dels_device.cuh"
@@ -488,7 +489,7 @@ cudaError_t launch_lse_rows(const SampleRowsArgs& a, bool f32, cudaStream_t s) {
 }
 
 int lse_slots_per_sm(bool f32) {
-  static int cache[2] = {-1, -1};   // a property of the kernel, queried once
+  static std::atomic<int> cache[2] = {{-1}, {-1}};   // a property of the kernel, queried once
   if (cache[f32] < 0) {
     int n = 0;
     const cudaError_t e =

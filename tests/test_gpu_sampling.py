@@ -227,6 +227,47 @@ def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
         assert st & dels.DELS_STATUS_NONFINITE
 
 
+def test_calls_from_several_host_threads():
+    """Blocks drafted and verified by threads with streams and workspaces of
+    their own, all at once, equal the same calls made one after another."""
+    import threading
+    names = ["gru", "gru_f32", "markov", "gru_b64"]
+    jobs = []
+    for name in names:
+        w = synth.stress(SMALL[name])
+        d = synth.make_inputs(w, device=DEV, target=False)
+        W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+        a, b = _learned_weights(w.n)
+        jobs.append((w, d, W, a, b, dels.dels_prior_from_counts(d["counts"]).to(DEV),
+                     synth.make_target_logits(w, d["long"], device=DEV)))
+
+    def one(job, rounds):
+        w, d, W, a, b, prior, target = job
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(rounds):
+                dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+                tok, lp, gap, state = dr.sample(d["long"], prior, a, b, 23, 7)
+                acc, bonus, bgap, st = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+            torch.cuda.current_stream().synchronize()
+            return [x.cpu().numpy() for x in (tok, lp, gap)] + [acc, bonus, bgap, np.array([st, dr.status()])]
+
+    torch.cuda.synchronize()
+    want = [one(j, 1) for j in jobs]
+    got = [None] * len(jobs)
+
+    def run(i):
+        got[i] = one(jobs[i], 8)
+
+    threads = [threading.Thread(target=run, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for x, y in zip(got, want):
+        for u, v in zip(x, y):
+            np.testing.assert_array_equal(u, v)
+
+
 def test_sampled_verify_right_behind_the_launch_that_writes_its_weights():
     """W_vocab of a float32 head written by a launch that lets its successors
     start early (an input table, 48 wide): the verification called right behind
