@@ -126,9 +126,10 @@ __device__ __forceinline__ void stage_rows(float* sx, const float* X, long long 
   __syncthreads();
 }
 
-// Y[b, o] = act(sum_k X[b, k] W[o, k]) for up to two independent products
-// with the same O (blockIdx.z). MERGE: the first product's input is the head
-// input of the position that m decodes (merge_requests), not X. KS warps split each row group's K (their sums
+// Y[b, o] = act(sum_k X[b, k] W[o, k]) for up to two independent products with
+// the same O (blockIdx.z); blockIdx.x: request group, blockIdx.y: row groups.
+// MERGE: the first product's input is the head input of the position that m
+// decodes (merge_requests), not X. KS warps split each row group's K (their sums
 // are added in order), so that small matrices still fill the chip.
 template <int R, int BG, bool STAGED, bool VEC, bool MERGE>
 __global__ void __launch_bounds__(kThreadsF32, 2)
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(kThreadsF32, 2)
   constexpr int NV = R * BG;
   if (threadIdx.x == 0 && !jobs.late) pdl_trigger();
   const GemvF32Job& jb = jobs.j[blockIdx.z];
-  const int b0 = blockIdx.y * BG, nb = min(BG, B - b0);
+  const int b0 = blockIdx.x * BG, nb = min(BG, B - b0);
   const int K = jb.K;
   const float* X = jb.X + (long long)b0 * jb.ldx;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -149,11 +150,11 @@ __global__ void __launch_bounds__(kThreadsF32, 2)
   const int k0 = (kw * 32 + lane) * 4;
   // the first weights go out before the wait: they are not the predecessor's
   float4 w[R];
-  load_rows<R, VEC>(jb.W, blockIdx.x * per + rg * R, O - 1, K, k0, w);
+  load_rows<R, VEC>(jb.W, blockIdx.y * per + rg * R, O - 1, K, k0, w);
   pdl_wait();
   if (threadIdx.x == 0 && jobs.late) pdl_trigger();
   if (MERGE && blockIdx.z == 0) {
-    const bool writer = blockIdx.x == 0;
+    const bool writer = blockIdx.y == 0;
     merge_requests(m, b0, nb, writer, s_tok);
     if (writer)
       for (int q = 0; q < nb; ++q) keep_draft_input(m.smp, b0 + q, m.n, m.j);
@@ -168,10 +169,10 @@ __global__ void __launch_bounds__(kThreadsF32, 2)
   }
   const int idx = lane / (32 / NV), r = idx / BG, b = idx % BG;
   const bool leader = lane % (32 / NV) == 0;
-  for (int base = blockIdx.x * per; base < O; base += gridDim.x * per) {
+  for (int base = blockIdx.y * per; base < O; base += gridDim.y * per) {
     const int o0 = base + rg * R;
     float acc[NV];
-    if (base > (int)(blockIdx.x * per)) load_rows<R, VEC>(jb.W, o0, O - 1, K, k0, w);
+    if (base > (int)(blockIdx.y * per)) load_rows<R, VEC>(jb.W, o0, O - 1, K, k0, w);
     dot_rows<R, BG, STAGED, VEC>(jb.W, o0, O - 1, K, STAGED ? sx : X, jb.ldx, nb, k0, KS * 128, w, acc);
     float s = transpose_reduce<NV>(acc);
     if (KS > 1) {
@@ -299,7 +300,6 @@ cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, in
   const bool stage = staged(bg, K);
   if (merge && (!stage || !vec)) return cudaErrorInvalidValue;
   const int groups = (B + bg - 1) / bg;
-  if (groups > 65535) return cudaErrorInvalidValue;
   // K split over the warps of a CTA until about eight warps per SM have work
   // (a split keeps at least one 128-wide step)
   const long long tasks = (long long)((O + R - 1) / R) * groups * njobs;
@@ -307,7 +307,7 @@ cudaError_t launch_gemv_f32(const GemvF32Jobs& jobs, int njobs, int B, int O, in
   while (KS < kWarpsF32 && tasks * KS < 8LL * sms && K >= 256 * KS) KS *= 2;
   const int per = kWarpsF32 / KS * R;
   const int ctas = std::min((O + per - 1) / per, std::max(1, 8 * sms / (groups * njobs)));
-  const dim3 grid((unsigned)ctas, (unsigned)groups, (unsigned)njobs);
+  const dim3 grid((unsigned)groups, (unsigned)ctas, (unsigned)njobs);   // ctas: at most 8 per SM
   const size_t smem = stage ? (size_t)bg * K * 4 : 0;
   switch (bg) {
     case 1: return launch_gemv_bg<8, 1>(jobs, B, O, act, ldy, stage, vec, KS, grid, smem, merge, s);

@@ -227,6 +227,24 @@ def test_sampled_verify_nonfinite_target_rows(target_dtype, what):
         assert st & dels.DELS_STATUS_NONFINITE
 
 
+def test_sampled_verify_of_every_request_that_a_counter_holds():
+    """65536 requests and a float32 width whose products take one request per
+    CTA: more groups than a launch has rows of CTAs."""
+    B, n, V, R = 65536, 1, 8, 12292
+    w = synth.Workload("many", B=B, n=n, V=V, logit_dtype="f32", head=synth.HeadSpec("markov", "f32", 0, 0, R),
+                       weight=1.0, seed=3)
+    W = {"emb": torch.zeros(V, R, device=DEV), "w_vocab": torch.zeros(V, R, device=DEV)}
+    state = torch.zeros(B * n * (R + 1) * 4 + 4096, dtype=torch.uint8, device=DEV)   # every q and input zero
+    tok = torch.zeros(B, n, dtype=torch.int32, device=DEV)
+    lp = torch.full((B, n), -60.0, device=DEV)                                       # p / q large: accepted
+    lp[1::2] = 60.0                                                                  # rejected
+    rows = torch.zeros(B, n, V, device=DEV)
+    target = torch.zeros(B, n + 1, V, device=DEV)
+    acc, bonus, bgap, st = _verify_raw(w, {"long": rows}, W, [0.0], [0.0], tok, lp, state, target,
+                                       torch.zeros(V, device=DEV))
+    assert st == 0 and np.array_equal(acc, 1 - np.arange(B) % 2) and np.all((bonus >= 0) & (bonus < V))
+
+
 def test_calls_from_several_host_threads():
     """Blocks drafted and verified by threads with streams and workspaces of
     their own, all at once, equal the same calls made one after another."""
