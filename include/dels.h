@@ -410,9 +410,11 @@ size_t dels_prior_workspace_bytes(int V, int64_t N);
  *        counted, tally[1] += loss-masked positions with an id outside [0, V).
  * workspace [device] >= dels_prior_workspace_bytes(V, N) (a workspace sized
  * for the longest piece serves every piece).
- * Large vocabularies count long pieces in two steps: the first positions
- * exactly, then the rest with the ids that are most frequent in `counts` so
- * far held on chip; the result is the exact count either way.
+ * Pieces may be counted into one set of counts on several streams at a time,
+ * each with its own workspace. Vocabularies above about 230,000 ids count
+ * pieces of 2^24 positions and more in two steps, the first positions exactly,
+ * then the rest with the ids that are most frequent in `counts` so far held on
+ * chip; the result is the exact count however a piece is counted.
  * Limits: N >= 0 (N = 0 enqueues nothing), 1 <= V < 2^31.
  */
 int dels_prior_count(const int32_t* tokens, const uint8_t* loss_mask, int64_t N, int V, uint64_t* counts,

@@ -157,15 +157,17 @@ def test_full_corpus_counts_match_oracle():
     _check_log_prior(out, c_ref, 1.0)
 
 
-# ------------------------------------------------------------- the hot/cold path
-# (large vocabularies over long ranges: a prefix counted exactly, the most
-# frequent ids so far on chip, the others through per-CTA cold buffers)
+# ------------------------------------------------------------- long ranges of large vocabularies
+# Vocabularies above 230400 ids: the hot/cold scheme (a prefix counted exactly,
+# the most frequent ids so far on chip, the others added to the global counts
+# directly). Up to that, the half-word slices; each test runs on both.
 
 HOT_N = (1 << 24) + 1234
+HALVES_V, HOT_V = 151936, 250000
 
 
-def test_hot_cold_path_matches_oracle_with_bad_ids():
-    V = 151936
+@pytest.mark.parametrize("V", [HALVES_V, HOT_V])
+def test_hot_cold_path_matches_oracle_with_bad_ids(V):
     tok, mask = _corpus(V, HOT_N, 8, bad=101)
     c_ref, n_in, n_out = oracle.count_masked_tokens(tok.numpy(), mask.numpy(), V)
     ws, nbytes = _ws(V, HOT_N)
@@ -179,10 +181,10 @@ def test_hot_cold_path_matches_oracle_with_bad_ids():
     _check_log_prior(out, c_ref, 1.0)
 
 
-def test_hot_cold_path_when_the_prefix_misleads():
+@pytest.mark.parametrize("V", [HALVES_V, HOT_V])
+def test_hot_cold_path_when_the_prefix_misleads(V):
     """The prefix holds one id only, the rest is uniform over V: almost every
-    later position is cold and the cold buffers overflow into direct adds."""
-    V = 151936
+    later position is cold and is added to the global counts."""
     g = torch.Generator().manual_seed(9)
     tok = torch.randint(0, V, (HOT_N,), generator=g, dtype=torch.int32)
     tok[: 1 << 23] = 77
@@ -193,9 +195,9 @@ def test_hot_cold_path_when_the_prefix_misleads():
     assert tally.tolist() == [n_in, n_out]
 
 
-def test_hot_cold_pieces_on_top_of_earlier_counts():
+@pytest.mark.parametrize("V", [HALVES_V, HOT_V])
+def test_hot_cold_pieces_on_top_of_earlier_counts(V):
     """A second long piece chooses its hot set from counts that already hold the first."""
-    V = 151936
     tok, mask = _corpus(V, 2 * HOT_N, 10)
     t_dev, m_dev = tok.to(DEV), mask.to(DEV)
     ws, nbytes = _ws(V, HOT_N)
@@ -209,23 +211,25 @@ def test_hot_cold_pieces_on_top_of_earlier_counts():
     assert tally.cpu().tolist() == [n_in, 0]
 
 
-def test_hot_path_hand_off_of_a_single_id():
-    """One id at every loss-masked position of a hot-path range: every CTA's
-    16-bit bin for it passes 2^15 twice and hands it to the global count."""
-    V, N = 151936, HOT_N
+@pytest.mark.parametrize("V", [HALVES_V, HOT_V])
+def test_hot_path_hand_off_of_a_single_id(V):
+    """One id at every loss-masked position of a long range: every CTA's 16-bit
+    bin for it passes 2^15 twice and hands it to the global count."""
+    N = HOT_N if V == HALVES_V else 2 * HOT_N     # the hot scheme's bins start after its prefix
     tok = torch.full((N,), 4242, dtype=torch.int32)
     mask = torch.full((N,), 3, dtype=torch.uint8)
     mask[::3] = 0
     out, c, tally = _estimate(tok.to(DEV), mask.to(DEV), V)
     expect = int((mask != 0).sum())
-    assert expect // torch.cuda.get_device_properties(0).multi_processor_count > 2 * 2 ** 15
+    counted = expect - ((1 << 22) if V == HOT_V else 0)
+    assert counted // torch.cuda.get_device_properties(0).multi_processor_count > 2 * 2 ** 15
     assert c[4242] == expect and c.sum() == expect and tally.tolist() == [expect, 0]
 
 
-def test_hot_path_vocabulary_a_multiple_of_15_with_bad_ids():
-    """V = 15 * 10129: an id clamped to V falls on the remap table's zero
-    sentinel word, past the last word that holds vocabulary ids."""
-    V = 151935
+@pytest.mark.parametrize("V", [15 * 10129, 15 * 16666])
+def test_hot_path_vocabulary_a_multiple_of_15_with_bad_ids(V):
+    """An id clamped to V falls on the remap table's zero sentinel word, past the
+    last word that holds vocabulary ids."""
     tok, mask = _corpus(V, HOT_N, 11, bad=57)
     c_ref, n_in, n_out = oracle.count_masked_tokens(tok.numpy(), mask.numpy(), V)
     out, c, tally = _estimate(tok.to(DEV), mask.to(DEV), V)
