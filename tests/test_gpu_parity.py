@@ -368,6 +368,21 @@ def test_draft_staged_activation_edges(B, r, ldt):
     check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
 
 
+@pytest.mark.parametrize("B,n,d,heads", [
+    (10, 4, 256, 4), (11, 4, 256, 4),      # the terms' rows fill one TMEM quadrant / one row more
+    (3, 17, 256, 4), (3, 18, 256, 4),      # 16 older positions at most / a second group of them
+    (2, 32, 256, 4),                       # the longest block
+    (2, 19, 2176, 2), (1, 5, 1088, 1),     # heads wider than a CTA's threads
+    (2, 6, 240, 15), (1, 4, 16, 1),        # narrow ones
+])
+def test_draft_transformer_edges(B, n, d, heads):
+    spec = synth.HeadSpec("xfmr", "bf16", d, 512, d, n_heads=heads, max_pos=n)
+    w = synth.stress(synth.Workload("xfmr_edges", B=B, n=n, V=1536, logit_dtype="f32", head=spec, weight=0.5, seed=B + n))
+    dd = synth.make_inputs(w, device=DEV, target=False)
+    tok, lp, gap, W, prior = _draft(w, dd)
+    check_draft(tok, lp, gap, _oracle_head(w, W), dd["long"].cpu(), prior, w.alpha, w.beta, LP_TOL_BF16)
+
+
 @pytest.mark.parametrize("head,B,V,d,h,r", [
     ("gru", 1, 1000, 132, 36, 20),          # one request; widths just past and below a 128-wide step
     ("gru", 2, 72, 8, 4, 4),                # two requests, the smallest widths

@@ -71,6 +71,47 @@ def test_sampled_draft_staged_activation_edges(B, r, ldt):
                 oracle.log_prior(d["counts"]), np.array(a), np.array(b), LP_TOL_BF16, sample=(17, 3))
 
 
+@pytest.mark.parametrize("layers,B,V", [(2, 3, 1024), (2, 9, 1024), (1, 3, 1024), (2, 9, 4096)])
+def test_sampled_f32_mlp_merged_in_its_first_product(layers, B, V):
+    """A float32 MLP's first product decodes the position before it, and keeps
+    that position's feature: two layers with few records (the fused launch),
+    one layer and many records (a merge launch of its own)."""
+    spec = synth.HeadSpec("mlp", "f32", 32, 100, 100, window=3, n_layers=layers)
+    w = synth.stress(synth.Workload("f32_mlp", B=B, n=5, V=V, logit_dtype="f32", head=spec, weight=0.5, seed=B))
+    d = synth.make_inputs(w, device=DEV, target=False)
+    a, b = _learned_weights(w.n)
+    W = {k[5:]: v for k, v in d.items() if k.startswith("head.")}
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    dr = dels.Drafter(w.head, W, w.B, w.n, w.V)
+    tok, lp, gap, state = dr.sample(d["long"], prior, a, b, 23, 7)
+    torch.cuda.synchronize()
+    assert dr.status() == 0
+    tok, lp, gap = tok.cpu().numpy(), lp.cpu().numpy(), gap.cpu().numpy()
+    check_draft(tok, lp, gap, _oracle_head(w, W), d["long"].cpu(), oracle.log_prior(d["counts"]), np.array(a),
+                np.array(b), LP_TOL_F32, sample=(23, 7))
+    # the kept features, through the verification that rebuilds q from them
+    target = synth.make_target_logits(w, d["long"], device=DEV)
+    acc, bonus, bgap, st = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+    assert st == 0
+    _check_verify(w, d, W, a, b, tok, acc, bonus, bgap, target, 23, 7, LP_TOL_F32)
+
+
+@pytest.mark.parametrize("offset", [1, 2])
+def test_sampled_verify_unaligned_f32_weights(offset):
+    """A float32 W_vocab off its 16-byte boundary gives the results of an aligned one."""
+    w, d, W, a, b, tok, lp, gap, state = _sampled("gru_f32", 23, 7)
+    target = synth.make_target_logits(w, d["long"], device=DEV)
+    prior = dels.dels_prior_from_counts(d["counts"]).to(DEV)
+    one = _verify_raw(w, d, W, a, b, tok, lp, state, target, prior)
+    wv = W["w_vocab"]
+    shifted = torch.empty(wv.numel() + 4, device=DEV)[offset:offset + wv.numel()].view_as(wv)
+    shifted.copy_(wv)
+    two = _verify_raw(w, d, dict(W, w_vocab=shifted), a, b, tok, lp, state, target, prior)
+    assert one[3] == 0 and two[3] == 0
+    for x, y in zip(one, two):
+        np.testing.assert_array_equal(x, y)
+
+
 def test_sampled_calls_reject_a_step_outside_the_counter_word():
     w = synth.stress(SMALL["gru"])
     d = synth.make_inputs(w, device=DEV, target=False)
