@@ -189,6 +189,9 @@ bool map_w(CUtensorMap* m, const void* W, int O, int K, int n_tile) {
 // other data out (64 requests 463 and 479, one request 949, 8 requests 3033).
 // Below 30 MB the matrix stays there anyway (25 MB: 344 us, kept 346).
 // Temperature-1 launches are bound by their variates (586 -> 587) and keep none.
+// Two blocks at once, on two streams, keep twice that between them: none kept ->
+// 32 MB each, two of the 64-request blocks 816 -> 810 us a pair, two MLP requests
+// 1568 -> 1590, the transformer and a 64-request block 3143 -> 3169.
 float keep_share(size_t bytes) {
   return bytes <= 30000000 ? 0.f : std::min(1.f, 32e6f / (float)bytes);
 }
@@ -383,9 +386,13 @@ bool plan_combine(Gemm& g, int B, int V, int n, const void* X, int K, const void
   // single 457; K 1536: 637 and 631; K 4096: 1592 and 1494).
   int pairs = std::min(a.stages / 2, (smem - (a.a_resident ? a_all : 0)) / (2 * stage));
   // Few packed rows would leave room for six pairs; the last ones only keep
-  // the neighbouring launches' CTAs off the SM (3 / 4 / 5 / 6 pairs: one MLP
-  // request, K 1024 899 / 885 / 895 / 907 us; 8 transformer requests, K 2560
-  // 2928 / 2878 / 2865 / 2904).
+  // the neighbouring launches' CTAs off the SM. Blocks of 8, V 151936, float32
+  // logits, 3 / 4 / 5 / 6 pairs: MLP heads, one request, K 512 245 / 245 / 247 /
+  // 249 us, 1024 392 / 387 / 387 / 394, 1536 556 / 544 / 549 / 554, 2048 719 /
+  // 709 / 707 / 723, 4096 1473 / 1436 / 1424 / 1460; 24 requests, 512 304 / 300 /
+  // 305 / 305, 1024 476 / 471 / 467 / 467, 2560 995 / 972 / 955 / 955; Markov
+  // heads, one request, 1024 336 / 331 / 328 / 330, 4096 1335 / 1293 / 1274 /
+  // 1312: four or five within 1 % of each other between K 512 and 1536.
   if (!a.a_resident) pairs = std::min(pairs, a.seg_chunks[0] <= 16 ? 4 : 5);
   if (pair_stages && K % 128 == 0 && pairs >= (a.a_resident || a.seg_chunks[0] <= 16 ? 2 : 3)) {
     a.b_chunks = 2;
