@@ -150,9 +150,8 @@ __device__ __noinline__ void wait_handed_off(const unsigned* word, unsigned u, i
 
 // One position of a half-word slice: adds 1 to id's bin if its mask byte is set
 // and id lies in [lo, lo + nb); returns the word before the add, or 0 if there
-// was none. Written as
-// predicated instructions: as C++ conditionals the compiler branched around
-// each add (20.7 instructions per position instead of 19.8).
+// was none. Written as predicated instructions: as C++ conditionals the compiler
+// branched around each add, an instruction more per position.
 template <int Q>
 __device__ __forceinline__ unsigned count_half(unsigned id, uint32_t mk, unsigned lo, unsigned nb, unsigned base2) {
   unsigned old;
@@ -176,8 +175,8 @@ __device__ __forceinline__ unsigned count_half(unsigned id, uint32_t mk, unsigne
 }
 
 // Half-word slices. CTA b counts slice b % P over the positions its group
-// member index b / P takes. Issue-bound, about 20 instructions per position and
-// group: the bin's word and half follow from the id directly, where the hot
+// member index b / P takes. Issue-bound, 18.5 instructions per position and
+// group (75 % issue active): the bin's word and half follow from the id directly, where the hot
 // scheme looks its slot up (about 43 per position). Out-of-range ids are
 // tallied by one group for each vector step, so that the groups do equal work;
 // the positions counted are the sum of the bins, which go to the partials.
@@ -808,7 +807,7 @@ PriorPlan plan_prior(int V, long long N, int sms) {
   // place of two or three 32-bit ones, from 2^23 positions on (151936 ids, both
   // with the same logarithm kernel's older form: 2^22 positions 29 us as 32-bit
   // slices, 33 as halves; 2^24 - 1 positions 58 and 52; against the hot scheme
-  // 2^24 positions 100 and 52, 2^28 466 and 376).
+  // 2^24 positions 100 and 52, 2^28 466 and 376; 49 and 362 with the bins' waits).
   const long long half_max = (smem - 2048) / 2 / 8 * 8;
   const long long halves = ((long long)V + half_max - 1) / half_max;
   if (p.slices > 1 && halves <= 2 && N >= kPriorHalvesMinN) {

@@ -118,7 +118,7 @@ __device__ __forceinline__ void block_reduce_rows(const RowAcc (&acc)[R], RowAcc
 // bf16 rows are close to issue-bound: 1024 rows of 151936 with both terms took
 // 126 us and 87 M warp instructions (17.9 per element) with a top-2 per thread,
 // whose update some lane of the warp needed for nearly every group, and tests
-// on every load; 106 us and 55 M (11.3) with the top-2 pruned by the warp's
+// on every load; 101 to 105 us and 56 M (11.5) with the top-2 pruned by the warp's
 // runner-up (WarpRow) and a loop of whole blocks (115 us with the loop alone).
 // ----------------------------------------------------------------------------
 template <typename T, int R, bool VEC, bool SH, bool PR, bool FINAL>
