@@ -229,12 +229,13 @@ __device__ __forceinline__ RowAcc rowacc_warp_reduce(const RowAcc& a) {
 // One row scanned by a whole warp, all lanes together: each lane keeps the
 // top-2 of its own elements and its share of the sum of exponentials, and the
 // warp shares the reference of the sums (the largest element met, nb =
-// -ref log2(e)) and its runner-up T. An element below T changes neither the
-// row's top-1 nor its top-2 whichever lane holds it, so the top-2 update runs
-// only where a lane meets an element at or above T: of a warp's n-th group of
-// 256 elements about 2/n do, where a lane's own runner-up would let 64/n
-// through and some lane of the warp nearly always. (T is -inf, and every group
-// let through, while the reference is past kMaxRef.)
+// -ref log2(e)) and its runner-up T. An element at or below T changes neither
+// the row's top-1 (columns only increase: of equal ones the first stays) nor its
+// top-2, whichever lane holds it, so the top-2 update runs only where a lane
+// meets an element above T: of a warp's n-th group of 256 elements about 2/n do,
+// where a lane's own runner-up would let 64/n through and some lane of the warp
+// nearly always. (T is -inf, and every group with an element above that let
+// through, while the reference is past kMaxRef.)
 struct WarpRow {
   float best, second, s;   // per lane; s relative to the warp's reference
   int idx;
@@ -257,7 +258,7 @@ struct WarpRow {
                     fmaxf(fmaxf(f[g][4], f[g][5]), fmaxf(f[g][6], f[g][7])));
       top = fmaxf(top, vm[g]);
     }
-    if (__any_sync(0xFFFFFFFFu, top >= T)) {
+    if (__any_sync(0xFFFFFFFFu, top > T)) {
 #pragma unroll
       for (int g = 0; g < G; ++g)
         if (vm[g] > second) {
@@ -265,11 +266,11 @@ struct WarpRow {
           for (int i = 0; i < 8; ++i) top2_push(f[g][i], c[g] + i, best, second, idx);
         }
       __syncwarp();
-      const float old = ref;
+      const float old = ref;                   // (-inf: s, 0 or NaN, times 0)
       ref = warp_max(best);
       T = warp_max(best == ref ? second : best);
-      if (past_ref_bound(ref) && ref != -INFINITY) {
-        if (old != ref && old != -INFINITY) s *= ex2_approx((old - ref) * kLog2e);
+      if (past_ref_bound(ref)) {               // something was above T: ref is not -inf
+        s *= ex2_approx((old - ref) * kLog2e);
         T = -INFINITY;
         nb = 0.f;
 #pragma unroll
@@ -278,7 +279,7 @@ struct WarpRow {
           for (int i = 0; i < 8; ++i) y[g][i] -= ref;
       } else if (ref != old) {
         nb = -ref * kLog2e;
-        if (old != -INFINITY) s *= ex2_approx(fmaf(old, kLog2e, nb));
+        s *= ex2_approx(fmaf(old, kLog2e, nb));
       }
     }
     float acc[2] = {0.f, 0.f};

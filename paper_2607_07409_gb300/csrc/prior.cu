@@ -709,8 +709,9 @@ __global__ void __launch_bounds__(kMapThreads) k_prior_total(PriorLogArgs a) {
 // ln(1 + r)); the series stops at r^5, an error below |r|^6 / 6 = 1e-17, so
 // that the last rounding is what is left: at most 2.9e-15 for x < 2^40 (under
 // one unit in the last place). Float64 units are few here (two operations per
-// cycle and SM): this is about a quarter of log()'s operations. x outside
-// [1e-300, 1e300] takes log().
+// cycle and SM): this is about a quarter of log()'s operations. A denormal or
+// infinite x takes log() (is_normal_positive, by integers: with two float64
+// comparisons 200000 ids took 1.2 us more).
 constexpr int kLogIntervals = 256;
 struct LogEntry {
   double inv, ln;   // 1 / c and ln c of interval i, c = 1 + (i + 1/2) / 256
@@ -731,6 +732,11 @@ constexpr LogTable make_log_table() {
   return t;
 }
 __device__ const LogTable kLogTable = make_log_table();
+
+// 2^-1022 <= x < infinity
+__device__ __forceinline__ bool is_normal_positive(double x) {
+  return (unsigned)__double2hiint(x) - 0x00100000u < 0x7FF00000u - 0x00100000u;
+}
 
 __device__ __forceinline__ double log_table(double x, const LogEntry* tab) {
   const int hi = __double2hiint(x);
@@ -760,7 +766,7 @@ __global__ void __launch_bounds__(kThreads) k_prior_log(PriorLogArgs a) {
   for (int i = threadIdx.x; i < kLogIntervals; i += blockDim.x) tab[i] = kLogTable.e[i];
   __syncthreads();
   // lambda may be any positive float64, denormal or large
-  auto ln = [&](double x) { return x >= 1e-300 && x <= 1e300 ? log_table(x, tab) : log(x); };
+  auto ln = [&](double x) { return is_normal_positive(x) ? log_table(x, tab) : log(x); };
   pdl_wait();
   if (threadIdx.x == 0) {
     half_sh = __ldcg(a.total) / 2;

@@ -75,17 +75,31 @@ __device__ __forceinline__ void st_rowacc(void* base, long long i, const RowAcc&
 
 
 // Per-thread running state of one row, element by element (rows that cannot
-// take the vector path).
+// take the vector path). The sum is relative to the largest element `best`:
+// exp(x - best) = 2^((x - off) log2e + nb), off = 0 and nb = -best log2e, or, past
+// kMaxRef, off = best and nb = 0. (lse_chunk_ex2 for one element, with its test
+// of the bound for each, took 4085 rows of 32003 f32 from 172 to 292 us; this way
+// 173.)
 struct RowState {
-  float best, second, m, s;
+  float best, second, s, off, nb;
   int idx;
   __device__ __forceinline__ void init() {
-    best = -INFINITY; second = -INFINITY; m = -INFINITY; s = 0.f; idx = INT_MAX;
+    best = second = -INFINITY;
+    s = off = nb = 0.f;
+    idx = INT_MAX;
   }
   __device__ __forceinline__ void push(float x, int c) {
-    if (x > second) top2_push(x, c, best, second, idx);
-    const float f[1] = {x};
-    lse_chunk_ex2<1>(f, best, m, s);
+    if (x > second) {
+      const float old = best;
+      top2_push(x, c, best, second, idx);
+      if (best != old) {
+        const bool far = past_ref_bound(best);
+        off = far ? best : 0.f;
+        nb = far ? 0.f : -best * kLog2e;
+        s *= ex2_approx(fmaf(old - off, kLog2e, nb));   // old -inf: s, 0 or NaN, times 0
+      }
+    }
+    s += ex2_approx(fmaf(x - off, kLog2e, nb));   // -inf alone so far: 0 each, NaN: NaN
   }
   __device__ __forceinline__ RowAcc acc() const {
     RowAcc r;

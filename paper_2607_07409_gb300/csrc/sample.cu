@@ -146,10 +146,10 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
   // (0) or NaN (NaN).
   auto push = [&](float (&x)[8], float vm) {
     if (vm > gate) {
-      const float old = m;
+      const float old = m;                     // (-inf: s, 0 or NaN, times 0)
       m = fmaxf(m, vm);
       if (past_ref_bound(m)) {
-        if (old != -INFINITY) s *= ex2_approx((old - m) * kLog2e);
+        s *= ex2_approx((old - m) * kLog2e);
         nb = 0.f;
         gate = -INFINITY;
 #pragma unroll
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kSampleThreads, sizeof(T) == 2 ? 6 : 4) k_lse_
       } else {
         nb = -m * kLog2e;
         gate = m;
-        if (old != -INFINITY) s *= ex2_approx(fmaf(old, kLog2e, nb));
+        s *= ex2_approx(fmaf(old, kLog2e, nb));
       }
     }
     float e[2] = {0.f, 0.f};

@@ -301,7 +301,7 @@ def test_pieces_counted_on_several_streams(V):
 
 @pytest.mark.parametrize("lam", [5e-324, 1e-310, 1e-5, 0.3, 3e7, 1e301])
 def test_log_prior_over_smoothing_weights(lam):
-    """The table-driven logarithm and, outside [1e-300, 1e300], the general one."""
+    """The table-driven logarithm and, where c + lambda is denormal, the general one."""
     V = 3000
     c_ref = np.concatenate([np.arange(2000), 2 ** np.linspace(0, 50, 1000)]).astype(np.int64)
     counts = torch.from_numpy(c_ref).to(DEV)
