@@ -119,20 +119,25 @@ constexpr float kLn2 = 0.693147180559945309f;
 // lowest value, where it overflows. Past the bound, where a row's largest
 // element so far is a mask, the difference is taken first, in place (a loop of
 // its own beside the hot one took 64 requests' block from 450 to 453 us; this
-// way 450, one MLP request 867 -> 873, temperature 1 572 -> 576).
+// way 450).
 constexpr float kMaxRef = 4096.f;
-__device__ __forceinline__ bool past_ref_bound(float ref) { return !(fabsf(ref) <= kMaxRef); }
+__device__ __forceinline__ bool past_ref_bound(float ref, float max_ref = kMaxRef) {
+  return !(fabsf(ref) <= max_ref);
+}
 
 // lse_chunk with the exponent pre-scaled to base 2: one FFMA + one ex2 per
 // element (exp(x - best) = 2^(x*log2e - best*log2e)). The running sum is
-// rescaled only when the maximum moved (rare after the first chunks).
+// rescaled only when the maximum moved (rare after the first chunks). max_ref:
+// infinity for a lane whose result is not used (its values may be anything, and
+// would take the warp through the far branch: one MLP request 867 -> 873 us).
 template <int K>
-__device__ __forceinline__ void lse_chunk_ex2(const float (&x)[K], float best, float& m, float& s) {
+__device__ __forceinline__ void lse_chunk_ex2(const float (&x)[K], float best, float& m, float& s,
+                                              float max_ref = kMaxRef) {
   float y[K];
 #pragma unroll
   for (int i = 0; i < K; ++i) y[i] = x[i];
   float nb = -best * kLog2e;
-  if (past_ref_bound(best)) {
+  if (past_ref_bound(best, max_ref)) {
     nb = 0.f;
     if (best != -INFINITY) {                   // else all -inf (0 each) or NaN (NaN)
       s *= ex2_approx((m - best) * kLog2e);    // m == -inf -> 0 (s was 0)

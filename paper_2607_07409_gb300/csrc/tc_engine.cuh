@@ -364,7 +364,7 @@ template <bool KEYS = false>
 __device__ __forceinline__ void combine_chunk(const float (&acc)[32], const uint8_t* lrow, int half, int swz,
                                               bool long_f32, const float* ptile, int cbase, int V, float alpha,
                                               float nbeta, float& best, float& second, int& idx, float& m,
-                                              float& ssum, const float (&g)[32]) {
+                                              float& ssum, const float (&g)[32], float max_ref) {
   float f[32];
   if (!long_f32) {
 #pragma unroll
@@ -417,7 +417,7 @@ __device__ __forceinline__ void combine_chunk(const float (&acc)[32], const uint
 #pragma unroll
     for (int i = 0; i < 32; ++i) top2_push(f[i], cbase + i, best, second, idx);
   }
-  lse_chunk_ex2<32>(f, best, m, ssum);
+  lse_chunk_ex2<32>(f, best, m, ssum, max_ref);
 }
 
 struct EpiState {
@@ -514,6 +514,7 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
   float best = -INFINITY, second = -INFINITY, m = -INFINITY, ssum = 0.f;
   int idx = 0x7FFFFFFF;
   const float alpha = a.alpha, nbeta = -a.beta;
+  const float max_ref = b < a.B ? kMaxRef : INFINITY;   // lanes past B hold whatever their rows held
   const int br = comb ? min(b, a.l_box_rows - 1) : 0;   // logits-box rows past B are never used
   const int swz = br & 7;
   const uint32_t box_bytes = (uint32_t)a.l_box_rows * 128u;
@@ -545,11 +546,11 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
         if (!a.long_f32) {
           // bf16 boxes of 64 columns: chunk cc is half (cc & 1) of box (cc >> 1)
           combine_chunk(acc, lbuf + (cc >> 1) * box_bytes + br * 128, cc & 1, swz, false, ptile + cc * 32,
-                        it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, acc);
+                        it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, acc, max_ref);
         } else {
           // f32 boxes of 32 columns: chunk cc is box cc
           combine_chunk(acc, lbuf + cc * box_bytes + br * 128, 0, swz, true, ptile + cc * 32,
-                        it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, acc);
+                        it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, acc, max_ref);
         }
       };
       if constexpr (SAMPLE) {
@@ -561,10 +562,10 @@ __device__ __forceinline__ bool epi_run(const Ctx& c, const Phase& p, EpiState& 
           tmem_ld_wait();
           if (!a.long_f32)
             combine_chunk<true>(acc, lbuf + (cc >> 1) * box_bytes + br * 128, cc & 1, swz, false, ptile + cc * 32,
-                                it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, g);
+                                it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, g, max_ref);
           else
             combine_chunk<true>(acc, lbuf + cc * box_bytes + br * 128, 0, swz, true, ptile + cc * 32,
-                                it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, g);
+                                it.o0 + cc * 32, a.V, alpha, nbeta, best, second, idx, m, ssum, g, max_ref);
         }
       } else {
         // one call site per type: the unrolled chunk is large, and more
